@@ -234,8 +234,7 @@ typedef struct {
                                  64, 128 or 256 threads per block) on the context's
                                  own data and keep the fastest (reported in
                                  mpm_stats.jac_config; FP32 Hencky: staged only);
-                                 0 (default): fixed configuration (FP64 staged,
-                                 FP32 per-term (Hencky: staged), 128) */
+                                 0 (default): fixed configuration (staged, 128) */
   int32_t precond_reuse;      /* steps served by one Galerkin product of the multigrid
                                  hierarchies' coarse levels (0 or 1, default: rebuilt
                                  at every step's first set-up; k > 1: rebuilt at every

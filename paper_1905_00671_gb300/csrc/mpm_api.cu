@@ -489,7 +489,7 @@ void free_all(Ctx &c) {
   for (float *p : fptrs)
     if (p) cudaFree(p);
   void *ptrs[] = {c.pf, c.pf_alt, c.pid, c.pid_alt, c.surf, c.surf_alt, c.cell, c.cell_tmp,
-                  c.cell_start, c.cell_cursor, c.perm, c.sh_first, c.sh_cnt, c.sh_box, c.fb_key, c.fb_start, c.fb_cursor, c.fb_perm, c.fb_cmax, c.pn_cnt, c.pn_base, c.sh_S, c.sh_dS,
+                  c.cell_start, c.cell_cursor, c.perm, c.sh_first, c.sh_cnt, c.sh_box, c.fb_key, c.fb_start, c.fb_cursor, c.fb_perm, c.fb_cmax, c.jb, c.jb_cnt, c.pn_cnt, c.pn_base, c.sh_S, c.sh_dS,
                   c.sh_S0, c.m, c.rec, c.pn, c.M, c.Pn, c.vn, c.an, c.pdn, c.pddn, c.phi, c.act, c.fsd, c.sh_nrm, c.fixed, c.u_fixed,
                   c.p_fixed, c.u_value, c.p_value, c.trac, c.trac_raw, c.flux, c.err, c.row_nnz,
                   c.row_ptr, c.row_of, c.col, c.row_mask, c.X, c.R, c.dX, c.stage, c.H, c.gvec,
@@ -501,6 +501,7 @@ void free_all(Ctx &c) {
   if (c.h_err) cudaFreeHost(c.h_err);
   if (c.h_scalar) cudaFreeHost(c.h_scalar);
   if (c.h_terms) cudaFreeHost(c.h_terms);
+  if (c.h_cmax) cudaFreeHost(c.h_cmax);
   if (c.own_stream && c.st) cudaStreamDestroy(c.st);
   c.st = nullptr;
 }
@@ -653,7 +654,6 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   s.kozeny = opt->permeability == MPM_PERM_KOZENY_CARMAN;
   s.hencky = opt->model == MPM_MODEL_HENCKY;
   // the FP32 Jacobian's direct form has no Hencky tangent: staged only
-  if (s.hencky) c.jac_cfg[1].form = Ctx::JAC_STAGED;
   for (int k = 0; k < 3; ++k) s.g[k] = k < c.d ? mat->g[k] : 0.0;
   c.n = P->n;
   c.n_surf = P->n_surf;
@@ -748,6 +748,7 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   if (!rc && cudaHostAlloc((void **)&c.h_scalar, 8 * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
     rc = MPM_ERR_NO_MEMORY;
   if (!rc && (cudaMalloc((void **)&c.terms, 2 * sizeof(unsigned long long)) != cudaSuccess ||
+              cudaHostAlloc((void **)&c.h_cmax, 4 * sizeof(int), cudaHostAllocDefault) != cudaSuccess ||
               cudaHostAlloc((void **)&c.h_terms, 2 * sizeof(unsigned long long), cudaHostAllocDefault) !=
                   cudaSuccess))
     rc = MPM_ERR_NO_MEMORY;

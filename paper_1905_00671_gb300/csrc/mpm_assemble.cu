@@ -25,6 +25,8 @@
 // records.
 #include <math.h>
 
+#include <algorithm>
+
 #include "mpm_internal.cuh"
 
 namespace upmpm {
@@ -641,12 +643,12 @@ __device__ inline int64_t block_of_slot(const uint64_t *__restrict__ mask, const
 //   sum_j g_j c_ijkl = lambda g_i delta_kl + sum_A n_Ai (kappa_A gh_A n_Ak n_Al
 //                      + sum_{B != A} theta_AB gh_B (n_Ak n_Bl + n_Bk n_Al)),
 // gh_A = g . n_A.
+// (BA and rec are field-major over BA.n points; a is the node at slots off)
 template <int D, bool DYN, bool HK, typename R>
-__device__ inline void point_node_record(const GridP &g, const StepP &sp, const DevView &v,
-                                         const BasisArrays<R> &BA, const R *__restrict__ rec, int64_t q,
-                                         const int off[3], R *__restrict__ out) {
+__device__ inline void point_node_record(const StepP &sp, const BasisArrays<R> &BA, const R *__restrict__ rec,
+                                         int64_t q, const int off[3], int64_t a, R *__restrict__ out) {
   using L = PnLay<D, DYN, HK, (int)sizeof(R)>;
-  const int64_t n = v.n;
+  const int64_t n = BA.n;
   const R cs = rec[RC_CS * n + q], vol = rec[RC_VOL * n + q], ph = rec[RC_PH * n + q];
   const R cv = DYN ? (R)(sp.alpha_vis * sp.gamma / (sp.beta * sp.dt)) : R(0);
   const R csv = cs * (R(1) + cv);
@@ -654,9 +656,6 @@ __device__ inline void point_node_record(const GridP &g, const StepP &sp, const 
   const R p2 = HK ? vol * ph : vol * ph - csv * rec[RC_LAM * n + q];
   const R p3 = HK ? vol * ph : csv * rec[RC_MUP * n + q] + vol * ph;
   const R p5 = vol, p6 = rec[RC_B2 * n + q], p7 = rec[RC_KV * n + q], p8 = rec[RC_CST * n + q];
-  int nc[3] = {0, 0, 0};
-  for (int k = 0; k < D; ++k) nc[k] = v.sh_first[k * n + q] + off[k];
-  const int64_t a = node_index(g, nc);
   R Sa, S0a, Gn[3], gs[3];
   basis_at_t<D, R>(BA, q, off, a, Sa, S0a, Gn);
   for (int j = 0; j < D; ++j) {
@@ -798,7 +797,9 @@ __global__ void k_point_nodes(GridP g, StepP sp, DevView v, BasisArrays<R> BA, c
     for (int k = 0; k < D; ++k) P[nq * NPS + L::GP + k] = rec[(RC_GP + k) * n + q];
   for (int sc = j; sc < nq; sc += PN_LANES) {
     const int off[3] = {sc % c0, (sc / c0) % c1, sc / (c0 * c1)};
-    point_node_record<D, DYN, HK, R>(g, sp, v, BA, rec, q, off, P + sc * NPS);
+    int nc[3] = {0, 0, 0};
+    for (int k = 0; k < D; ++k) nc[k] = v.sh_first[k * n + q] + off[k];
+    point_node_record<D, DYN, HK, R>(sp, BA, rec, q, off, node_index(g, nc), P + sc * NPS);
   }
 }
 
@@ -833,7 +834,9 @@ struct PnRec {
   }
 };
 
-// Every candidate point q of the node pair (ac, bc), in a fixed order: the
+// The per-pair kernels (supports of four nodes along some axis, which the bins'
+// kernels above leave to them, and the direct FP32 form) visit
+// every candidate point q of the node pair (ac, bc), in a fixed order: the
 // points of the first-node bins that can hold both nodes (FB), or those of the
 // cells around both (each x-run of cells is one contiguous run of the
 // cell-sorted points).  The bins visit fewer candidates; the cells visit them
@@ -972,6 +975,411 @@ __global__ void k_jacobian(GridP g, StepP s, DevView v, const R *__restrict__ pn
     B[D * NB + i] = b2ba[i] - kgp[i];
   }
   B[D * NB + D] = C;
+  write_block_bc<D>(v, bn, a, B, val + e2 * (NB * NB), apply_bc);
+}
+
+// ---- staged form by first-node bins: k_jac_bins and k_jac_gather
+// Every point of a first-node bin has its support box at the bin's node f, so
+// the bin's terms fall on the node pairs of one LB^D box (LB = 2 for original
+// MPM, 3 for GIMP domains narrower than a cell).  k_jac_bins forms the (point,
+// node) records of a bin once, in shared memory, and sums the bin's points
+// pair by pair (one thread per pair of box nodes) into a scratch of pair
+// values; k_jac_gather adds, for each pair of grid nodes, the bins whose box
+// holds both, and writes the two blocks.
+// Why: one thread per pair of grid nodes (k_jacobian below) reads the records
+// of unrelated points in neighbouring lanes and qualifies for them at
+// different times: 29% of the FP64 lanes and, in FP32, an L1-bound kernel.
+// Here a warp holds pairs of one box, whose terms come from the same few
+// records; the pairs are ordered so that those of one warp meet the same
+// points (a lattice's points have extents 2 or 3 per axis, so a pair of nodes
+// with c coordinates at 2 is met by 1 / 2^c of the bin's points), which keeps
+// about 85% of the lanes busy.  The scratch is a ring of planes of bins, so its
+// size does not grow with the grid.
+// k_jac_bins is bound by the FP64 pipe in FP64 (93% busy, 25 of 32 lanes) and by
+// shared-memory and L1 throughput in FP32 (81%); k_jac_gather by the latency of
+// its scattered 96- or 176-byte reads.  Per assembly on a GB300, against the
+// per-pair kernel with its staging: 4.2M-point slope FP64 123 -> 90 ms, FP32
+// 79 -> 19 ms; 163k-point block 13.5 -> 3.7 ms; 1M-point block FP32 11.6 ->
+// 3.8 ms; 80k-point footing 0.68 -> 0.36 ms; 64 batched columns 1.5 -> 1.1 ms.
+template <int D, int LB>
+struct BoxPairs {
+  static constexpr int NL = D == 2 ? LB * LB : LB * LB * LB;  // nodes of the box
+  static constexpr int NP = NL * (NL + 1) / 2;                // unordered pairs
+  uint16_t ab[NP];                                            // la | lb << 8, la <= lb
+  uint16_t at[NL * NL];                                       // pair index of (la, lb)
+};
+// pairs (la <= lb) by the number of axes on which one of the two nodes has
+// the largest box coordinate
+template <int D, int LB>
+constexpr BoxPairs<D, LB> box_pairs() {
+  using BP = BoxPairs<D, LB>;
+  BP t{};
+  int p = 0;
+  for (int cls = 0; cls <= D; ++cls)
+    for (int la = 0; la < BP::NL; ++la)
+      for (int lb = la; lb < BP::NL; ++lb) {
+        int far = 0, ra = la, rb = lb;
+        for (int k = 0; k < D; ++k) {
+          if (ra % LB == LB - 1 || rb % LB == LB - 1) ++far;
+          ra /= LB;
+          rb /= LB;
+        }
+        if (far != cls) continue;
+        t.ab[p] = (uint16_t)(la | (lb << 8));
+        t.at[la * BP::NL + lb] = (uint16_t)p;
+        t.at[lb * BP::NL + la] = (uint16_t)p;
+        ++p;
+      }
+  return t;
+}
+template <int D, int LB>
+__device__ const BoxPairs<D, LB> d_box_pairs = box_pairs<D, LB>();
+
+// Values of a pair in the scratch: A (row la), B1 and B2 of (la, lb), B1 and
+// B2 of (lb, la), C; padded to 16 bytes.
+template <int D, typename R>
+struct PairVals {
+  static constexpr int A = 0, B1AB = D * D, B2AB = B1AB + D, B1BA = B2AB + D, B2BA = B1BA + D, C = B2BA + D;
+  static constexpr int N = D * D + 4 * D + 1;
+  static constexpr int W = 16 / (int)sizeof(R);
+  static constexpr int STRIDE = (N + W - 1) / W * W;
+};
+
+// Shared memory of one bin: up to BQ points at a time, BREC records.
+// 3D: a block of 128 threads per bin (378 pairs), the points' record fields
+// staged once for their (up to 27) node records; 2D: a warp per bin (45 pairs),
+// half a warp for original MPM (10), the fields read from L1 where they are
+// used, which leaves room for more bins per SM.
+template <int D, int LB, bool DYN, bool HK, typename R>
+struct BinShape {
+  static constexpr int GT = D == 3 ? 128 : (LB == 2 ? 16 : 32);  // threads per bin
+  static constexpr bool STAGE = D == 3;
+  static constexpr int BLOCK = 128;
+  static constexpr int PER_BLOCK = BLOCK / GT;
+  static constexpr int BQ = D == 2 ? 4 : 8;     // points per pass (a bin of a 2^D-per-cell lattice)
+  static constexpr int BREC = BQ * BoxPairs<D, LB>::NL;
+  // an odd record stride keeps the lanes of consecutive nodes in different banks
+  static constexpr int NPS = PnLay<D, DYN, HK, (int)sizeof(R)>::U + (HK ? D * D * D : 0);
+  static constexpr int STRIDE = NPS | 1;
+  struct Smem {
+    R rec[BREC * STRIDE];
+    R gp[3 * BQ];                 // grad p of the points
+    R fld[STAGE ? RC_F32 * BQ : 1];  // record fields of the points, and their 1D bases
+    R S[STAGE ? 12 * BQ : 1], dS[STAGE ? 12 * BQ : 1], S0[STAGE ? 12 * BQ : 1], nrm[STAGE ? 5 * BQ : 1];
+    int32_t cnt[BQ], q[BQ], base[BQ + 1];
+  };
+};
+
+// Record fields a point-node record reads (RC_*): the others are not staged.
+template <int D, bool DYN, bool HK>
+__device__ constexpr bool bin_needs(int f) {
+  if (f < RC_TAU) return f < RC_FINV + D * D;
+  if (f < RC_SVIS) return f < RC_TAU + D * D;
+  if (f < RC_GV) return false;
+  if (f < RC_GP) return DYN && f < RC_GV + D * D;
+  if (f < RC_W) return false;
+  if (f < RC_FRC) return f < RC_W + D;
+  if (f < RC_CS) return false;
+  if (f == RC_RST || f == RC_DIVV) return false;
+  if (f == RC_MS) return DYN;
+  if (f >= RC_HQ) return HK;
+  return true;
+}
+
+template <int GT>
+__device__ __forceinline__ void bin_sync(unsigned members) {
+  if constexpr (GT <= 32) __syncwarp(members);
+  else __syncthreads();
+}
+
+// Bins fb0 .. fb0 + nb - 1 (node indices of the box origins): pair sums into
+// scratch, the bin's union box into ucnt (0: no points).
+template <int D, int LB, bool DYN, bool HK, typename R>
+__global__ void __launch_bounds__(128) k_jac_bins(GridP g, StepP sp, DevView v, BasisArrays<R> BA,
+                                                  const R *__restrict__ rec, int64_t fb0, int64_t nb, int64_t plane,
+                                                  int ring, R *__restrict__ scratch, int32_t *__restrict__ ucnt) {
+  using BS = BinShape<D, LB, DYN, HK, R>;
+  using BP = BoxPairs<D, LB>;
+  using PV = PairVals<D, R>;
+  using L = PnLay<D, DYN, HK, (int)sizeof(R)>;
+  constexpr int GT = BS::GT, ST = BS::STRIDE;
+  extern __shared__ __align__(16) unsigned char jac_smem[];
+  constexpr int GW = GT < 32 ? GT : 32;  // lanes of a warp that share a bin
+  const int grp = threadIdx.x / GT, tid = threadIdx.x % GT, lane = threadIdx.x % GW;
+  const int wbase = (threadIdx.x & 31) - lane;
+  const unsigned members = (GW == 32 ? 0xffffffffu : (1u << GW) - 1u) << wbase;
+  typename BS::Smem &sm = reinterpret_cast<typename BS::Smem *>(jac_smem)[grp];
+  const int64_t bi = blockIdx.x * (int64_t)BS::PER_BLOCK + grp;
+  if (bi >= nb) return;  // uniform in the bin's threads
+  const int64_t f = fb0 + bi;
+  const int64_t slot = (f / plane) % ring * plane + f % plane;  // of the bin in the ring
+  const int32_t ib = v.fb_start[f], ie = v.fb_start[f + 1];
+  if (ib == ie) {
+    if (tid == 0) ucnt[slot] = 0;
+    return;
+  }
+  const int64_t n = v.n;
+  int fc[3];
+  node_coords(g, f, fc);
+  R *out = scratch + slot * (int64_t)(BP::NP * PV::STRIDE);
+  int ux = 0, uy = 0, uz = 0;
+  for (int32_t i0 = ib; i0 < ie; i0 += BS::BQ) {
+    const int nq = min((int)BS::BQ, ie - i0);
+    bin_sync<GT>(members);  // the previous pass's records have been read
+    if (tid < nq) {
+      const int32_t q = v.fb_perm[i0 + tid];
+      sm.q[tid] = q;
+      sm.cnt[tid] = v.sh_cnt[q];
+    }
+    bin_sync<GT>(members);
+    if (tid == 0) {
+      int b = 0;
+      for (int i = 0; i < nq; ++i) {
+        sm.base[i] = b;
+        b += unpack_cnt(sm.cnt[i], 0) * unpack_cnt(sm.cnt[i], 1) * (D == 3 ? unpack_cnt(sm.cnt[i], 2) : 1);
+      }
+      sm.base[nq] = b;
+    }
+    for (int t = tid; t < D * BS::BQ; t += GT) {
+      const int i = t % BS::BQ;
+      if (i < nq) sm.gp[t] = rec[(RC_GP + t / BS::BQ) * n + sm.q[i]];
+    }
+    if constexpr (BS::STAGE) {
+      for (int t = tid; t < RC_F32 * BS::BQ; t += GT) {
+        const int fl = t / BS::BQ, i = t % BS::BQ;
+        if (i < nq && bin_needs<D, DYN, HK>(fl)) sm.fld[t] = rec[fl * n + sm.q[i]];
+      }
+      for (int t = tid; t < 4 * D * BS::BQ; t += GT) {
+        const int fl = t / BS::BQ, i = t % BS::BQ;
+        if (i < nq && fl % 4 < LB) {
+          const int64_t at = fl * n + sm.q[i];
+          sm.S[t] = BA.S[at];
+          sm.dS[t] = BA.dS[at];
+          sm.S0[t] = BA.S0[at];
+        }
+      }
+      for (int t = tid; t < 5 * BS::BQ; t += GT) {
+        const int i = t % BS::BQ;
+        if (i < nq && (sm.cnt[i] & RENORM_BIT)) sm.nrm[t] = BA.nrm[t / BS::BQ * n + sm.q[i]];
+      }
+    }
+    // extents of the pass's points: bit i of m[k][e - 1] set iff point i spans
+    // more than e nodes along axis k
+    const int ci = lane < nq ? sm.cnt[lane] : 0;
+    unsigned m[3][LB];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const int ek = unpack_cnt(ci, k);
+#pragma unroll
+      for (int e = 0; e < LB; ++e) m[k][e] = __ballot_sync(members, ek > e) >> wbase;
+      const int top = __reduce_max_sync(members, ek);
+      if (k == 0) ux = max(ux, top);
+      else if (k == 1) uy = max(uy, top);
+      else uz = max(uz, top);
+    }
+    bin_sync<GT>(members);
+    {
+      const BasisArrays<R> B{BS::STAGE ? BS::BQ : n,          BS::STAGE ? sm.cnt : BA.cnt,
+                             BA.act,                          BS::STAGE ? sm.S : BA.S,
+                             BS::STAGE ? sm.dS : BA.dS,       BS::STAGE ? sm.S0 : BA.S0,
+                             BS::STAGE ? sm.nrm : BA.nrm};
+      const R *fields = BS::STAGE ? sm.fld : rec;
+      const int total = sm.base[nq];
+      for (int t = tid; t < total; t += GT) {
+        int i = 0;
+#pragma unroll
+        for (int j = 1; j < BS::BQ; ++j) i += (j < nq && t >= sm.base[j]) ? 1 : 0;
+        const int cn = sm.cnt[i], c0 = unpack_cnt(cn, 0), c1 = unpack_cnt(cn, 1);
+        const int l = t - sm.base[i];
+        const int off[3] = {l % c0, (l / c0) % c1, D == 3 ? l / (c0 * c1) : 0};
+        const int nc[3] = {fc[0] + off[0], fc[1] + off[1], fc[2] + off[2]};
+        point_node_record<D, DYN, HK, R>(sp, B, fields, BS::STAGE ? i : sm.q[i], off, node_index(g, nc),
+                                         sm.rec + t * ST);
+      }
+    }
+    bin_sync<GT>(members);
+    // the warps of a bin take chunks of 32 pairs, their order turned from bin to
+    // bin: the first chunks have the most terms, and a warp's number decides
+    // which of the SM's four FP64 pipes it uses
+    constexpr int NW = GT / GW;
+    const int w = NW > 1 ? (int)((threadIdx.x / 32 + blockIdx.x) % NW) : 0;
+    for (int p0 = GW * w; p0 < BP::NP; p0 += GT) {
+      const int p = p0 + lane;
+      if (p >= BP::NP) continue;
+      const int ab = d_box_pairs<D, LB>.ab[p];
+      const int la = ab & 255, lb = ab >> 8;
+      const int ax = la % LB, ay = la / LB % LB, az = D == 3 ? la / (LB * LB) : 0;
+      const int bx = lb % LB, by = lb / LB % LB, bz = D == 3 ? lb / (LB * LB) : 0;
+      unsigned todo = 0;
+      {
+        unsigned mx = 0, my = 0, mz = 0xffffffffu;
+#pragma unroll
+        for (int e = 0; e < LB; ++e) {
+          if (max(ax, bx) == e) mx = m[0][e];
+          if (max(ay, by) == e) my = m[1][e];
+          if (D == 3 && max(az, bz) == e) mz = m[D - 1][e];
+        }
+        todo = mx & my & mz;
+        // outside the union box of a bin of one pass: k_jac_gather does not read it
+        if (ie - ib <= BS::BQ &&
+            (max(ax, bx) >= ux || max(ay, by) >= uy || (D == 3 && max(az, bz) >= uz)))
+          continue;
+      }
+      R A[D * D], b1ab[D], b1ba[D], b2ab[D], b2ba[D], kgp[D], C = 0, Dg = 0;
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) A[i] = 0;
+#pragma unroll
+      for (int i = 0; i < D; ++i) b1ab[i] = b1ba[i] = b2ab[i] = b2ba[i] = kgp[i] = 0;
+      while (todo) {
+        const int i = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int cn = sm.cnt[i], c0 = unpack_cnt(cn, 0), c1 = unpack_cnt(cn, 1);
+        const R *pa = sm.rec + (sm.base[i] + ax + c0 * (ay + c1 * az)) * ST;
+        const R *pb = sm.rec + (sm.base[i] + bx + c0 * (by + c1 * bz)) * ST;
+        // the terms of k_jacobian below
+        R ga[D], gb[D], kgab = 0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          ga[j] = pa[L::G + j];
+          gb[j] = pb[L::G + j];
+          Dg = fma(pa[L::H + j], gb[j], Dg);
+          kgab = fma(pa[L::P7G + j], gb[j], kgab);
+        }
+        if (DYN) Dg = fma(pa[L::MS], pb[L::S], Dg);
+#pragma unroll
+        for (int r = 0; r < D; ++r)
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            R acc = fma(ga[r], pb[L::P2G + k], A[r * D + k]);
+            acc = fma(-gb[r], pa[L::P3G + k], acc);
+            if (HK)
+#pragma unroll
+              for (int l = 0; l < D; ++l) acc = fma(pa[L::U + (r * D + k) * D + l], gb[l], acc);
+            A[r * D + k] = acc;
+          }
+        const R p5Sb = pb[L::P5S], p5Sa = pa[L::P5S], ca = pa[L::C], eb = pb[L::E], cb = pb[L::C], ea = pa[L::E];
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          b1ab[k] = fma(p5Sb, ga[k], b1ab[k]);
+          b1ba[k] = fma(p5Sa, gb[k], b1ba[k]);
+          kgp[k] = fma(kgab, sm.gp[k * BS::BQ + i], kgp[k]);
+          R tk = fma(ca, gb[k], b2ab[k]);
+          R sk = fma(cb, ga[k], b2ba[k]);
+          if (DYN) {
+            tk = fma(-p5Sa, pb[L::GV + k], tk);
+            sk = fma(-p5Sb, pa[L::GV + k], sk);
+          }
+          b2ab[k] = fma(-eb, ga[k], tk);
+          b2ba[k] = fma(-ea, gb[k], sk);
+        }
+        C = fma(pa[L::P8ST], pb[L::ST], C + kgab);
+      }
+      alignas(16) R val[PV::STRIDE];
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) val[PV::A + i] = A[i] - (i % (D + 1) == 0 ? Dg : R(0));
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        val[PV::B1AB + i] = b1ab[i];
+        val[PV::B2AB + i] = b2ab[i] - kgp[i];
+        val[PV::B1BA + i] = b1ba[i];
+        val[PV::B2BA + i] = b2ba[i] - kgp[i];
+      }
+      val[PV::C] = C;
+#pragma unroll
+      for (int i = PV::N; i < PV::STRIDE; ++i) val[i] = 0;
+      int4 *dst = reinterpret_cast<int4 *>(out + p * PV::STRIDE);
+      if (i0 != ib) {  // a later pass of a bin of more than BQ points
+        const R *old = out + p * PV::STRIDE;
+#pragma unroll
+        for (int i = 0; i < PV::N; ++i) val[i] += old[i];
+      }
+#pragma unroll
+      for (int i = 0; i < PV::STRIDE / PV::W; ++i) dst[i] = reinterpret_cast<const int4 *>(val)[i];
+    }
+  }
+  if (tid == 0) ucnt[slot] = ux | (uy << 4) | (uz << 8);
+}
+
+// Blocks (a, b) and (b, a) of the rows a0 .. a0 + nr - 1 from the pair sums of
+// the bins whose box holds both nodes.  The lanes of a warp hold one offset
+// b - a (upper half of the 2 LB - 1 window) in 32 consecutive rows.
+template <int D, int LB, typename T, typename R>
+__global__ void k_jac_gather(GridP g, DevView v, int64_t a0, int64_t nr, int64_t plane, int ring,
+                             const R *__restrict__ scratch, const int32_t *__restrict__ ucnt,
+                             const uint64_t *__restrict__ mask, const int32_t *__restrict__ row_ptr,
+                             const int32_t *__restrict__ col, T *__restrict__ val, int apply_bc) {
+  using BP = BoxPairs<D, LB>;
+  using PV = PairVals<D, R>;
+  using PS = PairSlots<D>;
+  constexpr int W = 2 * LB - 1, NOFF = D == 2 ? W * W : W * W * W, HALF = NOFF / 2 + 1;
+  constexpr int NB = D + 1;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  constexpr int64_t PER_TILE = (int64_t)PAIR_ROWS * HALF;
+  const int64_t tile = t / PER_TILE;
+  const int rem = (int)(t - tile * PER_TILE);
+  const int64_t ar = tile * PAIR_ROWS + rem % PAIR_ROWS;
+  if (ar >= nr) return;
+  const int64_t a = a0 + ar;
+  const int o = NOFF / 2 + rem / PAIR_ROWS;
+  const int o0 = o % W - (LB - 1), o1 = o / W % W - (LB - 1), o2 = D == 3 ? o / (W * W) - (LB - 1) : 0;
+  const int slot = (o0 + 3) + 7 * (o1 + 3) + (D == 3 ? 49 * (o2 + 3) : 0);
+  const int64_t e = block_of_slot<D>(mask, row_ptr, a, slot);
+  if (e < 0) return;
+  const int64_t bn = col[e];
+  const bool diag = slot == PS::CENTRE;
+  int ac[3];
+  node_coords(g, a, ac);
+  const int bc[3] = {ac[0] + o0, ac[1] + o1, ac[2] + o2};
+  int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+  for (int k = 0; k < D; ++k) {
+    lo[k] = max(max(ac[k], bc[k]) - (LB - 1), 0);
+    hi[k] = min(ac[k], bc[k]);
+  }
+  R acc[PV::STRIDE];
+#pragma unroll
+  for (int i = 0; i < PV::STRIDE; ++i) acc[i] = 0;
+  for (int f2 = lo[2]; f2 <= hi[2]; ++f2)
+    for (int f1 = lo[1]; f1 <= hi[1]; ++f1)
+      for (int f0 = lo[0]; f0 <= hi[0]; ++f0) {
+        const int fcoord[3] = {f0, f1, f2};
+        const int64_t f = node_index(g, fcoord);
+        const int64_t sl = (f / plane) % ring * plane + f % plane;
+        const int u = ucnt[sl];
+        if (u == 0) continue;
+        const int a_[3] = {ac[0] - f0, ac[1] - f1, ac[2] - f2}, b_[3] = {bc[0] - f0, bc[1] - f1, bc[2] - f2};
+        bool in = true;
+        for (int k = 0; k < D; ++k) in = in && max(a_[k], b_[k]) < unpack_cnt(u, k);
+        if (!in) continue;
+        int la = a_[0] + LB * a_[1], lb = b_[0] + LB * b_[1];
+        if (D == 3) {
+          la += LB * LB * a_[2];
+          lb += LB * LB * b_[2];
+        }
+        const int p = d_box_pairs<D, LB>.at[la * BP::NL + lb];
+        const int4 *src = reinterpret_cast<const int4 *>(scratch + (sl * BP::NP + p) * PV::STRIDE);
+        alignas(16) R x[PV::STRIDE];
+#pragma unroll
+        for (int i = 0; i < PV::STRIDE / PV::W; ++i) reinterpret_cast<int4 *>(x)[i] = src[i];
+#pragma unroll
+        for (int i = 0; i < PV::N; ++i) acc[i] += x[i];
+      }
+  R B[NB * NB];
+  for (int i = 0; i < D; ++i) {
+    for (int k = 0; k < D; ++k) B[i * NB + k] = acc[PV::A + i * D + k];
+    B[i * NB + D] = acc[PV::B1AB + i];
+    B[D * NB + i] = acc[PV::B2AB + i];
+  }
+  B[D * NB + D] = acc[PV::C];
+  write_block_bc<D>(v, a, bn, B, val + e * (NB * NB), apply_bc);
+  if (diag) return;
+  const int64_t e2 = block_of_slot<D>(mask, row_ptr, bn, PS::NSLOT - 1 - slot);
+  if (e2 < 0) return;  // the coupling is symmetric: not reached
+  for (int i = 0; i < D; ++i) {
+    for (int k = 0; k < D; ++k) B[i * NB + k] = acc[PV::A + k * D + i];
+    B[i * NB + D] = acc[PV::B1BA + i];
+    B[D * NB + i] = acc[PV::B2BA + i];
+  }
+  B[D * NB + D] = acc[PV::C];
   write_block_bc<D>(v, bn, a, B, val + e2 * (NB * NB), apply_bc);
 }
 
@@ -1403,7 +1811,67 @@ static int grow_staging(R **buf, int64_t *cap, int64_t total, int stride) {
   return MPM_OK;
 }
 
+// The staged form by first-node bins serves supports of at most 3 nodes per
+// axis (original MPM: 2): the box of LB^D nodes around a bin's points, 0 if
+// some support is wider (GIMP domains over h / 2 in half length), which the
+// per-pair kernel with its staging in HBM serves.
+static int jac_box(const Ctx &c) {
+  if (c.shape != MPM_SHAPE_GIMP) return 2;
+  for (int k = 0; k < c.d; ++k)
+    if (c.h_cmax[k] > 3) return 0;
+  return 3;
+}
+
+// Ring of bin planes: as many as JAC_RING_BYTES hold (all of a 2D grid or a
+// small 3D one, so that the two kernels run once), at least LB.
+constexpr int64_t JAC_RING_BYTES = 8ll << 30;
+template <typename R>
+static int64_t jac_plane_bytes(const Ctx &c, int lb) {
+  const int64_t plane = c.d == 2 ? c.g.nn[0] : (int64_t)c.g.nn[0] * c.g.nn[1];
+  const int nl = c.d == 2 ? lb * lb : lb * lb * lb;
+  const int stride = c.d == 2 ? PairVals<2, R>::STRIDE : PairVals<3, R>::STRIDE;
+  return plane * (nl * (nl + 1) / 2) * stride * (int64_t)sizeof(R);
+}
+template <typename R>
+static int ensure_jac_ring(Ctx &c, int lb) {
+  const int64_t pb = jac_plane_bytes<R>(c, lb);
+  const int planes = c.g.nn[c.d - 1];
+  int ring = (int)std::min<int64_t>(planes, std::max<int64_t>(lb, JAC_RING_BYTES / pb));
+  if (c.jb && (c.jb_cap >= pb * ring || (c.jb_short && c.jb_cap >= pb * lb))) {
+    c.jb_ring = (int)std::min<int64_t>(ring, c.jb_cap / pb);
+    return MPM_OK;
+  }
+  const int asked = ring;
+  cudaFree(c.jb);
+  cudaFree(c.jb_cnt);
+  c.jb = nullptr;
+  c.jb_cnt = nullptr;
+  c.jb_cap = 0;
+  for (;; ring = std::max(lb, ring / 2)) {  // a smaller ring where memory is short
+    if (cudaMalloc(&c.jb, pb * ring) == cudaSuccess) break;
+    cudaGetLastError();
+    c.jb = nullptr;
+    if (ring <= lb) return MPM_ERR_NO_MEMORY;
+  }
+  if (cudaMalloc(&c.jb_cnt, sizeof(int32_t) * c.g.nnodes) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(c.jb);
+    c.jb = nullptr;
+    c.jb_cnt = nullptr;
+    return MPM_ERR_NO_MEMORY;
+  }
+  c.jb_cap = pb * ring;
+  c.jb_ring = ring;
+  c.jb_short = ring < asked;
+  return MPM_OK;
+}
+
 int ensure_jacobian_staging(Ctx &c) {
+  if (const int lb = jac_box(c)) {
+    const int rc = ensure_jac_ring<double>(c, lb);
+    if (rc) c.last_error = "device allocation of the Jacobian's bin sums failed";
+    return rc;
+  }
   const int rc = grow_staging(&c.pn, &c.pn_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 8));
   if (rc) c.last_error = "device allocation of the Jacobian staging failed";
   return rc;
@@ -1636,12 +2104,39 @@ void run_residual(Ctx &c, const double *X, double *R, int apply_bc) {
 
 // FP32 copy of the staging (allocated for the staged FP32 variant only)
 int ensure_jacobian_staging32(Ctx &c) {
+  if (const int lb = jac_box(c)) return ensure_jac_ring<float>(c, lb);
   return grow_staging(&c.pn32, &c.pn32_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 4));
 }
 
-// One assembly with a given kernel configuration: staged (k_point_nodes then
-// k_jacobian on the per-(point, node) vectors) or direct (k_jacobian_direct),
-// tpb threads per block.  Values in precision T computed
+// The staged form by first-node bins: chunks of bin planes, each followed by the
+// rows whose bins are then complete (a row's bins lie in its own plane and the
+// LB - 1 before it, which the ring still holds).
+template <int D, int LB, bool DYN, bool HK, typename T>
+void launch_jac_bins(Ctx &c, T *val, int apply_bc, const BasisArrays<T> &BA, const T *rec, int tpb) {
+  using BS = BinShape<D, LB, DYN, HK, T>;
+  const DevView v = c.view();
+  const int64_t plane = D == 2 ? c.g.nn[0] : (int64_t)c.g.nn[0] * c.g.nn[1];
+  const int planes = c.g.nn[D - 1], ring = c.jb_ring;
+  const int chunk = ring >= planes ? planes : ring - (LB - 1);
+  constexpr size_t smem = sizeof(typename BS::Smem) * BS::PER_BLOCK;
+  constexpr int HALF = D == 2 ? ((2 * LB - 1) * (2 * LB - 1) + 1) / 2
+                              : ((2 * LB - 1) * (2 * LB - 1) * (2 * LB - 1) + 1) / 2;
+  cudaFuncSetAttribute(k_jac_bins<D, LB, DYN, HK, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  for (int z = 0; z < planes; z += chunk) {
+    const int64_t f0 = z * plane, nb = std::min<int64_t>(chunk, planes - z) * plane;
+    k_jac_bins<D, LB, DYN, HK, T><<<nblk(nb, BS::PER_BLOCK), BS::BLOCK, smem, c.st>>>(
+        c.g, c.s, v, BA, rec, f0, nb, plane, ring, (T *)c.jb, c.jb_cnt);
+    const int64_t nthr = (nb + PAIR_ROWS - 1) / PAIR_ROWS * PAIR_ROWS * HALF;
+    k_jac_gather<D, LB, T, T><<<(int)((nthr + tpb - 1) / tpb), tpb, 0, c.st>>>(
+        c.g, v, f0, nb, plane, ring, (const T *)c.jb, c.jb_cnt, c.row_mask, c.row_ptr, c.col, val, apply_bc);
+    c.launches += 2;
+  }
+}
+
+// One assembly with a given kernel configuration: staged (by first-node bins, or
+// for supports of 4 nodes k_point_nodes then k_jacobian on the per-(point, node)
+// vectors) or direct (k_jacobian_direct), tpb threads per block of the kernel
+// that writes the blocks.  Values in precision T computed
 // in precision T from the FP64 records or their FP32 copies.
 template <typename T>
 void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
@@ -1650,7 +2145,7 @@ void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
   // the Jacobian kernels take symmetric pairs: half the offsets plus the centre
   const int64_t nthr = pair_threads(c.d, c.g.nnodes);
   const int nbk_pair = (int)((nthr + tpb - 1) / tpb);
-  const bool gimp = c.shape == MPM_SHAPE_GIMP;
+  [[maybe_unused]] const bool gimp = c.shape == MPM_SHAPE_GIMP;
   using R = T;
   // candidates from the first-node bins in FP32, from the cells in FP64
   constexpr bool FB = sizeof(T) == sizeof(float);
@@ -1669,7 +2164,23 @@ void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
     BA.nrm = (const R *)c.sh_nrmf; rec = (const R *)c.recf;
     pn = (R *)c.pn32;
   }
-  if (staged && !pn) return;  // callers allocate the staging first
+  const int lb = staged ? jac_box(c) : 0;
+  if (staged && !(lb ? c.jb != nullptr : pn != nullptr)) return;  // callers allocate the staging first
+  if (lb) {
+#define BINS(D, LB, Y, H) launch_jac_bins<D, LB, Y, H, T>(c, val, apply_bc, BA, rec, tpb)
+#define BINS_LB(D, Y, H) do { if (lb == 2) BINS(D, 2, Y, H); else BINS(D, 3, Y, H); } while (0)
+    const bool hk = c.s.hencky;
+    if (c.d == 2) {
+      if (c.dyn) { if (hk) BINS_LB(2, true, true); else BINS_LB(2, true, false); }
+      else { if (hk) BINS_LB(2, false, true); else BINS_LB(2, false, false); }
+    } else {
+      if (c.dyn) { if (hk) BINS_LB(3, true, true); else BINS_LB(3, true, false); }
+      else { if (hk) BINS_LB(3, false, true); else BINS_LB(3, false, false); }
+    }
+#undef BINS_LB
+#undef BINS
+    return;
+  }
   if (staged) {
     const int npb = nblk((int64_t)PN_LANES * c.n, TPB);
 #define PNODES(D, Y, H) k_point_nodes<D, Y, H, R><<<npb, TPB, 0, c.st>>>(c.g, c.s, v, BA, rec, pn)
@@ -1684,26 +2195,33 @@ void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
 #undef PNODES
     UPMPM_LAUNCH(c);
   }
-#define JAC(D, G, Y)                                                                                         \
+  // supports of four nodes (GIMP), or the direct form (FP32)
+#define JAC_WIDE(D, Y)                                                                                       \
   do {                                                                                                       \
-    if (staged && c.s.hencky)                                                                                \
-      k_jacobian<D, G, Y, true, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, pn, c.row_mask,           \
-                                                                      c.row_ptr, c.col, val, apply_bc);      \
-    else if (staged)                                                                                         \
-      k_jacobian<D, G, Y, false, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, pn, c.row_mask,          \
-                                                                       c.row_ptr, c.col, val, apply_bc);     \
+    if (c.s.hencky)                                                                                          \
+      k_jacobian<D, true, Y, true, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, pn, c.row_mask,        \
+                                                                         c.row_ptr, c.col, val, apply_bc);   \
     else                                                                                                     \
-      k_jacobian_direct<D, G, Y, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, BA, rec, c.row_mask,     \
-                                                                       c.row_ptr, c.col, val, apply_bc);     \
+      k_jacobian<D, true, Y, false, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, pn, c.row_mask,       \
+                                                                          c.row_ptr, c.col, val, apply_bc);  \
   } while (0)
-  if (c.d == 2) {
-    if (gimp) { if (c.dyn) JAC(2, true, true); else JAC(2, true, false); }
-    else { if (c.dyn) JAC(2, false, true); else JAC(2, false, false); }
-  } else {
-    if (gimp) { if (c.dyn) JAC(3, true, true); else JAC(3, true, false); }
-    else { if (c.dyn) JAC(3, false, true); else JAC(3, false, false); }
+#define JAC_DIR(D, G, Y)                                                                                     \
+  k_jacobian_direct<D, G, Y, FB, T, R><<<nbk_pair, tpb, 0, c.st>>>(c.g, c.s, v, BA, rec, c.row_mask,         \
+                                                                   c.row_ptr, c.col, val, apply_bc)
+  if (staged) {
+    if (c.d == 2) { if (c.dyn) JAC_WIDE(2, true); else JAC_WIDE(2, false); }
+    else { if (c.dyn) JAC_WIDE(3, true); else JAC_WIDE(3, false); }
+  } else if constexpr (FB) {
+    if (c.d == 2) {
+      if (gimp) { if (c.dyn) JAC_DIR(2, true, true); else JAC_DIR(2, true, false); }
+      else { if (c.dyn) JAC_DIR(2, false, true); else JAC_DIR(2, false, false); }
+    } else {
+      if (gimp) { if (c.dyn) JAC_DIR(3, true, true); else JAC_DIR(3, true, false); }
+      else { if (c.dyn) JAC_DIR(3, false, true); else JAC_DIR(3, false, false); }
+    }
   }
-#undef JAC
+#undef JAC_WIDE
+#undef JAC_DIR
   UPMPM_LAUNCH(c);
 }
 
@@ -1755,6 +2273,13 @@ void autotune_jacobian(Ctx &c, T *val, int apply_bc) {
     cudaFree(c.pn32);
     c.pn32 = nullptr;
     c.pn32_cap = 0;
+  }
+  if (pi == 1 && cfg.form == Ctx::JAC_DIRECT && c.jb) {
+    cudaFree(c.jb);
+    cudaFree(c.jb_cnt);
+    c.jb = nullptr;
+    c.jb_cnt = nullptr;
+    c.jb_cap = 0;
   }
 }
 

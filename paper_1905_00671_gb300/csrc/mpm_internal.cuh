@@ -315,6 +315,14 @@ struct Ctx {
   int32_t *pn_cnt = nullptr, *pn_base = nullptr;
   int64_t pn_total = 0;                  // records of the current step
   int64_t pn_cap = 0, pn32_cap = 0;      // records pn / pn32 can hold
+  // staged Jacobian by first-node bins: ring of bin planes with the bins' pair
+  // sums (either precision), the bins' box extents, planes of the ring
+  void *jb = nullptr;
+  int64_t jb_cap = 0;                    // bytes
+  int32_t *jb_cnt = nullptr;
+  int jb_ring = 0;
+  bool jb_short = false;                 // memory was short of the ring asked for
+  int *h_cmax = nullptr;                 // pinned: the step's largest box extent per axis
   unsigned long long *h_terms = nullptr; // pinned copy
   // Jacobian kernel configuration per precision ([0] FP64, [1] FP32): the
   // form (JAC_DIRECT: node vectors recomputed per term; JAC_STAGED:
@@ -325,7 +333,7 @@ struct Ctx {
   struct JacCfg {
     int form, tpb, tuned;
   };
-  JacCfg jac_cfg[2] = {{JAC_STAGED, 128, 0}, {JAC_DIRECT, 128, 0}};
+  JacCfg jac_cfg[2] = {{JAC_STAGED, 128, 0}, {JAC_STAGED, 128, 0}};
 
   // sparsity + matrix
   int32_t *row_nnz = nullptr, *row_ptr = nullptr, *row_of = nullptr, *col = nullptr;

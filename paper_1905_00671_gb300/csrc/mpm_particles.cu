@@ -490,6 +490,8 @@ int run_first_bins(Ctx &c) {
   else
     k_fb_count<3><<<nblk(n), TPB, 0, c.st>>>(c.g, n, c.sh_first, c.sh_cnt, c.fb_key, c.fb_cursor, c.fb_cmax, c.err);
   UPMPM_LAUNCH(c);
+  // (the scan below synchronises)
+  cudaMemcpyAsync(c.h_cmax, c.fb_cmax, sizeof(int) * 3, cudaMemcpyDeviceToHost, c.st);
   if (scan_exclusive(c, c.fb_cursor, c.fb_start, nn + 1) != n) {
     int rc = read_dev_err(c);
     if (rc) return rc;
