@@ -210,10 +210,22 @@ def _options(w, stream, opts) -> mpm_options:
 _FIELDS = ("x", "u", "p", "v", "a", "F", "V", "lp", "pd", "pdd")
 
 
+def _touched(count):
+    """Host array for a device copy to fill, one word of every page written.
+
+    A copy into memory the host has not touched makes the GPU's copy engine
+    fault page by page (about 20 us each): reading back 12 MB took 0.5 to 8 ms
+    from np.zeros (whose pages are untouched unless the allocator recycles
+    some), 168 MB 58 ms; 0.2 and 8 ms when the host has touched them."""
+    a = np.empty(count)
+    a[::512] = 0.0  # 4 KiB
+    return a
+
+
 def _read(lib, ctx, n, d, fields, check):
     comps = {"x": d, "u": d, "p": 1, "v": d, "a": d, "F": d * d, "V": 1, "lp": d, "pd": 1,
              "pdd": 1}
-    out = {k: np.zeros((n, comps[k])) if comps[k] > 1 else np.zeros(n) for k in fields}
+    out = {k: _touched(n * comps[k]).reshape((n, comps[k]) if comps[k] > 1 else n) for k in fields}
     o = mpm_particles_out(**{k: _p(v) for k, v in out.items()})
     check(lib.mpm_read(ctx, C.byref(o)), "mpm_read")
     return out
