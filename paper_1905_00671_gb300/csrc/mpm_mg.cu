@@ -24,6 +24,7 @@
 // fixed summation order (deterministic, no atomics).
 #include <math.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "mpm_internal.cuh"

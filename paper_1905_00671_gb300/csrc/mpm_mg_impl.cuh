@@ -721,8 +721,11 @@ __global__ void k_dense_apply(int n, const real *__restrict__ Ai, const real *__
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   real s = 0.0;
-  if (i < n)
-    for (int j = lane; j < n; j += 32) s = fma(Ai[(int64_t)i * n + j], b[j], s);
+  if (i < n) {
+    const real *row = Ai + (int64_t)i * n;
+#pragma unroll 8
+    for (int j = lane; j < n; j += 32) s = fma(row[j], b[j], s);
+  }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (i < n && lane == 0) x[i] = s;
 }
@@ -809,128 +812,207 @@ __global__ void k_mg_prolong(LevelDev F, LevelDev Cl, real *__restrict__ xf,
   for (int i = 0; i < B; ++i) xf[a * B + i] += free_w(F, a, i) * acc[i];
 }
 
-// ---- coarse tail of a V-cycle in one thread block (FP32 hierarchies)
-// On the small coarse levels each kernel of a V-cycle is a few microseconds
-// of launch and drain for very little work; one block of 1024 threads runs the
-// whole tail (every level below a size limit down to the dense coarsest
-// solve) with a block barrier between the phases.  Same operations and order
-// of levels as the kernel-per-phase V(k, k) cycle.
-constexpr int TAIL_MAX_LEVELS = 8;
-constexpr int TAIL_MAX_NODES = 128;  // one pass of the block per phase: larger levels are latency-bound here
-constexpr int TAIL_THREADS = 1024;
+// ---- coarse tail of a V-cycle as one dense operator
+// From the first level of at most TAIL_MAX unknowns down, a V-cycle is a chain
+// of small kernels that each cost 2 to 4 us whatever their work (9 of the 45
+// kernels of an application per cycle on the 80k-point footing, every one on
+// the column).  That part of the cycle is a fixed linear map of its right-hand
+// side, so the set-up forms its matrix T by running the cycle on the unit
+// vectors (k_mg_tail_build), and an application is one product x = T b
+// (k_dense_apply): the same operator, its sums in another order.  The build
+// runs every column independently in shared memory, TAIL_COLS columns a block
+// (a level's blocks are read once for all of them), the two hierarchies of a
+// preconditioner side by side.
+// TAIL_MAX: a build costs about n^2 times a row's work (0.12 ms for the 966
+// unknowns of the harmonic footing's A-tail), a product n^2 FMAs (1.7 us of the
+// FP64 pipes at 1024).  An application on a GB300: column 37 -> 23 us, 17 x 17
+// deposit (FP32) 47 -> 19, harmonic footing 76 -> 46, 80k-point footing 139 -> 109,
+// 64 batched columns 430 -> 389; with 768 the harmonic footing keeps one level more.
+constexpr int TAIL_MAX = 1024;
+constexpr int TAIL_COLS = 4;
+constexpr int TAIL_LEVELS = 8;
+constexpr int TAIL_THREADS = 512;
 
-struct TailLevel {
-  LevelDev L;
-  real *x, *x2, *b, *r;
-};
 struct TailArgs {
   int nl;  // levels of the tail, the last one the dense coarsest level
-  TailLevel lv[TAIL_MAX_LEVELS];
-  const real *Ai;
-  int ncoarse;
+  LevelDev L[TAIL_LEVELS];
+  int st0;           // the first level is a stencil level (else the block-CSR finest level)
+  const real *Ai;    // inverse of the coarsest operator
+  int ncoarse, n;    // unknowns of the coarsest and of the tail's first level
   real omega;
-  int nsw;  // sweeps before and after the coarse correction
+  int nsw;
+  real *T;           // n x n, row-major
 };
 
-template <int B, int D, bool SMOOTH>
+// out = b - A x (SMOOTH: x + omega Dinv (b - A x)) for TAIL_COLS columns; vectors
+// [unknown][column]; a thread per row.  The thread's row sum is in slot order.
+template <int B, int D, bool ST, bool SMOOTH>
 __device__ inline void tail_rows(const LevelDev &L, const real *x, real *out, const real *b, real omega) {
-  constexpr int LN = LN_<D>::v;
-  const int64_t total = L.nnodes * LN;
-  for (int64_t base = 0; base < total; base += blockDim.x) {
-    const int64_t t = base + threadIdx.x;
-    const int64_t a = t / LN;
-    const int lane = (int)(t % LN);
-    const bool valid = a < L.nnodes;
-    real ax[B];
-    for (int i = 0; i < B; ++i) ax[i] = 0.0;
-    if (valid) row_partial<B, D, true, LN>(L, a, lane, x, ax);
-    lane_reduce<B, LN>(ax);
-    if (!valid || lane != 0) continue;
-    real r[B];
-    for (int i = 0; i < B; ++i) r[i] = b[a * B + i] - ax[i];
-    if (!SMOOTH) {
-      for (int i = 0; i < B; ++i) out[a * B + i] = r[i];
-      continue;
+  constexpr int NC = TAIL_COLS;
+  for (int a = threadIdx.x; a < (int)L.nnodes; a += blockDim.x) {
+    real acc[B][NC];
+#pragma unroll
+    for (int i = 0; i < B; ++i)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[i][c] = 0;
+    auto add = [&](const real *__restrict__ blk, int64_t nb) {
+#pragma unroll
+      for (int j = 0; j < B; ++j)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const real xv = x[(nb * B + j) * NC + c];
+#pragma unroll
+          for (int i = 0; i < B; ++i) acc[i][c] = fma(blk[i * B + j], xv, acc[i][c]);
+        }
+    };
+    if (!ST) {
+      for (int e = L.row_ptr[a]; e < L.row_ptr[a + 1]; ++e) add(L.val + (int64_t)e * B * B, L.col[e]);
+    } else if (L.nslot[a] != 0) {
+      int ac[3];
+      grid_xyz(L.nn[0], L.nn[1], a, ac);
+      const real *base = L.sval + (int64_t)a * NS_<D>::v * B * B;
+      for (int s = 0; s < NS_<D>::v; ++s) {
+        const int b0 = ac[0] + s % 5 - 2, b1 = ac[1] + (s / 5) % 5 - 2, b2 = ac[2] + (D == 3 ? s / 25 - 2 : 0);
+        if (b0 < 0 || b0 >= L.nn[0] || b1 < 0 || b1 >= L.nn[1] || b2 < 0 || b2 >= L.nn[2]) continue;
+        add(base + s * B * B, b0 + (int64_t)L.nn[0] * (b1 + (int64_t)L.nn[1] * b2));
+      }
     }
-    for (int i = 0; i < B; ++i) {
-      real sv = 0.0;
-      for (int j = 0; j < B; ++j) sv = fma(L.dinv[a * B * B + i * B + j], r[j], sv);
-      out[a * B + i] = x[a * B + i] + omega * sv;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      real r[B];
+#pragma unroll
+      for (int i = 0; i < B; ++i) r[i] = b[(a * B + i) * NC + c] - acc[i][c];
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        if (!SMOOTH) {
+          out[(a * B + i) * NC + c] = r[i];
+          continue;
+        }
+        real sv = 0;
+#pragma unroll
+        for (int j = 0; j < B; ++j) sv = fma(L.dinv[(int64_t)a * B * B + i * B + j], r[j], sv);
+        out[(a * B + i) * NC + c] = x[(a * B + i) * NC + c] + omega * sv;
+      }
     }
   }
 }
 
+template <int B, int D, bool SMOOTH>
+__device__ inline void tail_level(const TailArgs &A, int l, const real *x, real *out, const real *b) {
+  if (l == 0 && !A.st0) tail_rows<B, D, false, SMOOTH>(A.L[l], x, out, b, A.omega);
+  else tail_rows<B, D, true, SMOOTH>(A.L[l], x, out, b, A.omega);
+}
+
+// Columns c0 .. c0 + TAIL_COLS - 1 of T.  Dynamic shared memory: per level x,
+// b and r (x of the next sweep), tail_smem() bytes.
 template <int B, int D>
-__global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(TailArgs A) {
-  pdl_enter();
-  real *xs[TAIL_MAX_LEVELS], *x2s[TAIL_MAX_LEVELS];
+__device__ void tail_build(const TailArgs &A, int c0, real *sm) {
+  constexpr int NC = TAIL_COLS;
+  real *x[TAIL_LEVELS], *b[TAIL_LEVELS], *r[TAIL_LEVELS];
   for (int l = 0; l < A.nl; ++l) {
-    xs[l] = A.lv[l].x;
-    x2s[l] = A.lv[l].x2;
+    const int64_t n = A.L[l].nnodes * B * NC;
+    x[l] = sm;
+    b[l] = sm + n;
+    r[l] = sm + 2 * n;
+    sm += 3 * n;
   }
+  for (int t = threadIdx.x; t < A.n * NC; t += blockDim.x) b[0][t] = t / NC == c0 + t % NC ? real(1) : real(0);
+  __syncthreads();
+  auto swap = [](real *&p, real *&q) {
+    real *t = p;
+    p = q;
+    q = t;
+  };
   for (int l = 0; l + 1 < A.nl; ++l) {
-    const LevelDev &L = A.lv[l].L, &Ln = A.lv[l + 1].L;
-    for (int k = 1; k < A.nsw; ++k) {  // pre-smoothing sweeps after the first (from zero)
-      tail_rows<B, D, true>(L, xs[l], x2s[l], A.lv[l].b, A.omega);
-      __syncthreads();
-      real *t = xs[l]; xs[l] = x2s[l]; x2s[l] = t;
+    const LevelDev &L = A.L[l], &Ln = A.L[l + 1];
+    // first sweep from zero: x = omega Dinv b
+    for (int t = threadIdx.x; t < (int)L.nnodes * B * NC; t += blockDim.x) {
+      const int c = t % NC, a = t / NC / B, i = t / NC % B;
+      real sv = 0;
+      for (int j = 0; j < B; ++j) sv = fma(L.dinv[(int64_t)a * B * B + i * B + j], b[l][(a * B + j) * NC + c], sv);
+      x[l][t] = A.omega * sv;
     }
-    tail_rows<B, D, false>(L, xs[l], A.lv[l].r, A.lv[l].b, A.omega);
     __syncthreads();
-    real *xc = l + 2 < A.nl ? xs[l + 1] : nullptr;  // first sweep from zero of the next level
-    for (int64_t I = threadIdx.x; I < Ln.nnodes; I += blockDim.x) {
+    for (int k = 1; k < A.nsw; ++k) {
+      tail_level<B, D, true>(A, l, x[l], r[l], b[l]);
+      __syncthreads();
+      swap(x[l], r[l]);
+    }
+    tail_level<B, D, false>(A, l, x[l], r[l], b[l]);
+    __syncthreads();
+    for (int t = threadIdx.x; t < (int)Ln.nnodes * B * NC; t += blockDim.x) {  // restriction
+      const int c = t % NC, I = t / NC / B, i = t / NC % B;
       int Ic[3];
-      grid_xyz(Ln.nn[0], Ln.nn[1], (int)I, Ic);
-      real acc[B];
-      for (int i = 0; i < B; ++i) acc[i] = 0.0;
+      grid_xyz(Ln.nn[0], Ln.nn[1], I, Ic);
+      real acc = 0;
       const int lo2 = D == 3 ? -1 : 0, hi2 = D == 3 ? 1 : 0;
       for (int d2 = lo2; d2 <= hi2; ++d2)
         for (int d1 = -1; d1 <= 1; ++d1)
           for (int d0 = -1; d0 <= 1; ++d0) {
             const int a0 = 2 * Ic[0] + d0, a1 = 2 * Ic[1] + d1, a2 = D == 3 ? 2 * Ic[2] + d2 : 0;
             if (a0 < 0 || a0 >= L.nn[0] || a1 < 0 || a1 >= L.nn[1] || a2 < 0 || a2 >= L.nn[2]) continue;
-            const real wgt = pw(a0, Ic[0]) * pw(a1, Ic[1]) * (D == 3 ? pw(a2, Ic[2]) : 1.0);
             const int64_t a = a0 + (int64_t)L.nn[0] * (a1 + (int64_t)L.nn[1] * a2);
             if (L.inst && L.inst[a] != Ln.inst[I]) continue;
-            for (int i = 0; i < B; ++i) acc[i] += wgt * A.lv[l].r[a * B + i];
+            const real wgt = pw(a0, Ic[0]) * pw(a1, Ic[1]) * (D == 3 ? pw(a2, Ic[2]) : real(1));
+            acc += wgt * free_w(L, a, i) * r[l][(a * B + i) * NC + c];
           }
-      for (int i = 0; i < B; ++i) A.lv[l + 1].b[I * B + i] = acc[i];
-      if (xc)
-        for (int i = 0; i < B; ++i) {
-          real sv = 0.0;
-          for (int j = 0; j < B; ++j) sv = fma(Ln.dinv[I * B * B + i * B + j], acc[j], sv);
-          xc[I * B + i] = A.omega * sv;
-        }
+      b[l + 1][t] = acc;
     }
     __syncthreads();
   }
-  {  // dense coarsest solve, one warp per row
+  {  // exact solve on the coarsest grid
     const int lc = A.nl - 1;
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i < A.ncoarse; i += blockDim.x >> 5) {
-      real sv = 0.0;
-      for (int j = lane; j < A.ncoarse; j += 32) sv = fma(A.Ai[(int64_t)i * A.ncoarse + j], A.lv[lc].b[j], sv);
-      for (int o = 16; o > 0; o >>= 1) sv += __shfl_xor_sync(0xffffffffu, sv, o);
-      if (lane == 0) xs[lc][i] = sv;
+    for (int t = threadIdx.x; t < A.ncoarse * NC; t += blockDim.x) {
+      const int c = t % NC, i = t / NC;
+      real sv = 0;
+      for (int j = 0; j < A.ncoarse; ++j) sv = fma(A.Ai[(int64_t)i * A.ncoarse + j], b[lc][j * NC + c], sv);
+      x[lc][t] = sv;
     }
     __syncthreads();
   }
   for (int l = A.nl - 2; l >= 0; --l) {
-    const LevelDev &L = A.lv[l].L, &Ln = A.lv[l + 1].L;
-    for (int64_t a = threadIdx.x; a < L.nnodes; a += blockDim.x) {
+    const LevelDev &L = A.L[l], &Ln = A.L[l + 1];
+    for (int t = threadIdx.x; t < (int)L.nnodes * B * NC; t += blockDim.x) {  // prolongation
+      const int c = t % NC, a = t / NC / B, i = t / NC % B;
       int ac[3];
-      grid_xyz(L.nn[0], L.nn[1], (int)a, ac);
-      real acc[B];
-      prolong_at<B, D>(Ln, xs[l + 1], ac, L.inst ? L.inst[a] : 0, acc);
-      for (int i = 0; i < B; ++i) xs[l][a * B + i] += acc[i];
+      grid_xyz(L.nn[0], L.nn[1], a, ac);
+      const int inst_a = L.inst ? L.inst[a] : 0;
+      real acc = 0;
+      for (int cmb = 0; cmb < (1 << D); ++cmb) {
+        real w = 1;
+        int I[3] = {0, 0, 0};
+        for (int k = 0; k < D; ++k) {
+          const int odd = ac[k] & 1, up = (cmb >> k) & 1;
+          I[k] = (ac[k] >> 1) + up;
+          w *= up ? (odd && I[k] < Ln.nn[k] ? real(0.5) : real(0)) : (odd ? real(0.5) : real(1));
+        }
+        if (w == real(0)) continue;
+        const int64_t In = I[0] + (int64_t)Ln.nn[0] * (I[1] + (int64_t)Ln.nn[1] * I[2]);
+        if (Ln.inst && Ln.inst[In] != inst_a) continue;
+        acc = fma(w, x[l + 1][(In * B + i) * NC + c], acc);
+      }
+      x[l][t] += free_w(L, a, i) * acc;
     }
     __syncthreads();
-    for (int k = 0; k < A.nsw; ++k) {  // post-smoothing sweeps
-      tail_rows<B, D, true>(L, xs[l], x2s[l], A.lv[l].b, A.omega);
+    for (int k = 0; k < A.nsw; ++k) {
+      tail_level<B, D, true>(A, l, x[l], r[l], b[l]);
       __syncthreads();
-      real *t = xs[l]; xs[l] = x2s[l]; x2s[l] = t;
+      swap(x[l], r[l]);
     }
   }
+  for (int t = threadIdx.x; t < A.n * NC; t += blockDim.x) {
+    const int c = c0 + t % NC;
+    if (c < A.n) A.T[(int64_t)(t / NC) * A.n + c] = x[0][t];
+  }
+}
+
+// blocks 0 .. nblk0 - 1: the A hierarchy (B = D), the others the S hierarchy
+template <int D>
+__global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail_build(TailArgs A, TailArgs S, int nblk0) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  real *sm = reinterpret_cast<real *>(dyn_smem);
+  if ((int)blockIdx.x < nblk0) tail_build<D, D>(A, blockIdx.x * TAIL_COLS, sm);
+  else tail_build<1, D>(S, ((int)blockIdx.x - nblk0) * TAIL_COLS, sm);
 }
 
 // Galerkin product P^T A P in two passes, from the block-CSR finest level
@@ -1090,6 +1172,8 @@ struct MGHier<MG_REAL> {
   int *piv = nullptr;                    // row interchanges of the LU factorisation
   MG_REAL *apT = nullptr;                // finest level x 5^d window: A P, first pass of a level's product
   int ncoarse = 0;                       // unknowns of the coarsest level
+  int tail = 15;                         // first level of the dense tail (nlev - 1: the coarsest alone)
+  MG_REAL *T = nullptr;                  // its operator
 };
 
 namespace MG_NS {
@@ -1143,6 +1227,45 @@ void dense_invert_pair(Ctx &c, MGHier<real> &H0, MGHier<real> &H1) {
   c.launches += 2;
 }
 
+real mg_omega(const Ctx &c);
+
+// Dense tail operators of the two hierarchies (after the coarsest inverses).
+// finest_only: the coarse levels are those of an earlier set-up, so only a tail
+// that starts at the finest level has changed.
+void tail_build_pair(Ctx &c, MGHier<real> &HA, MGHier<real> &HS, bool finest_only) {
+  auto args = [&](MGHier<real> &H, size_t *smem) {
+    TailArgs A{};
+    if (H.tail == H.nlev - 1 || (finest_only && H.tail > 0)) return A;
+    A.nl = H.nlev - H.tail;
+    int64_t vals = 0;
+    for (int l = 0; l < A.nl; ++l) {
+      A.L[l] = H.L[H.tail + l];
+      vals += 3 * A.L[l].nnodes * H.B * TAIL_COLS;
+    }
+    A.st0 = H.tail > 0;
+    A.Ai = H.Ai;
+    A.ncoarse = H.ncoarse;
+    A.n = (int)(A.L[0].nnodes * H.B);
+    A.omega = mg_omega(c);
+    A.nsw = c.mg_sweeps();
+    A.T = H.T;
+    *smem = std::max(*smem, sizeof(real) * (size_t)vals);
+    return A;
+  };
+  size_t smem = 0;
+  const TailArgs A = args(HA, &smem), S = args(HS, &smem);
+  const int na = nblk(A.n, TAIL_COLS), ns = nblk(S.n, TAIL_COLS);
+  if (na + ns == 0) return;
+  if (c.d == 2) {
+    cudaFuncSetAttribute(k_mg_tail_build<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_mg_tail_build<2><<<na + ns, TAIL_THREADS, smem, c.st>>>(A, S, na);
+  } else {
+    cudaFuncSetAttribute(k_mg_tail_build<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_mg_tail_build<3><<<na + ns, TAIL_THREADS, smem, c.st>>>(A, S, na);
+  }
+  UPMPM_LAUNCH(c);
+}
+
 // Damping of the block-Jacobi smoother.  A damped Jacobi sweep is stable only
 // while omega * lambda_max(Dinv A) < 2 on every level.  Measured lambda_max:
 // at most 2.5 for the plane-strain blocks of the strip footing (2D), 3.25 on
@@ -1153,7 +1276,7 @@ void dense_invert_pair(Ctx &c, MGHier<real> &H0, MGHier<real> &H1) {
 // fewer FGMRES iterations than V(2,2) at 0.56 of its cost per application,
 // and V(3,3) stalled there.
 // (the defaults of Ctx::mg_omega; mpm_options.mg_omega overrides them)
-inline real mg_omega(const Ctx &c) { return (real)c.mg_omega(); }
+real mg_omega(const Ctx &c) { return (real)c.mg_omega(); }
 
 // one damped block-Jacobi sweep on level l: x <- x + omega Dinv (b - A x)
 template <int B, int D>
@@ -1182,27 +1305,16 @@ void sweep(Ctx &c, MGHier<real> &H, int l) {
 // the result.
 template <int B, int D>
 void vcycle_t(Ctx &c, MGHier<real> &H, int l) {
-  if (sizeof(real) == sizeof(float) && l >= 1 && l < H.nlev - 1 && H.L[l].nnodes <= TAIL_MAX_NODES &&
-      H.nlev - l <= TAIL_MAX_LEVELS) {  // the rest of the cycle in one block
-    TailArgs A{};
-    A.nl = H.nlev - l;
-    for (int k = 0; k < A.nl; ++k) A.lv[k] = TailLevel{H.L[l + k], H.x[l + k], H.x2[l + k], H.b[l + k], H.r[l + k]};
-    A.Ai = H.Ai;
-    A.ncoarse = H.ncoarse;
-    A.omega = mg_omega(c);
-    A.nsw = c.mg_sweeps();
-    launch_pdl(c, k_mg_tail<B, D>, 1, TAIL_THREADS, 0, A);
-    // 2 nsw - 1 sweeps per level (odd) swapped x and x2 (as sweep() does on the host)
-    for (int k = l; k < H.nlev - 1; ++k) std::swap(H.x[k], H.x2[k]);
-    return;
-  }
-  if (l == H.nlev - 1) {  // exact solve on the coarsest grid
-    const Geom g = geom(c, (int64_t)H.ncoarse * 32);
-    launch_pdl(c, k_dense_apply, g.blocks, g.tpb, 0, H.ncoarse, (const real *)H.Ai, (const real *)H.b[l], H.x[l]);
+  if (l == H.tail) {  // the rest of the cycle (the exact solve on the coarsest grid)
+    const bool last = l == H.nlev - 1;
+    const int n = (int)(H.L[l].nnodes * B);
+    const Geom g = geom(c, (int64_t)n * 32);
+    launch_pdl(c, k_dense_apply, g.blocks, g.tpb, 0, n, (const real *)(last ? H.Ai : H.T), (const real *)H.b[l],
+               H.x[l]);
     return;
   }
   LevelDev &L = H.L[l], &Ln = H.L[l + 1];
-  real *xn_first = l + 1 == H.nlev - 1 ? nullptr : H.x[l + 1];
+  real *xn_first = l + 1 == H.tail ? nullptr : H.x[l + 1];
   for (int k = 1; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // pre-smoothing after the first
   const Geom gr = geom(c, L.nnodes * LN_<D>::v), gc = geom(c, Ln.nnodes), gf = geom(c, L.nnodes);
   if (l == 0 && B <= 2) {
@@ -1296,6 +1408,12 @@ int mg_alloc(Ctx &c, MGHier<real> &H, int B) {
   if (cudaMalloc(&H.Ad, sizeof(real) * H.ncoarse * H.ncoarse) ||
       cudaMalloc(&H.Ai, sizeof(real) * H.ncoarse * H.ncoarse) || cudaMalloc(&H.piv, sizeof(int) * H.ncoarse))
     return MPM_ERR_NO_MEMORY;
+  H.tail = H.nlev - 1;
+  while (H.tail > 0 && H.L[H.tail - 1].nnodes * B <= TAIL_MAX && H.nlev - H.tail < TAIL_LEVELS) --H.tail;
+  if (H.tail < H.nlev - 1) {
+    const int64_t n = H.L[H.tail].nnodes * B;
+    if (cudaMalloc(&H.T, sizeof(real) * n * n)) return MPM_ERR_NO_MEMORY;
+  }
   if (H.nlev > 1 && cudaMalloc(&H.apT, sizeof(real) * H.L[0].nnodes * NS * B * B)) return MPM_ERR_NO_MEMORY;
   return MPM_OK;
 }
@@ -1305,7 +1423,8 @@ void mg_free(MGHier<real> &H) {
   cudaFree(H.Ai);
   cudaFree(H.piv);
   cudaFree(H.apT);
-  H.Ad = H.Ai = H.apT = nullptr;
+  cudaFree(H.T);
+  H.Ad = H.Ai = H.apT = H.T = nullptr;
   H.piv = nullptr;
   for (int l = 0; l < H.nlev; ++l) {
     cudaFree(const_cast<int32_t *>(H.L[l].inst));
@@ -1465,6 +1584,7 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
     S.coarse_built = true;
     S.coarse_step = c.steps;
   }
+  tail_build_pair(c, *S.mgA, *S.mgS, !full);
   return check_cuda(c, cudaGetLastError(), "schur setup");
 }
 
