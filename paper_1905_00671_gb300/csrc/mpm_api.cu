@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <new>
 #include <string>
 
@@ -65,11 +66,44 @@ int check_cuda(Ctx &c, cudaError_t e, const char *what) {
   return MPM_ERR_CUDA;
 }
 
-int read_dev_err(Ctx &c) {
-  cudaMemcpyAsync(c.h_err, c.err, sizeof(int), cudaMemcpyDeviceToHost, c.st);
-  cudaError_t e = cudaStreamSynchronize(c.st);
-  if (e != cudaSuccess) return check_cuda(c, e, "kernel execution");
-  const int f = *c.h_err;
+// A word no kernel writes (a NaN pattern of its own).
+constexpr uint64_t SLOT_EMPTY = 0xfff8a5a5a5a5a5a5ull;
+
+void slot_reset(Ctx &c, int slot) {
+  *reinterpret_cast<volatile uint64_t *>(c.h_slot + slot) = SLOT_EMPTY;
+  std::atomic_thread_fence(std::memory_order_release);
+}
+
+int slot_wait(Ctx &c, int slot, double *value) {
+  const volatile uint64_t *p = reinterpret_cast<const volatile uint64_t *>(c.h_slot + slot);
+  bool idle = false;  // the stream had finished before the last look at the word
+  for (unsigned n = 1;; ++n) {
+    const uint64_t v = *p;
+    if (v != SLOT_EMPTY) {
+      std::atomic_thread_fence(std::memory_order_acquire);
+      memcpy(value, const_cast<const uint64_t *>(&v), sizeof(double));
+      return MPM_OK;
+    }
+    if (idle) {
+      c.last_error = "a result was not written by the kernels that should have";
+      return MPM_ERR_CUDA;
+    }
+    if (n % 4096 == 0) {  // a failed launch or kernel never writes it
+      cudaError_t e = cudaPeekAtLastError();
+      if (e == cudaSuccess) {
+        e = cudaStreamQuery(c.st);
+        if (e == cudaErrorNotReady) {
+          cudaGetLastError();
+          continue;
+        }
+      }
+      if (e != cudaSuccess) return check_cuda(c, e, "kernel execution");
+      idle = true;
+    }
+  }
+}
+
+int dev_err_code(Ctx &c, int f) {
   if (!f) return MPM_OK;
   cudaMemsetAsync(c.err, 0, sizeof(int), c.st);
   if (f & DE_OUT_OF_GRID) {
@@ -333,15 +367,13 @@ int prepare_step(Ctx &c, double dt, const mpm_loads *L, const mpm_bcs *B) {
 
 int eval_residual(Ctx &c, double *rnorm) {
   run_point_eval(c, c.X);
-  int rc = read_dev_err(c);
-  if (rc) return rc;
   run_residual(c, c.X, c.R, 1);
   if (c.ninst > 1) {  // per-instance norms (h_inorm) for the Newton test
     k_inst_norm<<<c.ninst, 256, 0, c.st>>>(c.g, c.nb, c.inst, c.R, c.inorm);
     UPMPM_LAUNCH(c);
     cudaMemcpyAsync(c.h_inorm, c.inorm, sizeof(double) * c.ninst, cudaMemcpyDeviceToHost, c.st);
   }
-  *rnorm = run_norm(c, c.R);  // synchronises
+  if (int rc = run_norm(c, c.R, rnorm)) return rc;  // waits; also the point evaluation's error word
   if (!isfinite(*rnorm)) {
     c.last_error = "non-finite residual";
     return MPM_ERR_NONFINITE;
@@ -376,8 +408,8 @@ int newton_correction(Ctx &c, LinSys<T> &S, int k, int *its) {
     run_block_jacobi<T>(c, S);
   }
   prof_end(c, MPM_PROF_SETUP);
-  rc = read_dev_err(c);
-  if (rc) return rc;
+  // (the Schur preconditioner's set-up raises no device error)
+  if (c.opt.precond != MPM_PRECOND_SCHUR_MG && (rc = read_dev_err(c))) return rc;
   const bool inexact = sizeof(T) < sizeof(double);
   const double rtol = inexact ? fmax(c.opt.krylov_rtol, 1e-6) : c.opt.krylov_rtol;
   rc = run_fgmres<T>(c, S, rtol, c.opt.krylov_max, its);
@@ -465,7 +497,8 @@ int do_step(Ctx &c, double dt, const mpm_loads *L, const mpm_bcs *B) {
   if (rc) return rc;
   run_g2p(c);
   cudaMemcpyAsync(c.h_terms, c.terms, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c.st);
-  rc = read_dev_err(c);  // synchronises the stream
+  rc = read_dev_err(c);
+  if (!rc) rc = check_cuda(c, cudaStreamSynchronize(c.st), "step");
   if (rc) return rc;
   c.stats.jac_terms = (int64_t)c.h_terms[0];
   c.stats.jac_point_nodes = (int64_t)c.h_terms[1];
@@ -493,15 +526,15 @@ void free_all(Ctx &c) {
                   c.sh_S0, c.m, c.rec, c.pn, c.M, c.Pn, c.vn, c.an, c.pdn, c.pddn, c.phi, c.act, c.fsd, c.sh_nrm, c.fixed, c.u_fixed,
                   c.p_fixed, c.u_value, c.p_value, c.trac, c.trac_raw, c.flux, c.err, c.row_nnz,
                   c.row_ptr, c.row_of, c.col, c.row_mask, c.X, c.R, c.dX, c.stage, c.H, c.gvec,
-                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i};
+                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (c.h_inorm) cudaFreeHost(c.h_inorm);
   if (c.h_bk) cudaFreeHost(c.h_bk);
-  if (c.h_err) cudaFreeHost(c.h_err);
   if (c.h_scalar) cudaFreeHost(c.h_scalar);
   if (c.h_terms) cudaFreeHost(c.h_terms);
   if (c.h_cmax) cudaFreeHost(c.h_cmax);
+  if (c.h_slot) cudaFreeHost(c.h_slot);
   if (c.own_stream && c.st) cudaStreamDestroy(c.st);
   c.st = nullptr;
 }
@@ -728,6 +761,8 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   A(&c.hcol, 2 * 129);
   A(&c.part, 304 * 129);
   A(&c.scal, 8);
+  A(&c.ctl, 1);
+  A(&c.npart, 304);
   c.scan_cap = 4096;
   A(&c.scan_tmp, c.scan_cap);
   c.have32 = c.precision == MPM_MIXED;
@@ -743,7 +778,8 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   }
   if (!rc) rc = linsys_alloc<double>(c, c.L64, !c.have32);
   if (!rc && c.have32) rc = linsys_alloc<float>(c, c.L32, true);
-  if (!rc && cudaHostAlloc((void **)&c.h_err, sizeof(int), cudaHostAllocDefault) != cudaSuccess)
+  if (!rc && (cudaHostAlloc((void **)&c.h_slot, SLOTS * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+              cudaHostGetDevicePointer((void **)&c.d_slot, c.h_slot, 0) != cudaSuccess))
     rc = MPM_ERR_NO_MEMORY;
   if (!rc && cudaHostAlloc((void **)&c.h_scalar, 8 * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
     rc = MPM_ERR_NO_MEMORY;

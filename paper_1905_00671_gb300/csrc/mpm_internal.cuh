@@ -60,6 +60,34 @@ struct LinSys {
   int g_lower = 0;     // order the graph was captured for
   const void *gkey_col = nullptr, *gkey_val = nullptr;
   int64_t gkernels = 0;
+  // One FGMRES iteration (multigrid core, merge, product, Gram-Schmidt, Givens,
+  // next basis vector with its split) as a CUDA graph, for single-instance
+  // systems below KRYLOV_GRAPH_MAX unknowns; it reads the iteration's number
+  // from ctl.  Dropped and captured again like gexec.
+  cudaGraphExec_t itexec = nullptr;
+  T *it_x0 = nullptr;  // the first sub-solve's first sweep at capture time
+  const void *itkey_col = nullptr, *itkey_val = nullptr;
+  int64_t itkernels = 0;
+};
+
+// The split of a scaled vector v into the right-hand side of the
+// preconditioner's first sub-solve (b0), its first sweep from zero
+// (x0 = omega dinv b0) and the other block's part (other), per node.
+template <typename T>
+struct SplitP {
+  const T *dsi;  // D^-1
+  const T *dinv;
+  T *b0, *x0, *other;
+  T omega;
+  int lower;     // first sub-solve: the displacement block (else the pressure's)
+};
+// Control words of the FGMRES iteration on the device: the column being built
+// (x) and whether it waits for a second Gram-Schmidt pass (y).  The finishing
+// kernel of an iteration writes next, the merge kernel of the following one
+// reads next and writes cur, and every kernel between reads cur: no kernel
+// reads a word that one of its own blocks writes.
+struct KrylovCtl {
+  int2 cur, next;
 };
 
 // 64-bit words of the per-node coupling mask of the block sparsity: bit
@@ -298,7 +326,6 @@ struct Ctx {
   int has_flux = 0;
   double trac_scale = 1.0;
   int *err = nullptr;
-  int *h_err = nullptr;                  // pinned
   double *h_scalar = nullptr;            // pinned scratch for scalars read by the host
   unsigned long long *terms = nullptr;   // device: Jacobian term counts (n_p^2, n_p sums)
   // consistent-mass Stage 1: the mass on the node pattern and the CG workspace
@@ -350,6 +377,12 @@ struct Ctx {
   bool have32 = false;
   double *H = nullptr, *gvec = nullptr, *cs = nullptr, *sn = nullptr, *yv = nullptr;
   double *hcol = nullptr, *part = nullptr, *scal = nullptr;
+  KrylovCtl *ctl = nullptr;              // FGMRES control word
+  double *npart = nullptr;               // partial squared norms of the Gram-Schmidt updates
+  // results the host waits for: words of mapped pinned memory that kernels
+  // write and the host polls (slot_reset / slot_wait), against a copy and a
+  // stream synchronisation each
+  double *h_slot = nullptr, *d_slot = nullptr;
 
   // scan scratch
   int32_t *scan_tmp = nullptr;
@@ -407,7 +440,8 @@ void run_precond(Ctx &c, LinSys<T> &S, const T *v, T *z);  // z = M^{-1} v (scal
 template <typename T>
 void run_unscale_add(Ctx &c, const LinSys<T> &S, double *X);  // X += D x
 
-double run_norm(Ctx &c, const double *x);          // synchronises
+// |x| and the device error word (waits for both); an MPM_ERR_* code of the latter
+int run_norm(Ctx &c, const double *x, double *norm);
 
 // Schur-complement multigrid preconditioner
 template <typename T>
@@ -419,13 +453,27 @@ int schur_setup(Ctx &c, LinSys<T> &S, bool coarse = true);  // before run_scale_
                                                              // coarse = false: the finest levels only
 template <typename T>
 void schur_apply(Ctx &c, LinSys<T> &S, const T *v, T *z);  // z = M^{-1} v
+// its parts, for a caller that captures them: the split's buffers as they are
+// before the core, and the core (results in *zu, *zp)
+template <typename T>
+SplitP<T> schur_split_args(Ctx &c, LinSys<T> &S);
+template <typename T>
+void schur_core_launch(Ctx &c, LinSys<T> &S, const T **zu, const T **zp);
+
+// Mapped result words.  A reset word holds a bit pattern no result has; the
+// wait returns the word once a kernel has written it, or reports a failed or
+// finished stream that never did.
+constexpr int SLOTS = 192, SLOT_BETA = 130, SLOT_NORM = 131, SLOT_ERR = 132, SLOT_SCAN = 133, SLOT_WORD = 134;
+void slot_reset(Ctx &c, int slot);
+int slot_wait(Ctx &c, int slot, double *value);
 
 // scan: out[i] = sum_{j<i} in[j]; returns the total (synchronises)
 int64_t scan_exclusive(Ctx &c, const int32_t *in, int32_t *out, int64_t n);
 
 // helpers
 int check_cuda(Ctx &c, cudaError_t e, const char *what);
-int read_dev_err(Ctx &c);   // synchronises; returns MPM_ERR_* or 0
+int read_dev_err(Ctx &c);   // waits for the work before it; returns MPM_ERR_* or 0
+int dev_err_code(Ctx &c, int f);  // the code of a device error word (clears it on the device)
 
 #define UPMPM_LAUNCH(ctx) ((ctx).launches++)
 
@@ -441,6 +489,12 @@ int read_dev_err(Ctx &c);   // synchronises; returns MPM_ERR_* or 0
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Write a mapped result word that the host polls (one word carries the whole
+// result, so no fence orders it against others).
+__device__ __forceinline__ void slot_write(double *slot, double v) {
+  *reinterpret_cast<volatile double *>(slot) = v;
 }
 
 template <typename... P, typename... A>

@@ -1506,7 +1506,8 @@ void schur_free<MG_REAL>(LinSys<MG_REAL> &S) {
   for (MG_REAL *p : ptrs) cudaFree(p);
   S.Aval = S.Sval = S.B1c = S.W = S.B1rs = S.DAinv = S.vu = S.B2c = S.vp = nullptr;
   if (S.gexec) cudaGraphExecDestroy(S.gexec);
-  S.gexec = nullptr;
+  if (S.itexec) cudaGraphExecDestroy(S.itexec);
+  S.gexec = S.itexec = nullptr;
   S.gkey_col = S.gkey_val = nullptr;
   S.g_x0 = S.g_zp = S.g_zu = nullptr;
   S.sub_cap = 0;
@@ -1523,7 +1524,8 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
     // the captured graph reads these buffers (B1c, and Aval / Sval through
     // the finest multigrid level): drop it, it is re-captured on next use
     if (S.gexec) cudaGraphExecDestroy(S.gexec);
-    S.gexec = nullptr;
+    if (S.itexec) cudaGraphExecDestroy(S.itexec);
+    S.gexec = S.itexec = nullptr;
     MG_REAL *ptrs[] = {S.Aval, S.Sval, S.B1c, S.W, S.B2c};
     for (MG_REAL *p : ptrs) cudaFree(p);
     S.Aval = S.Sval = S.B1c = S.W = S.B2c = nullptr;
@@ -1648,6 +1650,22 @@ void schur_merge(Ctx &c, LinSys<MG_REAL> &S, const MG_REAL *zu, const MG_REAL *z
   else launch_pdl(c, k_merge<3>, g.blocks, g.tpb, 0, nn, zu, zp, dsc, z);
 }
 }  // namespace MG_NS
+
+template <>
+SplitP<MG_REAL> schur_split_args<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S) {
+  using namespace MG_NS;
+  const int lower = c.schur_lower();
+  MGHier<real> &H = lower ? *S.mgA : *S.mgS;
+  return SplitP<MG_REAL>{S.dscinv, H.L[0].dinv, H.b[0], H.x[0], lower ? S.vp : S.vu, mg_omega(c), lower};
+}
+
+template <>
+void schur_core_launch<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, const MG_REAL **zu, const MG_REAL **zp) {
+  using namespace MG_NS;
+  schur_core(c, S);
+  *zu = S.mgA->x[0];
+  *zp = S.mgS->x[0];
+}
 
 // The multigrid core is a fixed sequence of small kernels on fixed buffers: it
 // is captured once into a CUDA graph and replayed between the split and merge

@@ -108,13 +108,13 @@ __global__ void k_scan_top(int32_t *__restrict__ blk, int nb) {
 }
 
 __global__ void k_scan_add(int32_t *__restrict__ out, int64_t n, const int32_t *__restrict__ blk,
-                           const int32_t *__restrict__ in, double *__restrict__ total_out) {
+                           const int32_t *__restrict__ in, double *total_out) {
   const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_I;
   const int32_t add = blk[blockIdx.x];
   for (int i = 0; i < SCAN_I; ++i)
     if (base + i < n) {
       out[base + i] += add;
-      if (base + i == n - 1) total_out[0] = (double)out[base + i] + (double)in[base + i];
+      if (base + i == n - 1) slot_write(total_out, (double)out[base + i] + (double)in[base + i]);
     }
 }
 
@@ -138,6 +138,21 @@ __global__ void k_reduce(const double *__restrict__ part, int np, double *__rest
   acc = block_sum(acc);
   if (threadIdx.x == 0) out[0] = acc;
 }
+
+// The same into a mapped result word, with the device error word beside it.
+__global__ void k_reduce_post(const double *__restrict__ part, int np, const int *__restrict__ err, double *out,
+                              double *out_err) {
+  pdl_enter();
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) acc += part[i];
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) {
+    slot_write(out_err, (double)*err);
+    slot_write(out, acc);
+  }
+}
+
+__global__ void k_post_err(const int *__restrict__ err, double *out) { slot_write(out, (double)*err); }
 
 template <typename T>
 __global__ void k_scale_copy(T *__restrict__ y, const T *__restrict__ x, const double *s, int64_t n) {
@@ -312,8 +327,14 @@ __global__ void k_bj_apply(int64_t nnodes, const T *__restrict__ dinv, const T *
 template <int NB, int SPL, typename T>
 __global__ void k_bsr_spmv(int64_t nnodes, const int32_t *__restrict__ row_ptr,
                            const int32_t *__restrict__ col, const T *__restrict__ val,
-                           const T *__restrict__ x, T *__restrict__ y) {
+                           const T *__restrict__ x, T *__restrict__ y, const KrylovCtl *__restrict__ ctl,
+                           int64_t xstride) {
   pdl_enter();
+  if (ctl) {  // iteration graph: x is the vector of the iteration's number
+    const int2 it = ctl->cur;
+    if (it.y) return;
+    x += it.x * xstride;
+  }
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t o = t / SPL;
   const int part = (int)(t - o * SPL);
@@ -471,14 +492,292 @@ __global__ void k_update_x(T *__restrict__ x, const T *__restrict__ Z, const dou
   x[k] = s;
 }
 
+// ------------------------------------- one iteration as a CUDA graph
+// Below KRYLOV_GRAPH_MAX unknowns an FGMRES iteration is a chain of kernels of
+// a few microseconds, and what it costs is their number, their launches and the
+// host's read of the residual estimate.  So the whole iteration is one graph:
+// its kernels read the iteration's number from a control word; the reductions
+// of partial sums are done by every block of the kernel that needs them (no
+// kernel of their own); the kernel that scales the next basis vector also
+// finishes the Arnoldi column and splits the vector for the preconditioner; the
+// estimate is written to mapped host memory, which the host polls; and the
+// host launches iteration j + 1 before it has seen j's estimate while the last
+// one seen is far above the target (SPEC_MARGIN), so that the GPU does not wait
+// for it.  An iteration launched past convergence is not counted and leaves
+// the solution alone (it writes column j + 1 and later words only).
+// In FP64 the second Gram-Schmidt pass is rare (REORTH_THETA): the finishing
+// kernel then only raises ctl->halt, which stops what was launched ahead, and
+// the host launches the second pass.
+// Against kernels launched one by one with a reduction kernel per pass and a
+// copy and stream synchronisation per iteration (GB300, whole steps): column 2.40 ->
+// 1.61 ms (25 iterations), 17 x 17 deposit in FP32 6.45 -> 4.52 (70), harmonic
+// footing 6.3 -> 5.1 (43), 80k-point footing 11.3 -> 9.9 (50), 50k-point footing in
+// FP32 12.7 -> 10.6 (83), 163k-point block 48.9 -> 47.0 (60).  From
+// KRYLOV_GRAPH_MAX unknowns on, an iteration takes milliseconds and the kernels
+// with a grid sized to the iteration serve.
+constexpr int64_t KRYLOV_GRAPH_MAX = 1 << 20;
+constexpr double SPEC_MARGIN = 16.0;
+constexpr double EST_REORTH = -2.0;  // posted instead of an estimate: second pass needed
+constexpr int GS_SLICE = 512;        // vector elements per block of the inner products
+
+// part[b * PSTR + i] = block (b, .)'s part of V_i . w, i < cnt (= ctl->j + 1), and
+// of w . w at i = cnt (with_norm): a warp per product and slice, all of them side
+// by side (the grid has blocks for m products; those past cnt leave at once)
+template <typename T>
+__global__ void k_gs_dots(const T *__restrict__ V, const T *__restrict__ w, int64_t n, int64_t slice,
+                          const KrylovCtl *__restrict__ ctl, int with_norm, int force, double *__restrict__ part) {
+  pdl_enter();
+  const int2 it = ctl->cur;
+  if (it.y && !force) return;
+  const int cnt = it.x + 1, lane = threadIdx.x & 31;
+  const int i = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i >= cnt + with_norm) return;
+  const int64_t k0 = blockIdx.x * slice, k1 = min(k0 + slice, n);
+  const T *vi = i < cnt ? V + (int64_t)i * n : w;
+  T acc = 0;
+#pragma unroll 8
+  for (int64_t k = k0 + lane; k < k1; k += 32) acc += vi[k] * w[k];
+  double s = (double)acc;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) part[(int64_t)blockIdx.x * PSTR + i] = s;
+}
+
+// w -= sum_i h_i V_i with h summed from the np partials here; block 0 keeps h
+// (with |w|^2 at h[cnt] when with_norm); npart: partial squared norms of the
+// result (null: not wanted)
+template <typename T>
+__global__ void k_gs_update(T *__restrict__ w, const T *__restrict__ V, int64_t n, const KrylovCtl *__restrict__ ctl,
+                            const double *__restrict__ part, int np, int with_norm, int force,
+                            double *__restrict__ h, double *__restrict__ npart) {
+  pdl_enter();
+  const int2 it = ctl->cur;
+  if (it.y && !force) return;
+  __shared__ T hs[PSTR];
+  const int cnt = it.x + 1;
+  {  // the sums side by side: G = 2^lg lanes per coefficient
+    const int nh = cnt + with_norm;
+    int lg = 5;
+    while (lg > 0 && (nh << lg) > (int)blockDim.x) --lg;
+    const int G = 1 << lg, i = threadIdx.x >> lg, sub = threadIdx.x & (G - 1);
+    double s = 0.0;
+    if (i < nh) {
+#pragma unroll 4
+      for (int b = sub; b < np; b += G) s += part[(int64_t)b * PSTR + i];
+    }
+    for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (i < nh && sub == 0) {
+      hs[i] = (T)s;  // (converted once: a conversion costs as much as an FP64 FMA)
+      if (blockIdx.x == 0) h[i] = s;
+    }
+  }
+  __syncthreads();
+  T nacc = 0;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    T sv = w[k];
+#pragma unroll 16
+    for (int i = 0; i < cnt; ++i) sv -= hs[i] * V[(int64_t)i * n + k];
+    w[k] = sv;
+    nacc += sv * sv;
+  }
+  if (npart) {
+    const double sn = block_sum((double)nacc);
+    if (threadIdx.x == 0) npart[blockIdx.x] = sn;
+  }
+}
+
+// v = s w at node a into the basis vector, and its split
 template <int NB, typename T>
-void spmv(Ctx &c, const LinSys<T> &S, const T *x, T *y) {
+__device__ inline void scale_split(int64_t a, const T *__restrict__ w, T s, T *__restrict__ v, const SplitP<T> &P) {
+  constexpr int D = NB - 1;
+  T u[NB];
+#pragma unroll
+  for (int r = 0; r < NB; ++r) {
+    const T x = w[a * NB + r] * s;
+    v[a * NB + r] = x;
+    u[r] = x * P.dsi[a * NB + r];
+  }
+  if (P.lower) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      T t = 0;
+#pragma unroll
+      for (int k = 0; k < D; ++k) t = fma(P.dinv[a * D * D + i * D + k], u[k], t);
+      P.b0[a * D + i] = u[i];
+      P.x0[a * D + i] = P.omega * t;
+    }
+    P.other[a] = u[D];
+  } else {
+#pragma unroll
+    for (int k = 0; k < D; ++k) P.other[a * D + k] = u[k];
+    P.b0[a] = u[D];
+    P.x0[a] = P.omega * (P.dinv[a] * u[D]);
+  }
+}
+
+// Finish Arnoldi column j: |w| from the partials, H(:, j) = h1 (+ h2), the
+// previous Givens rotations and the new one (block 0), V_{j+1} = w / |w| with
+// its split; the residual estimate goes to est[j].  With h1 holding |w|^2 from
+// before the update at h1[j + 1] (theta > 0), a column that kept less than
+// theta of it halts for a second pass instead.  The square root and the
+// reciprocal are one thread's (as every thread's they would cost the SM's FP64
+// pipe microseconds).
+template <int NB, typename T>
+__global__ void k_gs_finish(const T *__restrict__ w, T *__restrict__ V, int64_t nnodes, int m, KrylovCtl *ctl,
+                            const double *__restrict__ npart, int np,
+                            const double *__restrict__ h1, const double *__restrict__ h2, double theta, int force,
+                            double *__restrict__ H, double *__restrict__ g, double *__restrict__ cs,
+                            double *__restrict__ sn, double *est, SplitP<T> P) {
+  pdl_enter();
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < np; b += blockDim.x) acc += npart[b];
+  const int2 it = ctl->cur;
+  if (it.y && !force) return;
+  __shared__ T sh_scale;
+  __shared__ int sh_again;
+  __shared__ double col[PSTR], sc[PSTR], ss[PSTR];
+  const int j = it.x;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+      col[i] = h1[i] + (h2 ? h2[i] : 0.0);
+      sc[i] = cs[i];
+      ss[i] = sn[i];
+    }
+  const double w0 = theta > 0.0 ? h1[j + 1] : 0.0;
+  acc = block_sum(acc);
+  double hn = 0.0;
+  if (threadIdx.x == 0) {
+    hn = sqrt(acc);
+    sh_again = theta > 0.0 && acc < theta * theta * w0;
+    sh_scale = (T)(hn > 0.0 ? 1.0 / hn : 0.0);
+  }
+  __syncthreads();
+  const bool again = sh_again != 0;
+  if (!again) {
+    const T s = sh_scale;
+    T *v = V + (int64_t)(j + 1) * (nnodes * NB);
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < nnodes; a += (int64_t)gridDim.x * blockDim.x)
+      scale_split<NB, T>(a, w, s, v, P);
+    if (blockIdx.x == 0) {
+      if (threadIdx.x == 0) {
+        double below = col[0];
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) {  // (one dependent FMA per rotation)
+          const double nx = col[i + 1];
+          col[i] = sc[i] * below + ss[i] * nx;
+          below = fma(-ss[i], below, sc[i] * nx);
+        }
+        double r = fma(below, below, hn * hn);
+        r = r > 1e-280 && r < 1e280 ? sqrt(r) : hypot(below, hn);
+        double c = 1.0, s2 = 0.0;
+        if (r > 0.0) {
+          c = below / r;
+          s2 = hn / r;
+        }
+        cs[j] = c;
+        sn[j] = s2;
+        col[j] = r;
+        const double gj = g[j];
+        g[j + 1] = -s2 * gj;
+        g[j] = c * gj;
+        slot_write(est + j, fabs(s2 * gj));
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i <= j; i += blockDim.x) H[i * m + j] = col[i];
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ctl->next = make_int2(again ? j : j + 1, again ? 1 : 0);
+    if (again) slot_write(est + j, EST_REORTH);
+  }
+}
+
+// V_0 = r / |r| with its split, |r|^2 from np partials; block 0 starts the
+// Givens right-hand side, the control word and posts |r|
+template <int NB, typename T>
+__global__ void k_gs_start(const T *__restrict__ r, T *__restrict__ V, int64_t nnodes, int m, KrylovCtl *ctl,
+                           const double *__restrict__ npart, int np, double *__restrict__ g, double *beta_slot,
+                           SplitP<T> P) {
+  __shared__ double sh_nrm;
+  __shared__ T sh_scale;
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < np; b += blockDim.x) acc += npart[b];
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) {
+    sh_nrm = sqrt(acc);
+    sh_scale = (T)(sh_nrm > 0.0 ? 1.0 / sh_nrm : 0.0);
+  }
+  __syncthreads();
+  const double beta = sh_nrm;
+  if (blockIdx.x == 0) {
+    for (int i = threadIdx.x; i <= m; i += blockDim.x) g[i] = i == 0 ? beta : 0.0;
+    if (threadIdx.x == 0) {
+      ctl->next = make_int2(0, 0);
+      slot_write(beta_slot, beta);
+    }
+  }
+  const T s = sh_scale;
+  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < nnodes; a += (int64_t)gridDim.x * blockDim.x)
+    scale_split<NB, T>(a, r, s, V, P);
+}
+
+// Z_j = D^-1 [zu; zp]
+template <int NB, typename T>
+__global__ void k_it_merge(int64_t nnodes, const T *__restrict__ zu, const T *__restrict__ zp,
+                           const T *__restrict__ dsi, T *__restrict__ Z, KrylovCtl *ctl) {
+  pdl_enter();
+  const int2 it = ctl->next;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cur = it;
+  if (it.y) return;
+  const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (a >= nnodes) return;
+  constexpr int D = NB - 1;
+  T *z = Z + (int64_t)it.x * (nnodes * NB);
+#pragma unroll
+  for (int k = 0; k < D; ++k) z[a * NB + k] = zu[a * D + k] * dsi[a * NB + k];
+  z[a * NB + D] = zp[a] * dsi[a * NB + D];
+}
+
+// x += Z y with H y = g solved by every block (jc x jc, back substitution by
+// columns; the triangle in shared memory when it fits, smem doubles)
+template <typename T>
+__global__ void k_solve_update_x(T *__restrict__ x, const T *__restrict__ Z, const double *__restrict__ H,
+                                 const double *__restrict__ g, int jc, int m, int64_t n, int in_smem) {
+  extern __shared__ __align__(16) unsigned char solve_smem[];
+  double *R = reinterpret_cast<double *>(solve_smem);
+  __shared__ double y[PSTR], rinv[PSTR];
+  if (in_smem)
+    for (int t = threadIdx.x; t < jc * jc; t += blockDim.x) R[t] = H[t / jc * m + t % jc];
+  for (int i = threadIdx.x; i < jc; i += blockDim.x) {
+    y[i] = g[i];
+    rinv[i] = 1.0 / H[i * m + i];
+  }
+  __syncthreads();
+  for (int i = jc - 1; i >= 0; --i) {
+    const double yi = y[i] * rinv[i];
+    __syncthreads();
+    for (int l = threadIdx.x; l < i; l += blockDim.x) y[l] -= (in_smem ? R[l * jc + i] : H[l * m + i]) * yi;
+    if (threadIdx.x == 0) y[i] = yi;
+    __syncthreads();
+  }
+  T *yt = reinterpret_cast<T *>(rinv);  // (no longer needed)
+  for (int i = threadIdx.x; i < jc; i += blockDim.x) yt[i] = (T)y[i];
+  __syncthreads();
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    T s = x[k];
+#pragma unroll 16
+    for (int i = 0; i < jc; ++i) s += yt[i] * Z[(int64_t)i * n + k];
+    x[k] = s;
+  }
+}
+
+template <int NB, typename T>
+void spmv(Ctx &c, const LinSys<T> &S, const T *x, T *y, const KrylovCtl *ctl = nullptr, int64_t xstride = 0) {
   constexpr int SPL = NB == 3 ? 2 : 4;  // 25 (2D) / 125 (3D) blocks per GIMP row
   const int64_t threads = c.g.nnodes * NB * SPL;
   prof_begin(c, MPM_PROF_SPMV);
   const int32_t *rp = c.row_ptr, *cl = c.col;
   const T *val = S.val;
-  launch_pdl(c, k_bsr_spmv<NB, SPL, T>, nblk(threads), TPB, 0, c.g.nnodes, rp, cl, val, x, y);
+  launch_pdl(c, k_bsr_spmv<NB, SPL, T>, nblk(threads), TPB, 0, c.g.nnodes, rp, cl, val, x, y, ctl, xstride);
   prof_end(c, MPM_PROF_SPMV);
 }
 
@@ -499,9 +798,191 @@ double read_scalar(Ctx &c, const double *dptr) {
   return c.h_scalar[0];
 }
 
+// Geometry of the Gram-Schmidt kernels of the iteration graph.
+struct GsGeom {
+  int64_t slice;
+  int ndot, ydot, nupd, nnode;
+};
+inline GsGeom gs_geom(const Ctx &c) {
+  const int64_t N = c.N();
+  GsGeom q;
+  q.slice = std::max<int64_t>(GS_SLICE, (N + NPART - 1) / NPART);
+  q.slice = (q.slice + 31) / 32 * 32;
+  q.ndot = (int)((N + q.slice - 1) / q.slice);
+  q.ydot = (c.m_restart + 1 + TPB / 32 - 1) / (TPB / 32);
+  q.nupd = std::min(NPART, nblk(N));
+  q.nnode = std::min(NPART, nblk(c.g.nnodes));
+  return q;
+}
+
+// The kernels of one iteration, from the preconditioner's core (its first
+// sub-solve's split is in place) to the split of the next basis vector.
+template <int NB, typename T>
+void enqueue_iteration(Ctx &c, LinSys<T> &S) {
+  const int64_t N = c.N(), nn = c.g.nnodes;
+  const GsGeom q = gs_geom(c);
+  const KrylovCtl *ctl = c.ctl;
+  double *h1 = c.hcol, *h2 = c.hcol + PSTR;
+  const SplitP<T> before = schur_split_args<T>(c, S);
+  const T *zu, *zp, *dsi = S.dscinv, *V = S.V, *w = S.w;
+  prof_begin(c, MPM_PROF_PRECOND);
+  schur_core_launch<T>(c, S, &zu, &zp);
+  launch_pdl(c, k_it_merge<NB, T>, nblk(nn), TPB, 0, nn, zu, zp, dsi, S.Z, c.ctl);
+  prof_end(c, MPM_PROF_PRECOND);
+  spmv<NB, T>(c, S, S.Z, S.w, ctl, N);
+  prof_begin(c, MPM_PROF_ORTH);
+  // FP64: one pass, |w|^2 beside the products for the test of the second;
+  // FP32: always two (one leaves the basis orthogonal to about 1e-6 only)
+  const bool sel = sizeof(T) == sizeof(double);
+  const double *part = c.part;
+  launch_pdl(c, k_gs_dots<T>, dim3(q.ndot, q.ydot), TPB, 0, V, w, N, q.slice, ctl, sel ? 1 : 0, 0, c.part);
+  launch_pdl(c, k_gs_update<T>, q.nupd, TPB, 0, S.w, V, N, ctl, part, q.ndot, sel ? 1 : 0, 0, h1,
+             sel ? c.npart : (double *)nullptr);
+  if (!sel) {
+    launch_pdl(c, k_gs_dots<T>, dim3(q.ndot, q.ydot), TPB, 0, V, w, N, q.slice, ctl, 0, 0, c.part);
+    launch_pdl(c, k_gs_update<T>, q.nupd, TPB, 0, S.w, V, N, ctl, part, q.ndot, 0, 0, h2, c.npart);
+  }
+  // the split goes where the next core reads it: a replayed graph's core is the
+  // one captured here, a directly launched one has swapped its buffers
+  const SplitP<T> next = c.capturing ? before : schur_split_args<T>(c, S);
+  launch_pdl(c, k_gs_finish<NB, T>, q.nnode, TPB, 0, w, S.V, nn, c.m_restart, c.ctl, (const double *)c.npart, q.nupd, (const double *)h1, sel ? (const double *)nullptr : (const double *)h2,
+             sel ? REORTH_THETA : 0.0, 0, c.H, c.gvec, c.cs, c.sn, c.d_slot, next);
+  prof_end(c, MPM_PROF_ORTH);
+}
+
+// The second Gram-Schmidt pass of the halted column and its finish (FP64).
+template <int NB, typename T>
+void enqueue_second_pass(Ctx &c, LinSys<T> &S, const SplitP<T> &next) {
+  const int64_t N = c.N(), nn = c.g.nnodes;
+  const GsGeom q = gs_geom(c);
+  double *h1 = c.hcol, *h2 = c.hcol + PSTR;
+  k_gs_dots<T><<<dim3(q.ndot, q.ydot), TPB, 0, c.st>>>(S.V, S.w, N, q.slice, c.ctl, 0, 1, c.part);
+  k_gs_update<T><<<q.nupd, TPB, 0, c.st>>>(S.w, S.V, N, c.ctl, c.part, q.ndot, 0, 1, h2, c.npart);
+  k_gs_finish<NB, T><<<q.nnode, TPB, 0, c.st>>>(S.w, S.V, nn, c.m_restart, c.ctl, c.npart, q.nupd,
+                                                h1, h2, 0.0, 1, c.H, c.gvec, c.cs, c.sn, c.d_slot, next);
+  c.launches += 3;
+}
+
+template <int NB, typename T>
+int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
+  const int64_t N = c.N(), nn = c.g.nnodes;
+  const int m = c.m_restart;
+  const GsGeom q = gs_geom(c);
+  const T *b = S.rhs;
+  T *x = S.x, *w = S.w;
+  // events around the classes of an iteration cannot be inside a graph
+  const int timed = (1 << MPM_PROF_SPMV) | (1 << MPM_PROF_ORTH) | (1 << MPM_PROF_PRECOND);
+  const bool graph = !(c.opt.profile & timed);
+  if (graph && (!S.itexec || S.itkey_col != c.col || S.itkey_val != S.val)) {
+    if (S.itexec) cudaGraphExecDestroy(S.itexec);
+    S.itexec = nullptr;
+    const int64_t before = c.launches;
+    const SplitP<T> sp = schur_split_args<T>(c, S);
+    cudaGraph_t gr = nullptr;
+    bool ok = cudaStreamBeginCapture(c.st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+      c.capturing = true;
+      enqueue_iteration<NB, T>(c, S);
+      c.capturing = false;
+      ok = cudaStreamEndCapture(c.st, &gr) == cudaSuccess && gr;
+    }
+    if (ok) ok = cudaGraphInstantiate(&S.itexec, gr, 0) == cudaSuccess;
+    if (gr) cudaGraphDestroy(gr);
+    S.itkernels = c.launches - before;
+    c.launches = before;
+    if (ok) {
+      S.it_x0 = sp.x0;
+      S.itkey_col = c.col;
+      S.itkey_val = S.val;
+    } else {  // capture unavailable: the kernels are launched directly
+      cudaGetLastError();
+      S.itexec = nullptr;
+    }
+  }
+  const bool use = graph && S.itexec;
+  auto split = [&]() {
+    SplitP<T> P = schur_split_args<T>(c, S);
+    if (use) P.x0 = S.it_x0;
+    return P;
+  };
+  auto launch = [&](int j) {
+    slot_reset(c, j);
+    if (use) {
+      cudaGraphLaunch(S.itexec, c.st);
+      c.launches += S.itkernels;
+    } else {
+      enqueue_iteration<NB, T>(c, S);
+    }
+  };
+  auto start = [&](const T *r, double *beta) {
+    slot_reset(c, SLOT_BETA);
+    k_dot_partial<T><<<q.nupd, TPB, 0, c.st>>>(r, r, N, c.npart);
+    k_gs_start<NB, T><<<q.nnode, TPB, 0, c.st>>>(r, S.V, nn, m, c.ctl, c.npart, q.nupd, c.gvec,
+                                                 c.d_slot + SLOT_BETA, split());
+    c.launches += 2;
+    return slot_wait(c, SLOT_BETA, beta);
+  };
+  cudaMemsetAsync(x, 0, sizeof(T) * N, c.st);
+  *iters = 0;
+  double beta0;
+  if (int rc = start(b, &beta0)) return rc;
+  if (!(beta0 > 0.0)) return MPM_OK;
+  if (!isfinite(beta0)) return MPM_ERR_NONFINITE;
+  const double target = rtol * beta0;
+  int total = 0;
+  bool converged = false;
+  double seen = beta0;  // the last estimate the host has read
+  while (true) {
+    int jc = 0, launched = 0;
+    for (int j = 0; j < m; ++j) {
+      if (launched <= j) launch(launched++);
+      if (launched == j + 1 && launched < m && total + 1 < maxit && seen > SPEC_MARGIN * target) launch(launched++);
+      double est;
+      if (int rc = slot_wait(c, j, &est)) return rc;
+      if (est == EST_REORTH) {  // what was launched ahead did nothing
+        slot_reset(c, j);
+        enqueue_second_pass<NB, T>(c, S, split());
+        launched = j + 1;
+        if (int rc = slot_wait(c, j, &est)) return rc;
+      }
+      ++total;
+      jc = j + 1;
+      *iters = total;
+      if (!isfinite(est)) return MPM_ERR_NONFINITE;
+      seen = est;
+      if (est <= target) {
+        converged = true;
+        break;
+      }
+      if (total >= maxit) break;
+    }
+    const int in_smem = jc * jc * (int)sizeof(double) <= 40 * 1024;
+    k_solve_update_x<T><<<q.nupd, TPB, in_smem ? sizeof(double) * jc * jc : 0, c.st>>>(x, S.Z, c.H, c.gvec, jc, m, N,
+                                                                                       in_smem);
+    UPMPM_LAUNCH(c);
+    if (converged || total >= maxit) break;
+    // restart from the true residual r = b - A x
+    spmv<NB, T>(c, S, x, w);
+    k_residual_vec<T><<<nblk(N), TPB, 0, c.st>>>(w, b, N);
+    UPMPM_LAUNCH(c);
+    double br;
+    if (int rc = start(w, &br)) return rc;
+    if (br <= target) {
+      converged = true;
+      break;
+    }
+    seen = br;
+  }
+  *iters = total;
+  if (check_cuda(c, cudaGetLastError(), "fgmres")) return MPM_ERR_CUDA;
+  return converged ? MPM_OK : MPM_ERR_KRYLOV_STAGNATED;
+}
+
 template <int NB, typename T>
 int fgmres_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
   const int64_t N = c.N();
+  if (c.opt.precond == MPM_PRECOND_SCHUR_MG && N < KRYLOV_GRAPH_MAX)
+    return fgmres_graph_impl<NB, T>(c, S, rtol, maxit, iters);
   const int m = c.m_restart;
   const int gN = nblk(N);
   const T *b = S.rhs;
@@ -763,16 +1244,35 @@ int64_t scan_exclusive(Ctx &c, const int32_t *in, int32_t *out, int64_t n) {
   }
   k_scan_blocks<<<nb, SCAN_T, 0, c.st>>>(in, out, n, c.scan_tmp);
   k_scan_top<<<1, SCAN_T, 0, c.st>>>(c.scan_tmp, nb);
-  k_scan_add<<<nb, SCAN_T, 0, c.st>>>(out, n, c.scan_tmp, in, c.scal + 4);
+  slot_reset(c, SLOT_SCAN);
+  k_scan_add<<<nb, SCAN_T, 0, c.st>>>(out, n, c.scan_tmp, in, c.d_slot + SLOT_SCAN);
   c.launches += 3;
-  return (int64_t)llround(read_scalar(c, c.scal + 4));
+  double total;
+  if (slot_wait(c, SLOT_SCAN, &total)) return -1;
+  return (int64_t)llround(total);
 }
 
-double run_norm(Ctx &c, const double *x) {
+int run_norm(Ctx &c, const double *x, double *norm) {
+  slot_reset(c, SLOT_NORM);
+  slot_reset(c, SLOT_ERR);
   k_dot_partial<double><<<NPART, TPB, 0, c.st>>>(x, x, c.N(), c.part);
-  k_reduce<<<1, TPB, 0, c.st>>>(c.part, NPART, c.scal + 3);
+  k_reduce_post<<<1, TPB, 0, c.st>>>(c.part, NPART, c.err, c.d_slot + SLOT_NORM, c.d_slot + SLOT_ERR);
   c.launches += 2;
-  return sqrt(read_scalar(c, c.scal + 3));
+  double n2, err;
+  int rc = slot_wait(c, SLOT_NORM, &n2);
+  if (!rc) rc = slot_wait(c, SLOT_ERR, &err);
+  if (!rc) rc = dev_err_code(c, (int)err);
+  *norm = sqrt(n2);
+  return rc;
+}
+
+int read_dev_err(Ctx &c) {
+  slot_reset(c, SLOT_WORD);
+  k_post_err<<<1, 1, 0, c.st>>>(c.err, c.d_slot + SLOT_WORD);
+  UPMPM_LAUNCH(c);
+  double err;
+  const int rc = slot_wait(c, SLOT_WORD, &err);
+  return rc ? rc : dev_err_code(c, (int)err);
 }
 
 template <typename T>
