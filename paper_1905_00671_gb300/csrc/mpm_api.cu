@@ -526,11 +526,10 @@ void free_all(Ctx &c) {
                   c.sh_S0, c.m, c.rec, c.pn, c.M, c.Pn, c.vn, c.an, c.pdn, c.pddn, c.phi, c.act, c.fsd, c.sh_nrm, c.fixed, c.u_fixed,
                   c.p_fixed, c.u_value, c.p_value, c.trac, c.trac_raw, c.flux, c.err, c.row_nnz,
                   c.row_ptr, c.row_of, c.col, c.row_mask, c.X, c.R, c.dX, c.stage, c.H, c.gvec,
-                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i};
+                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i, c.bk_post, c.bn_nodes, c.bn_s0, c.bn_slices, c.bn_part, c.bn_npart};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (c.h_inorm) cudaFreeHost(c.h_inorm);
-  if (c.h_bk) cudaFreeHost(c.h_bk);
   if (c.h_scalar) cudaFreeHost(c.h_scalar);
   if (c.h_terms) cudaFreeHost(c.h_terms);
   if (c.h_cmax) cudaFreeHost(c.h_cmax);
@@ -791,12 +790,16 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   A(&c.inst, c.ninst);
   A(&c.inorm, c.ninst);
   A(&c.node_inst, nn);
-  // batched FGMRES state: H ((m+1) m), g, cs, sn, y (m+1 each), h1, h2 (PSTR
-  // each), norm, scale, beta, target, residual per instance
-  A(&c.bk, (int64_t)c.ninst * ((int64_t)(m + 1) * m + 5 * (m + 1) + 2 * 129 + 5));
-  A(&c.bk_i, 2 * (int64_t)c.ninst + 1);
-  if (!rc && (cudaHostAlloc((void **)&c.h_inorm, sizeof(double) * c.ninst, cudaHostAllocDefault) != cudaSuccess ||
-              cudaHostAlloc((void **)&c.h_bk, sizeof(double) * 4, cudaHostAllocDefault) != cudaSuccess))
+  if (c.ninst > 1) {
+    // batched FGMRES state per instance: H ((m+1) m), g, cs, sn (m+1 each), h1,
+    // h2 (PSTR each), target, residual; the column it is frozen at, columns,
+    // second-pass mark
+    A(&c.bk, (int64_t)c.ninst * ((int64_t)(m + 1) * m + 3 * (m + 1) + 2 * 129 + 2));
+    A(&c.bk_i, 3 * (int64_t)c.ninst);
+    A(&c.bk_post, 1);
+    if (!rc) cudaMemset(c.bk_post, 0, sizeof(BatchPost));
+  }
+  if (!rc && cudaHostAlloc((void **)&c.h_inorm, sizeof(double) * c.ninst, cudaHostAllocDefault) != cudaSuccess)
     rc = MPM_ERR_NO_MEMORY;
   if (rc) {
     free_all(c);
@@ -815,6 +818,10 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
     }
     cudaMemcpyAsync(c.node_inst, ni.data(), sizeof(int32_t) * nn, cudaMemcpyHostToDevice, c.st);
     cudaStreamSynchronize(c.st);  // ni is a host temporary
+    if (c.ninst > 1 && (rc = batch_slices(c, ni))) {
+      free_all(c);
+      return create_abort(h, rc, "device memory allocation failed (node slices)");
+    }
   }
   cudaMemsetAsync(c.err, 0, sizeof(int), c.st);
   cudaMemsetAsync(c.row_nnz, 0, sizeof(int32_t) * (nn + 1), c.st);  // [nn] stays 0 for the scan

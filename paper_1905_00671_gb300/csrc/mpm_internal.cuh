@@ -89,6 +89,11 @@ struct SplitP {
 struct KrylovCtl {
   int2 cur, next;
 };
+// Reports of a batched iteration's instances (mpm_solver.cu).
+struct BatchPost {
+  unsigned arrived, active, again;
+  unsigned long long ratio;  // bits of the largest estimate / target
+};
 
 // 64-bit words of the per-node coupling mask of the block sparsity: bit
 // (o0 + 3) + 7 (o1 + 3) + 49 (o2 + 3) is set iff node a + o couples with a.
@@ -294,7 +299,13 @@ struct Ctx {
   // batched FGMRES: per-instance Krylov state (ninst x ...), see mpm_solver.cu
   double *bk = nullptr;                // one block of device doubles, carved below
   int32_t *bk_i = nullptr;             // per-instance flags / column counts
-  double *h_bk = nullptr;              // pinned: active-instance count
+  BatchPost *bk_post = nullptr;
+  // slices of the nodes by instance (bn_live of them), then of the nodes
+  // between instances (to bn_all); the instances' first slices; partial sums
+  int32_t *bn_nodes = nullptr, *bn_s0 = nullptr;
+  int4 *bn_slices = nullptr;
+  int bn_live = 0, bn_all = 0;
+  double *bn_part = nullptr, *bn_npart = nullptr;
   bool capturing = false;    // a CUDA graph capture is in progress on st
   int64_t n = 0;
   int32_t n_surf = 0;
@@ -453,6 +464,7 @@ int schur_setup(Ctx &c, LinSys<T> &S, bool coarse = true);  // before run_scale_
                                                              // coarse = false: the finest levels only
 template <typename T>
 void schur_apply(Ctx &c, LinSys<T> &S, const T *v, T *z);  // z = M^{-1} v
+int batch_slices(Ctx &c, const std::vector<int32_t> &node_inst);  // bn_* of a batched context
 // its parts, for a caller that captures them: the split's buffers as they are
 // before the core, and the core (results in *zu, *zp)
 template <typename T>

@@ -13,6 +13,9 @@
 // the FP64 block sum.  No tensor cores: the work is sparse.
 #include <math.h>
 
+#include <algorithm>
+#include <vector>
+
 #include "mpm_internal.cuh"
 
 namespace upmpm {
@@ -493,7 +496,7 @@ __global__ void k_update_x(T *__restrict__ x, const T *__restrict__ Z, const dou
 }
 
 // ------------------------------------- one iteration as a CUDA graph
-// Below KRYLOV_GRAPH_MAX unknowns an FGMRES iteration is a chain of kernels of
+// Below KRYLOV_GRAPH_MAX unknowns (and for batched contexts) an FGMRES iteration is a chain of kernels of
 // a few microseconds, and what it costs is their number, their launches and the
 // host's read of the residual estimate.  So the whole iteration is one graph:
 // its kernels read the iteration's number from a control word; the reductions
@@ -586,16 +589,17 @@ __global__ void k_gs_update(T *__restrict__ w, const T *__restrict__ V, int64_t 
 }
 
 // v = s w at node a into the basis vector, and its split
-template <int NB, typename T>
-__device__ inline void scale_split(int64_t a, const T *__restrict__ w, T s, T *__restrict__ v, const SplitP<T> &P) {
+template <int NB, typename T, typename Q>
+__device__ inline void scale_split(int64_t a, const T *__restrict__ w, Q s, T *__restrict__ v, const SplitP<T> &P) {
   constexpr int D = NB - 1;
   T u[NB];
 #pragma unroll
   for (int r = 0; r < NB; ++r) {
-    const T x = w[a * NB + r] * s;
+    const T x = (T)(w[a * NB + r] * s);
     v[a * NB + r] = x;
-    u[r] = x * P.dsi[a * NB + r];
+    u[r] = P.dsi ? x * P.dsi[a * NB + r] : x;
   }
+  if (!P.dsi) return;  // no split: block-Jacobi preconditioner
   if (P.lower) {
 #pragma unroll
     for (int i = 0; i < D; ++i) {
@@ -656,7 +660,7 @@ __global__ void k_gs_finish(const T *__restrict__ w, T *__restrict__ V, int64_t 
     const T s = sh_scale;
     T *v = V + (int64_t)(j + 1) * (nnodes * NB);
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < nnodes; a += (int64_t)gridDim.x * blockDim.x)
-      scale_split<NB, T>(a, w, s, v, P);
+      scale_split<NB>(a, w, s, v, P);
     if (blockIdx.x == 0) {
       if (threadIdx.x == 0) {
         double below = col[0];
@@ -717,7 +721,7 @@ __global__ void k_gs_start(const T *__restrict__ r, T *__restrict__ V, int64_t n
   }
   const T s = sh_scale;
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < nnodes; a += (int64_t)gridDim.x * blockDim.x)
-    scale_split<NB, T>(a, r, s, V, P);
+    scale_split<NB>(a, r, s, V, P);
 }
 
 // Z_j = D^-1 [zu; zp]
@@ -735,6 +739,27 @@ __global__ void k_it_merge(int64_t nnodes, const T *__restrict__ zu, const T *__
 #pragma unroll
   for (int k = 0; k < D; ++k) z[a * NB + k] = zu[a * D + k] * dsi[a * NB + k];
   z[a * NB + D] = zp[a] * dsi[a * NB + D];
+}
+
+// Z_j = Dinv V_j (node-block Jacobi)
+template <int NB, typename T>
+__global__ void k_it_bj(int64_t nnodes, const T *__restrict__ dinv, const T *__restrict__ V, T *__restrict__ Z,
+                        KrylovCtl *ctl) {
+  pdl_enter();
+  const int2 it = ctl->next;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cur = it;
+  if (it.y) return;
+  const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (a >= nnodes) return;
+  const T *x = V + (int64_t)it.x * (nnodes * NB);
+  T *z = Z + (int64_t)it.x * (nnodes * NB);
+  T xv[NB];
+  for (int j = 0; j < NB; ++j) xv[j] = x[a * NB + j];
+  for (int i = 0; i < NB; ++i) {
+    T s = 0;
+    for (int j = 0; j < NB; ++j) s += dinv[a * NB * NB + i * NB + j] * xv[j];
+    z[a * NB + i] = s;
+  }
 }
 
 // x += Z y with H y = g solved by every block (jc x jc, back substitution by
@@ -798,6 +823,322 @@ double read_scalar(Ctx &c, const double *dptr) {
   return c.h_scalar[0];
 }
 
+// ------------------------------------------------ batched FGMRES (instances)
+// A batched context solves one block-diagonal system (the instances never
+// couple; the preconditioner keeps that structure), so FGMRES runs per
+// instance: every inner product, Hessenberg column, Givens rotation and
+// convergence test is the instance's own, while each kernel serves all
+// instances at once.  An instance that meets its tolerance in column j is
+// frozen from column j + 1 on (its Krylov vectors are zero from then) until
+// the others finish.
+// The vectors are walked in slices of up to BG_NODES nodes of one instance
+// (Ctx::bn_*; the nodes between instances form slices of their own, kept at
+// zero): a block per slice and group of products forms partial sums, and every
+// block that needs an instance's sum adds its slices.  (One block per instance
+// and product, walking the instance's node box, took 33 us a pass on 64 columns
+// of 4,200 nodes and three passes an iteration.)  The iteration is a graph, as
+// for one instance; frozen_at holds the first column an instance skips, so that
+// the blocks of an instance agree on it while its first block moves it on.
+// Measured (GB300, 64 instances, whole steps): columns 74.8 -> 56.4 ms (95
+// iterations), footings 140 -> 120 ms (125); the Gram-Schmidt kernels then run at
+// the FP64 rate of their products.
+constexpr int BG_NODES = 256;
+
+struct BatchK {  // device pointers of the batched solve, by value
+  int ni, m;
+  const int32_t *nodes, *s0;  // node lists by slice; first slice of every instance (ni + 1)
+  const int4 *slices;         // (instance or -1, start in nodes, count, -)
+  double *H, *g, *cs, *sn, *h1, *h2, *tgt, *res;
+  int32_t *frozen_at, *jc, *again;
+  double *part, *npart;
+  BatchPost *post;
+  KrylovCtl *ctl;
+  double *slot;
+};
+
+// sum of p over the slices of instance i, in thread 0 (block-wide)
+__device__ inline double slices_sum(const BatchK &K, int i, const double *__restrict__ p) {
+  double acc = 0.0;
+  for (int b = K.s0[i] + threadIdx.x; b < K.s0[i + 1]; b += blockDim.x) acc += p[b];
+  return block_sum(acc);
+}
+
+// An instance's first block reports (thread 0): whether it goes on, how far its
+// estimate is from its target, whether it needs a second pass; the last report
+// of the kernel posts the largest ratio (0: all done) and moves the control word
+__device__ inline void batch_report(const BatchK &K, int j, double *slot, bool active, double ratio, bool again) {
+  BatchPost *q = K.post;
+  if (active) {
+    atomicAdd(&q->active, 1u);
+    atomicMax(&q->ratio, (unsigned long long)__double_as_longlong(ratio));
+  }
+  if (again) atomicAdd(&q->again, 1u);
+  __threadfence();
+  if (atomicAdd(&q->arrived, 1u) != (unsigned)K.ni - 1) return;
+  __threadfence();
+  const unsigned act = atomicAdd(&q->active, 0u), ag = atomicAdd(&q->again, 0u);
+  const double worst = __longlong_as_double((long long)atomicMax(&q->ratio, 0ull));
+  q->active = q->again = q->arrived = 0;
+  q->ratio = 0;
+  K.ctl->next = make_int2(ag ? j : j + 1, ag ? 1 : 0);
+  slot_write(slot, ag ? EST_REORTH : (act ? worst : 0.0));
+}
+
+template <int NB, typename T>
+__global__ void k_bgs_norm(BatchK K, const T *__restrict__ r) {
+  const int4 sl = K.slices[blockIdx.x];
+  double acc = 0.0;
+  if ((int)threadIdx.x < sl.z) {
+    const int64_t a = K.nodes[sl.y + threadIdx.x];
+    for (int c = 0; c < NB; ++c) acc += (double)r[a * NB + c] * (double)r[a * NB + c];
+  }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) K.npart[blockIdx.x] = acc;
+}
+
+// start of a cycle: V_0 = r / |r| with its split, g = |r| e_1 per instance; the
+// tolerance rtol |r| is fixed at the first start; an instance within it is done
+template <int NB, typename T>
+__global__ void k_bgs_start(BatchK K, const T *__restrict__ r, T *__restrict__ V, double rtol, int set_target,
+                            SplitP<T> P) {
+  const int4 sl = K.slices[blockIdx.x];
+  const int i = sl.x;
+  __shared__ double sh_scale;
+  if (threadIdx.x == 0) sh_scale = 0.0;
+  if (i >= 0) {
+    const double n2 = slices_sum(K, i, K.npart);
+    if (threadIdx.x == 0) {
+      const double beta = sqrt(n2), tgt = set_target ? rtol * beta : K.tgt[i];
+      const bool done = !(beta > tgt);
+      sh_scale = !done && beta > 0.0 ? 1.0 / beta : 0.0;
+      if ((int)blockIdx.x == K.s0[i]) {
+        if (set_target) K.tgt[i] = tgt;
+        double *g = K.g + (int64_t)i * (K.m + 1);
+        for (int k = 1; k <= K.m; ++k) g[k] = 0.0;
+        g[0] = beta;
+        K.jc[i] = 0;
+        K.frozen_at[i] = done ? 0 : 0x7fffffff;
+        batch_report(K, -1, K.slot + SLOT_BETA, !done, beta / tgt, false);
+      }
+    }
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < sl.z) scale_split<NB>(K.nodes[sl.y + threadIdx.x], r, sh_scale, V, P);
+}
+
+// products of a slice, a warp each; summed in FP64
+template <int NB, typename T>
+__global__ void k_bgs_dots(BatchK K, const T *__restrict__ V, const T *__restrict__ w, int64_t n, int with_norm,
+                           int force) {
+  pdl_enter();
+  const int2 it = K.ctl->cur;
+  const int cnt = it.x + 1, lane = threadIdx.x & 31;
+  const int k = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (k >= cnt + with_norm || (it.y && !force)) return;
+  const int4 sl = K.slices[blockIdx.x];
+  if (K.frozen_at[sl.x] <= it.x || (force && !K.again[sl.x])) return;
+  const T *vk = k < cnt ? V + (int64_t)k * n : w;
+  double s = 0.0;
+#pragma unroll 4
+  for (int e = lane; e < sl.z; e += 32) {
+    const int64_t a = K.nodes[sl.y + e];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) s += (double)vk[a * NB + c] * (double)w[a * NB + c];
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) K.part[(int64_t)blockIdx.x * PSTR + k] = s;
+}
+
+// w -= sum_k h_k V_k on a slice, h its instance's sums over the slices (kept in
+// h by the instance's first block); npart: the slice's squared norm after
+template <int NB, typename T>
+__global__ void k_bgs_update(BatchK K, T *__restrict__ w, const T *__restrict__ V, int64_t n, int with_norm,
+                             int force, double *__restrict__ h, int want_norm) {
+  pdl_enter();
+  const int2 it = K.ctl->cur;
+  if (it.y && !force) return;
+  const int4 sl = K.slices[blockIdx.x];
+  const int i = sl.x, cnt = it.x + 1;
+  if (K.frozen_at[i] <= it.x || (force && !K.again[i])) return;
+  __shared__ T hs[PSTR];
+  {
+    const int nh = cnt + with_norm, b1 = K.s0[i + 1];
+    int lg = 5;
+    while (lg > 0 && (nh << lg) > (int)blockDim.x) --lg;
+    const int G = 1 << lg, k = threadIdx.x >> lg, sub = threadIdx.x & (G - 1);
+    double s = 0.0;
+    if (k < nh) {
+#pragma unroll 4
+      for (int b = K.s0[i] + sub; b < b1; b += G) s += K.part[(int64_t)b * PSTR + k];
+    }
+    for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (k < nh && sub == 0) {
+      hs[k] = (T)s;
+      if ((int)blockIdx.x == K.s0[i]) h[(int64_t)i * PSTR + k] = s;
+    }
+  }
+  __syncthreads();
+  double nacc = 0.0;
+  if ((int)threadIdx.x < sl.z) {
+    const int64_t a = (int64_t)K.nodes[sl.y + threadIdx.x] * NB;
+    T x[NB];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) x[c] = w[a + c];
+#pragma unroll 8
+    for (int k = 0; k < cnt; ++k)
+#pragma unroll
+      for (int c = 0; c < NB; ++c) x[c] -= hs[k] * V[(int64_t)k * n + a + c];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      w[a + c] = x[c];
+      nacc += (double)x[c] * (double)x[c];
+    }
+  }
+  if (want_norm) {
+    nacc = block_sum(nacc);
+    if (threadIdx.x == 0) K.npart[blockIdx.x] = nacc;
+  }
+}
+
+// Arnoldi column j of every active instance (its first block): H(:, j) = h1
+// (+ h2), the rotations, g, the estimate; V_{j+1} = w / |w| with its split (all
+// blocks), zero for a frozen instance and between instances.  theta as in
+// k_gs_finish, per instance: one that needs a second pass is marked in again
+// and finished by the forced call after it.
+template <int NB, typename T>
+__global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ V, int64_t n, double theta,
+                             int force, int two, SplitP<T> P) {
+  pdl_enter();
+  const int2 it = K.ctl->cur;
+  if (it.y && !force) return;
+  const int j = it.x;
+  const int4 sl = K.slices[blockIdx.x];
+  const int i = sl.x;
+  const bool lead = i >= 0 && (int)blockIdx.x == K.s0[i];
+  const bool live = i >= 0 && K.frozen_at[i] > j && (!force || K.again[i]);
+  __shared__ double sh_scale;
+  __shared__ int sh_skip;
+  __shared__ double col[PSTR], sc[PSTR], ss[PSTR];
+  double n2 = 0.0;
+  if (live) {
+    if (lead)
+      for (int k = threadIdx.x; k <= j; k += blockDim.x) {
+        const int64_t hk = (int64_t)i * PSTR + k, rk = (int64_t)i * (K.m + 1) + k;
+        col[k] = K.h1[hk] + (two ? K.h2[hk] : 0.0);
+        sc[k] = K.cs[rk];
+        ss[k] = K.sn[rk];
+      }
+    n2 = slices_sum(K, i, K.npart);
+  }
+  if (threadIdx.x == 0) {
+    sh_scale = 0.0;
+    sh_skip = i >= 0 && force && !live;  // its vector is in place from the first pass
+    double hn = 0.0;
+    bool again = false;
+    if (live) {
+      hn = sqrt(n2);
+      sh_scale = hn > 0.0 ? 1.0 / hn : 0.0;
+      again = theta > 0.0 && n2 < theta * theta * K.h1[(int64_t)i * PSTR + j + 1];
+      if (again) sh_skip = 1;
+    }
+    if (lead) {
+      if (!force) K.again[i] = again ? 1 : 0;
+      if (live && !again) {
+        double *g = K.g + (int64_t)i * (K.m + 1), *H = K.H + (int64_t)i * (K.m + 1) * K.m;
+        double below = col[0];
+#pragma unroll 4
+        for (int k = 0; k < j; ++k) {
+          const double nx = col[k + 1];
+          H[k * K.m + j] = sc[k] * below + ss[k] * nx;
+          below = fma(-ss[k], below, sc[k] * nx);
+        }
+        const double r = hypot(below, hn);
+        double c = 1.0, sv = 0.0;
+        if (r > 0.0) {
+          c = below / r;
+          sv = hn / r;
+        }
+        K.cs[(int64_t)i * (K.m + 1) + j] = c;
+        K.sn[(int64_t)i * (K.m + 1) + j] = sv;
+        H[j * K.m + j] = r;
+        const double gj = g[j], res = fabs(sv * gj);
+        g[j + 1] = -sv * gj;
+        g[j] = c * gj;
+        K.res[i] = res;
+        K.jc[i] = j + 1;
+        if (res <= K.tgt[i] || !(hn > 0.0)) K.frozen_at[i] = j + 1;
+      }
+      const bool on = K.frozen_at[i] > j + 1;
+      batch_report(K, j, K.slot + j, on, on ? K.res[i] / K.tgt[i] : 0.0, again);
+    }
+  }
+  __syncthreads();
+  if (sh_skip) return;
+  if ((int)threadIdx.x < sl.z)
+    scale_split<NB>(K.nodes[sl.y + threadIdx.x], w, sh_scale, V + (int64_t)(j + 1) * n, P);
+}
+
+// x += Z y per slice, its instance's triangle solved by every block
+template <int NB, typename T>
+__global__ void k_bgs_solve_x(BatchK K, T *__restrict__ x, const T *__restrict__ Z, int64_t n) {
+  const int4 sl = K.slices[blockIdx.x];
+  const int i = sl.x, jc = K.jc[i];
+  const double *H = K.H + (int64_t)i * (K.m + 1) * K.m, *g = K.g + (int64_t)i * (K.m + 1);
+  __shared__ double y[PSTR], rinv[PSTR];
+  __shared__ T yt[PSTR];
+  for (int k = threadIdx.x; k < jc; k += blockDim.x) {
+    const double d = H[k * K.m + k];
+    y[k] = g[k];
+    rinv[k] = d != 0.0 ? 1.0 / d : 0.0;
+  }
+  __syncthreads();
+  for (int k = jc - 1; k >= 0; --k) {
+    const double yk = y[k] * rinv[k];
+    __syncthreads();
+    for (int l = threadIdx.x; l < k; l += blockDim.x) y[l] -= H[l * K.m + k] * yk;
+    if (threadIdx.x == 0) yt[k] = (T)yk;
+    __syncthreads();
+  }
+  if ((int)threadIdx.x >= sl.z) return;
+  const int64_t a = (int64_t)K.nodes[sl.y + threadIdx.x] * NB;
+  T s[NB];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) s[c] = x[a + c];
+#pragma unroll 8
+  for (int k = 0; k < jc; ++k)
+#pragma unroll
+    for (int c = 0; c < NB; ++c) s[c] += yt[k] * Z[(int64_t)k * n + a + c];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) x[a + c] = s[c];
+}
+
+inline BatchK batch_k(const Ctx &c) {
+  const int64_t ni = c.ninst, m = c.m_restart;
+  BatchK K{};
+  K.ni = c.ninst;
+  K.m = c.m_restart;
+  K.nodes = c.bn_nodes;
+  K.s0 = c.bn_s0;
+  K.slices = c.bn_slices;
+  K.H = c.bk;
+  K.g = K.H + ni * (m + 1) * m;
+  K.cs = K.g + ni * (m + 1);
+  K.sn = K.cs + ni * (m + 1);
+  K.h1 = K.sn + ni * (m + 1);
+  K.h2 = K.h1 + ni * PSTR;
+  K.tgt = K.h2 + ni * PSTR;
+  K.res = K.tgt + ni;
+  K.frozen_at = c.bk_i;
+  K.jc = c.bk_i + ni;
+  K.again = c.bk_i + 2 * ni;
+  K.part = c.bn_part;
+  K.npart = c.bn_npart;
+  K.post = c.bk_post;
+  K.ctl = c.ctl;
+  K.slot = c.d_slot;
+  return K;
+}
+
 // Geometry of the Gram-Schmidt kernels of the iteration graph.
 struct GsGeom {
   int64_t slice;
@@ -815,6 +1156,11 @@ inline GsGeom gs_geom(const Ctx &c) {
   return q;
 }
 
+template <typename T>
+SplitP<T> next_split(Ctx &c, LinSys<T> &S) {
+  return c.opt.precond == MPM_PRECOND_SCHUR_MG ? schur_split_args<T>(c, S) : SplitP<T>{};
+}
+
 // The kernels of one iteration, from the preconditioner's core (its first
 // sub-solve's split is in place) to the split of the next basis vector.
 template <int NB, typename T>
@@ -823,11 +1169,15 @@ void enqueue_iteration(Ctx &c, LinSys<T> &S) {
   const GsGeom q = gs_geom(c);
   const KrylovCtl *ctl = c.ctl;
   double *h1 = c.hcol, *h2 = c.hcol + PSTR;
-  const SplitP<T> before = schur_split_args<T>(c, S);
+  const SplitP<T> before = next_split<T>(c, S);
   const T *zu, *zp, *dsi = S.dscinv, *V = S.V, *w = S.w;
   prof_begin(c, MPM_PROF_PRECOND);
-  schur_core_launch<T>(c, S, &zu, &zp);
-  launch_pdl(c, k_it_merge<NB, T>, nblk(nn), TPB, 0, nn, zu, zp, dsi, S.Z, c.ctl);
+  if (c.opt.precond == MPM_PRECOND_SCHUR_MG) {
+    schur_core_launch<T>(c, S, &zu, &zp);
+    launch_pdl(c, k_it_merge<NB, T>, nblk(nn), TPB, 0, nn, zu, zp, dsi, S.Z, c.ctl);
+  } else {
+    launch_pdl(c, k_it_bj<NB, T>, nblk(nn), TPB, 0, nn, (const T *)S.dinv, V, S.Z, c.ctl);
+  }
   prof_end(c, MPM_PROF_PRECOND);
   spmv<NB, T>(c, S, S.Z, S.w, ctl, N);
   prof_begin(c, MPM_PROF_ORTH);
@@ -835,6 +1185,22 @@ void enqueue_iteration(Ctx &c, LinSys<T> &S) {
   // FP32: always two (one leaves the basis orthogonal to about 1e-6 only)
   const bool sel = sizeof(T) == sizeof(double);
   const double *part = c.part;
+  // the split goes where the next core reads it: a replayed graph's core is the
+  // one captured here, a directly launched one has swapped its buffers
+  const SplitP<T> next = c.capturing ? before : next_split<T>(c, S);
+  if (c.ninst > 1) {
+    const BatchK K = batch_k(c);
+    launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N, sel ? 1 : 0, 0);
+    launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, sel ? 1 : 0, 0, K.h1, sel ? 1 : 0);
+    if (!sel) {
+      launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N, 0, 0);
+      launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, 0, 0, K.h2, 1);
+    }
+    launch_pdl(c, k_bgs_finish<NB, T>, c.bn_all, BG_NODES, 0, K, w, S.V, N, sel ? REORTH_THETA : 0.0, 0,
+               sel ? 0 : 1, next);
+    prof_end(c, MPM_PROF_ORTH);
+    return;
+  }
   launch_pdl(c, k_gs_dots<T>, dim3(q.ndot, q.ydot), TPB, 0, V, w, N, q.slice, ctl, sel ? 1 : 0, 0, c.part);
   launch_pdl(c, k_gs_update<T>, q.nupd, TPB, 0, S.w, V, N, ctl, part, q.ndot, sel ? 1 : 0, 0, h1,
              sel ? c.npart : (double *)nullptr);
@@ -842,10 +1208,8 @@ void enqueue_iteration(Ctx &c, LinSys<T> &S) {
     launch_pdl(c, k_gs_dots<T>, dim3(q.ndot, q.ydot), TPB, 0, V, w, N, q.slice, ctl, 0, 0, c.part);
     launch_pdl(c, k_gs_update<T>, q.nupd, TPB, 0, S.w, V, N, ctl, part, q.ndot, 0, 0, h2, c.npart);
   }
-  // the split goes where the next core reads it: a replayed graph's core is the
-  // one captured here, a directly launched one has swapped its buffers
-  const SplitP<T> next = c.capturing ? before : schur_split_args<T>(c, S);
-  launch_pdl(c, k_gs_finish<NB, T>, q.nnode, TPB, 0, w, S.V, nn, c.m_restart, c.ctl, (const double *)c.npart, q.nupd, (const double *)h1, sel ? (const double *)nullptr : (const double *)h2,
+  launch_pdl(c, k_gs_finish<NB, T>, q.nnode, TPB, 0, w, S.V, nn, c.m_restart, c.ctl, (const double *)c.npart,
+             q.nupd, (const double *)h1, sel ? (const double *)nullptr : (const double *)h2,
              sel ? REORTH_THETA : 0.0, 0, c.H, c.gvec, c.cs, c.sn, c.d_slot, next);
   prof_end(c, MPM_PROF_ORTH);
 }
@@ -856,11 +1220,18 @@ void enqueue_second_pass(Ctx &c, LinSys<T> &S, const SplitP<T> &next) {
   const int64_t N = c.N(), nn = c.g.nnodes;
   const GsGeom q = gs_geom(c);
   double *h1 = c.hcol, *h2 = c.hcol + PSTR;
+  c.launches += 3;
+  if (c.ninst > 1) {
+    const BatchK K = batch_k(c);
+    k_bgs_dots<NB, T><<<dim3(c.bn_live, q.ydot), TPB, 0, c.st>>>(K, S.V, S.w, N, 0, 1);
+    k_bgs_update<NB, T><<<c.bn_live, BG_NODES, 0, c.st>>>(K, S.w, S.V, N, 0, 1, K.h2, 1);
+    k_bgs_finish<NB, T><<<c.bn_all, BG_NODES, 0, c.st>>>(K, S.w, S.V, N, 0.0, 1, 1, next);
+    return;
+  }
   k_gs_dots<T><<<dim3(q.ndot, q.ydot), TPB, 0, c.st>>>(S.V, S.w, N, q.slice, c.ctl, 0, 1, c.part);
   k_gs_update<T><<<q.nupd, TPB, 0, c.st>>>(S.w, S.V, N, c.ctl, c.part, q.ndot, 0, 1, h2, c.npart);
-  k_gs_finish<NB, T><<<q.nnode, TPB, 0, c.st>>>(S.w, S.V, nn, c.m_restart, c.ctl, c.npart, q.nupd,
-                                                h1, h2, 0.0, 1, c.H, c.gvec, c.cs, c.sn, c.d_slot, next);
-  c.launches += 3;
+  k_gs_finish<NB, T><<<q.nnode, TPB, 0, c.st>>>(S.w, S.V, nn, c.m_restart, c.ctl, c.npart, q.nupd, h1, h2, 0.0, 1,
+                                                c.H, c.gvec, c.cs, c.sn, c.d_slot, next);
 }
 
 template <int NB, typename T>
@@ -877,7 +1248,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
     if (S.itexec) cudaGraphExecDestroy(S.itexec);
     S.itexec = nullptr;
     const int64_t before = c.launches;
-    const SplitP<T> sp = schur_split_args<T>(c, S);
+    const SplitP<T> sp = next_split<T>(c, S);
     cudaGraph_t gr = nullptr;
     bool ok = cudaStreamBeginCapture(c.st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
@@ -901,7 +1272,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
   }
   const bool use = graph && S.itexec;
   auto split = [&]() {
-    SplitP<T> P = schur_split_args<T>(c, S);
+    SplitP<T> P = next_split<T>(c, S);
     if (use) P.x0 = S.it_x0;
     return P;
   };
@@ -914,8 +1285,18 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
       enqueue_iteration<NB, T>(c, S);
     }
   };
-  auto start = [&](const T *r, double *beta) {
+  // the first start's norm and target: of the system, or (batched) the largest
+  // ratio of an instance's norm to its target against 1 (0: nothing to do)
+  const bool batch = c.ninst > 1;
+  auto start = [&](const T *r, double *beta, int first) {
     slot_reset(c, SLOT_BETA);
+    if (batch) {
+      const BatchK K = batch_k(c);
+      k_bgs_norm<NB, T><<<c.bn_live, BG_NODES, 0, c.st>>>(K, r);
+      k_bgs_start<NB, T><<<c.bn_all, BG_NODES, 0, c.st>>>(K, r, S.V, rtol, first, split());
+      c.launches += 2;
+      return slot_wait(c, SLOT_BETA, beta);
+    }
     k_dot_partial<T><<<q.nupd, TPB, 0, c.st>>>(r, r, N, c.npart);
     k_gs_start<NB, T><<<q.nnode, TPB, 0, c.st>>>(r, S.V, nn, m, c.ctl, c.npart, q.nupd, c.gvec,
                                                  c.d_slot + SLOT_BETA, split());
@@ -925,10 +1306,10 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
   cudaMemsetAsync(x, 0, sizeof(T) * N, c.st);
   *iters = 0;
   double beta0;
-  if (int rc = start(b, &beta0)) return rc;
+  if (int rc = start(b, &beta0, 1)) return rc;
   if (!(beta0 > 0.0)) return MPM_OK;
   if (!isfinite(beta0)) return MPM_ERR_NONFINITE;
-  const double target = rtol * beta0;
+  const double target = batch ? 0.5 : rtol * beta0;  // (a batch posts 0 or a ratio above 1)
   int total = 0;
   bool converged = false;
   double seen = beta0;  // the last estimate the host has read
@@ -956,9 +1337,13 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
       }
       if (total >= maxit) break;
     }
-    const int in_smem = jc * jc * (int)sizeof(double) <= 40 * 1024;
-    k_solve_update_x<T><<<q.nupd, TPB, in_smem ? sizeof(double) * jc * jc : 0, c.st>>>(x, S.Z, c.H, c.gvec, jc, m, N,
-                                                                                       in_smem);
+    if (batch) {
+      k_bgs_solve_x<NB, T><<<c.bn_live, BG_NODES, 0, c.st>>>(batch_k(c), x, S.Z, N);
+    } else {
+      const int in_smem = jc * jc * (int)sizeof(double) <= 40 * 1024;
+      k_solve_update_x<T><<<q.nupd, TPB, in_smem ? sizeof(double) * jc * jc : 0, c.st>>>(x, S.Z, c.H, c.gvec, jc, m, N,
+                                                                                         in_smem);
+    }
     UPMPM_LAUNCH(c);
     if (converged || total >= maxit) break;
     // restart from the true residual r = b - A x
@@ -966,7 +1351,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
     k_residual_vec<T><<<nblk(N), TPB, 0, c.st>>>(w, b, N);
     UPMPM_LAUNCH(c);
     double br;
-    if (int rc = start(w, &br)) return rc;
+    if (int rc = start(w, &br, 0)) return rc;
     if (br <= target) {
       converged = true;
       break;
@@ -981,7 +1366,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
 template <int NB, typename T>
 int fgmres_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
   const int64_t N = c.N();
-  if (c.opt.precond == MPM_PRECOND_SCHUR_MG && N < KRYLOV_GRAPH_MAX)
+  if (c.ninst > 1 || N < KRYLOV_GRAPH_MAX)
     return fgmres_graph_impl<NB, T>(c, S, rtol, maxit, iters);
   const int m = c.m_restart;
   const int gN = nblk(N);
@@ -1076,157 +1461,6 @@ int fgmres_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
   return converged ? MPM_OK : MPM_ERR_KRYLOV_STAGNATED;
 }
 
-// ------------------------------------------------ batched FGMRES (instances)
-// A batched context solves one block-diagonal system (the instances never
-// couple; the preconditioner keeps that structure), so FGMRES runs per
-// instance: every inner product, Hessenberg column, Givens rotation and
-// convergence test is the instance's own, while each kernel serves all
-// instances at once.  An instance that meets its tolerance is frozen (its next
-// Krylov vectors are zero) until the others finish.
-
-// out[i * ostride + k] = sum over the DOFs of instance i of V_k . w, k < cnt;
-// block (i, k) walks instance i's node box in a fixed order
-template <typename T>
-__global__ void k_inst_dots(GridP g, int nb, const InstDev *__restrict__ inst, const T *__restrict__ V,
-                            int64_t vstride, const T *__restrict__ w, double *__restrict__ out, int ostride) {
-  pdl_enter();
-  const InstDev I = inst[blockIdx.x];
-  const int k = blockIdx.y;
-  const T *Vk = V + (int64_t)k * vstride;
-  const int64_t m0 = I.nc[0] + 1, m1 = g.d > 1 ? I.nc[1] + 1 : 1, m2 = g.d > 2 ? I.nc[2] + 1 : 1;
-  double acc = 0.0;
-  for (int64_t t = threadIdx.x; t < m0 * m1 * m2; t += blockDim.x) {
-    const int64_t i0 = t % m0, i1 = (t / m0) % m1, i2 = t / (m0 * m1);
-    const int64_t a = (i0 + I.off[0]) + (int64_t)g.nn[0] * ((i1 + I.off[1]) + (int64_t)g.nn[1] * (i2 + I.off[2]));
-    for (int d = 0; d < nb; ++d) acc += (double)Vk[a * nb + d] * (double)w[a * nb + d];
-  }
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) out[(int64_t)blockIdx.x * ostride + k] = acc;
-}
-
-// w -= sum_k h[inst, k] V_k
-template <typename T>
-__global__ void k_inst_orth(int64_t N, int nb, const int32_t *__restrict__ node_inst, T *__restrict__ w,
-                            const T *__restrict__ V, int64_t vstride, const double *__restrict__ h, int cnt) {
-  pdl_enter();
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= N) return;
-  const int i = node_inst[e / nb];
-  if (i < 0) return;
-  T s = w[e];
-  for (int k = 0; k < cnt; ++k) s -= (T)h[(int64_t)i * PSTR + k] * V[(int64_t)k * vstride + e];
-  w[e] = s;
-}
-
-// out = scale[inst] w (0 between instances)
-template <typename T>
-__global__ void k_inst_scale(int64_t N, int nb, const int32_t *__restrict__ node_inst, const T *__restrict__ w,
-                             const double *__restrict__ scl, T *__restrict__ out) {
-  pdl_enter();
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= N) return;
-  const int i = node_inst[e / nb];
-  out[e] = i < 0 ? T(0) : (T)(scl[i] * (double)w[e]);
-}
-
-// start of a cycle: beta_i = ||r_i||, g_i = beta_i e_1, scale 1 / beta_i; the
-// tolerance rtol beta_i is fixed at the first start; an instance already
-// within it is frozen
-__global__ void k_inst_init(int ni, int m, const double *__restrict__ nrm, double *__restrict__ g,
-                            double *__restrict__ scl, double *__restrict__ tgt, int32_t *__restrict__ frozen,
-                            int32_t *__restrict__ jc, int32_t *__restrict__ active, double rtol, int set_target) {
-  pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ni) return;
-  const double beta = sqrt(nrm[i]);
-  if (set_target) tgt[i] = rtol * beta;
-  for (int k = 0; k <= m; ++k) g[(int64_t)i * (m + 1) + k] = 0.0;
-  g[(int64_t)i * (m + 1)] = beta;
-  jc[i] = 0;
-  const bool done = !(beta > tgt[i]);
-  frozen[i] = done ? 1 : 0;
-  scl[i] = (!done && beta > 0.0) ? 1.0 / beta : 0.0;
-  if (!done) atomicAdd(active, 1);
-}
-
-// Arnoldi column j of every active instance: H(:, j) = h1 + h2, previous
-// rotations, new rotation, g update, residual estimate |g_{j+1}|; an instance
-// whose estimate reaches its tolerance (or whose new vector vanishes) freezes
-// with j + 1 columns
-__global__ void k_inst_arnoldi(int ni, int j, int m, const double *__restrict__ h1, const double *__restrict__ h2,
-                               const double *__restrict__ nrm, double *__restrict__ H, double *__restrict__ g,
-                               double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ scl,
-                               const double *__restrict__ tgt, double *__restrict__ res,
-                               int32_t *__restrict__ frozen, int32_t *__restrict__ jc, int32_t *__restrict__ active) {
-  pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ni) return;
-  if (frozen[i]) {
-    scl[i] = 0.0;
-    return;
-  }
-  double *Hi = H + (int64_t)i * (m + 1) * m, *gi = g + (int64_t)i * (m + 1);
-  double *csi = cs + (int64_t)i * (m + 1), *sni = sn + (int64_t)i * (m + 1);
-  const double hn = sqrt(nrm[i]);
-  double col[PSTR];
-  for (int k = 0; k <= j; ++k) col[k] = h1[(int64_t)i * PSTR + k] + h2[(int64_t)i * PSTR + k];
-  for (int k = 0; k < j; ++k) {
-    const double t = csi[k] * col[k] + sni[k] * col[k + 1];
-    col[k + 1] = -sni[k] * col[k] + csi[k] * col[k + 1];
-    col[k] = t;
-  }
-  const double r = hypot(col[j], hn);
-  double c = 1.0, sv = 0.0;
-  if (r > 0.0) {
-    c = col[j] / r;
-    sv = hn / r;
-  }
-  csi[j] = c;
-  sni[j] = sv;
-  col[j] = r;
-  for (int k = 0; k <= j; ++k) Hi[k * m + j] = col[k];
-  const double gj = gi[j];
-  gi[j + 1] = -sv * gj;
-  gi[j] = c * gj;
-  res[i] = fabs(gi[j + 1]);
-  jc[i] = j + 1;
-  if (res[i] <= tgt[i] || !(hn > 0.0)) {
-    frozen[i] = 1;
-    scl[i] = 0.0;
-  } else {
-    scl[i] = 1.0 / hn;
-    atomicAdd(active, 1);
-  }
-}
-
-__global__ void k_inst_backsolve(int ni, int m, const double *__restrict__ H, const double *__restrict__ g,
-                                 const int32_t *__restrict__ jc, double *__restrict__ y) {
-  pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ni) return;
-  const double *Hi = H + (int64_t)i * (m + 1) * m, *gi = g + (int64_t)i * (m + 1);
-  double *yi = y + (int64_t)i * (m + 1);
-  for (int k = jc[i] - 1; k >= 0; --k) {
-    double sv = gi[k];
-    for (int l = k + 1; l < jc[i]; ++l) sv -= Hi[k * m + l] * yi[l];
-    yi[k] = Hi[k * m + k] != 0.0 ? sv / Hi[k * m + k] : 0.0;
-  }
-}
-
-template <typename T>
-__global__ void k_inst_update_x(int64_t N, int nb, const int32_t *__restrict__ node_inst, T *__restrict__ x,
-                                const T *__restrict__ Z, int64_t zstride, const double *__restrict__ y, int m,
-                                const int32_t *__restrict__ jc) {
-  pdl_enter();
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= N) return;
-  const int i = node_inst[e / nb];
-  if (i < 0) return;
-  T sv = x[e];
-  for (int k = 0; k < jc[i]; ++k) sv += (T)y[(int64_t)i * (m + 1) + k] * Z[(int64_t)k * zstride + e];
-  x[e] = sv;
-}
-
 template <typename T>
 int dmalloc(T **p, int64_t n) {
   return cudaMalloc((void **)p, sizeof(T) * (size_t)(n > 0 ? n : 1)) == cudaSuccess ? MPM_OK
@@ -1273,6 +1507,30 @@ int read_dev_err(Ctx &c) {
   double err;
   const int rc = slot_wait(c, SLOT_WORD, &err);
   return rc ? rc : dev_err_code(c, (int)err);
+}
+
+int batch_slices(Ctx &c, const std::vector<int32_t> &node_inst) {
+  const int ni = c.ninst;
+  std::vector<std::vector<int32_t>> of(ni + 1);  // nodes by instance; those between instances last
+  for (size_t a = 0; a < node_inst.size(); ++a) of[node_inst[a] < 0 ? ni : node_inst[a]].push_back((int32_t)a);
+  std::vector<int32_t> nodes, s0;
+  std::vector<int4> sl;
+  for (int i = 0; i <= ni; ++i) {
+    s0.push_back((int32_t)sl.size());
+    if (i == ni) c.bn_live = (int)sl.size();
+    const int len = (int)of[i].size();
+    for (int b = 0; b < len; b += BG_NODES)
+      sl.push_back(make_int4(i < ni ? i : -1, (int)nodes.size() + b, std::min(BG_NODES, len - b), 0));
+    nodes.insert(nodes.end(), of[i].begin(), of[i].end());
+  }
+  c.bn_all = (int)sl.size();
+  if (dmalloc(&c.bn_nodes, nodes.size()) || dmalloc(&c.bn_s0, s0.size()) || dmalloc(&c.bn_slices, sl.size()) ||
+      dmalloc(&c.bn_part, (int64_t)c.bn_live * PSTR) || dmalloc(&c.bn_npart, c.bn_live))
+    return MPM_ERR_NO_MEMORY;
+  cudaMemcpy(c.bn_nodes, nodes.data(), sizeof(int32_t) * nodes.size(), cudaMemcpyHostToDevice);
+  cudaMemcpy(c.bn_s0, s0.data(), sizeof(int32_t) * s0.size(), cudaMemcpyHostToDevice);
+  cudaMemcpy(c.bn_slices, sl.data(), sizeof(int4) * sl.size(), cudaMemcpyHostToDevice);
+  return check_cuda(c, cudaGetLastError(), "node slices");
 }
 
 template <typename T>
@@ -1363,88 +1621,8 @@ void run_precond(Ctx &c, LinSys<T> &S, const T *v, T *z) {
   else precond<4, T>(c, S, v, z);
 }
 
-int read_active(Ctx &c, const int32_t *dptr) {
-  int32_t *h = reinterpret_cast<int32_t *>(c.h_bk);
-  cudaMemcpyAsync(h, dptr, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st);
-  cudaStreamSynchronize(c.st);
-  return h[0];
-}
-
-template <int NB, typename T>
-int fgmres_batched_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
-  const int64_t N = c.N();
-  const int m = c.m_restart, ni = c.ninst;
-  const int gN = nblk(N);
-  const T *b = S.rhs;
-  T *x = S.x, *w = S.w;
-  double *H = c.bk, *g = H + (int64_t)ni * (m + 1) * m, *cs = g + (int64_t)ni * (m + 1);
-  double *sn = cs + (int64_t)ni * (m + 1), *y = sn + (int64_t)ni * (m + 1);
-  double *h1 = y + (int64_t)ni * (m + 1), *h2 = h1 + (int64_t)ni * PSTR, *nrm = h2 + (int64_t)ni * PSTR;
-  double *scl = nrm + ni, *tgt = scl + ni, *res = tgt + ni;
-  int32_t *frozen = c.bk_i, *jc = frozen + ni, *active = jc + ni;
-  const int ib = nblk(ni, 128);
-  cudaMemsetAsync(x, 0, sizeof(T) * N, c.st);
-  auto start = [&](const T *r, int set_target) {
-    k_inst_dots<T><<<dim3(ni, 1), TPB, 0, c.st>>>(c.g, NB, c.inst, r, N, r, nrm, 1);
-    cudaMemsetAsync(active, 0, sizeof(int32_t), c.st);
-    k_inst_init<<<ib, 128, 0, c.st>>>(ni, m, nrm, g, scl, tgt, frozen, jc, active, rtol, set_target);
-    k_inst_scale<T><<<gN, TPB, 0, c.st>>>(N, NB, c.node_inst, r, scl, S.V);
-    c.launches += 3;
-    return read_active(c, active);
-  };
-  *iters = 0;
-  int nact = start(b, 1);
-  if (nact == 0) return MPM_OK;
-  int total = 0;
-  bool converged = false;
-  while (true) {
-    for (int j = 0; j < m; ++j) {
-      T *Vj = S.V + (int64_t)j * N, *Zj = S.Z + (int64_t)j * N, *Vn = S.V + (int64_t)(j + 1) * N;
-      precond<NB, T>(c, S, Vj, Zj);
-      spmv<NB, T>(c, S, Zj, w);
-      prof_begin(c, MPM_PROF_ORTH);
-      k_inst_dots<T><<<dim3(ni, j + 1), TPB, 0, c.st>>>(c.g, NB, c.inst, S.V, N, w, h1, PSTR);
-      k_inst_orth<T><<<gN, TPB, 0, c.st>>>(N, NB, c.node_inst, w, S.V, N, h1, j + 1);
-      k_inst_dots<T><<<dim3(ni, j + 1), TPB, 0, c.st>>>(c.g, NB, c.inst, S.V, N, w, h2, PSTR);
-      k_inst_orth<T><<<gN, TPB, 0, c.st>>>(N, NB, c.node_inst, w, S.V, N, h2, j + 1);
-      k_inst_dots<T><<<dim3(ni, 1), TPB, 0, c.st>>>(c.g, NB, c.inst, w, N, w, nrm, 1);
-      prof_end(c, MPM_PROF_ORTH);
-      cudaMemsetAsync(active, 0, sizeof(int32_t), c.st);
-      k_inst_arnoldi<<<ib, 128, 0, c.st>>>(ni, j, m, h1, h2, nrm, H, g, cs, sn, scl, tgt, res, frozen, jc,
-                                           active);
-      k_inst_scale<T><<<gN, TPB, 0, c.st>>>(N, NB, c.node_inst, w, scl, Vn);
-      c.launches += 7;
-      ++total;
-      nact = read_active(c, active);
-      if (nact == 0) {
-        converged = true;
-        break;
-      }
-      if (total >= maxit) break;
-    }
-    k_inst_backsolve<<<ib, 128, 0, c.st>>>(ni, m, H, g, jc, y);
-    k_inst_update_x<T><<<gN, TPB, 0, c.st>>>(N, NB, c.node_inst, x, S.Z, N, y, m, jc);
-    c.launches += 2;
-    if (converged || total >= maxit) break;
-    // restart every instance from its true residual r = b - A x
-    spmv<NB, T>(c, S, x, w);
-    k_residual_vec<T><<<gN, TPB, 0, c.st>>>(w, b, N);
-    UPMPM_LAUNCH(c);
-    if (start(w, 0) == 0) {
-      converged = true;
-      break;
-    }
-  }
-  *iters = total;
-  if (check_cuda(c, cudaGetLastError(), "fgmres")) return MPM_ERR_CUDA;
-  return converged ? MPM_OK : MPM_ERR_KRYLOV_STAGNATED;
-}
-
 template <typename T>
 int run_fgmres(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
-  if (c.ninst > 1)
-    return c.nb == 3 ? fgmres_batched_impl<3, T>(c, S, rtol, maxit, iters)
-                     : fgmres_batched_impl<4, T>(c, S, rtol, maxit, iters);
   if (c.nb == 3) return fgmres_impl<3, T>(c, S, rtol, maxit, iters);
   return fgmres_impl<4, T>(c, S, rtol, maxit, iters);
 }
