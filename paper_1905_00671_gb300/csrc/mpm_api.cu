@@ -419,7 +419,7 @@ int newton_correction(Ctx &c, LinSys<T> &S, int k, int *its) {
     else if (rc == MPM_ERR_NONFINITE) c.last_error = "non-finite value in FGMRES";
     return rc;
   }
-  run_unscale_add<T>(c, S, c.X);
+  run_add_solution<T>(c, S, c.X);
   return MPM_OK;
 }
 
@@ -1361,6 +1361,7 @@ int mpm_debug_precond(mpm_ctx *h, const double *X, const double *v, double *z) {
   }
   cudaMemcpyAsync(S.w, v, sizeof(double) * N, cudaMemcpyHostToDevice, c.st);
   run_precond<double>(c, S, S.w, S.x);
+  run_to_scaled<double>(c, S, S.x);
   cudaMemcpyAsync(z, S.x, sizeof(double) * N, cudaMemcpyDeviceToHost, c.st);
   return check_cuda(c, cudaStreamSynchronize(c.st), "debug_precond");
 }

@@ -27,10 +27,13 @@ template <typename T>
 struct MGHier;
 
 // The scaled Newton system D J D y = -D R and its solver workspace in the
-// precision T of the Krylov solve (FP64, or FP32 in the mixed mode).
+// precision T of the Krylov solve (FP64, or FP32 in the mixed mode).  The matrix
+// is kept unscaled: the basis vectors V are of the scaled system, the
+// preconditioned vectors Z and the solution x = D y are in the unscaled
+// unknowns, and a product is y = D J z.
 template <typename T>
 struct LinSys {
-  T *val = nullptr;            // nnzb_cap * nb * nb block values (scaled in place)
+  T *val = nullptr;            // nnzb_cap * nb * nb block values
   int64_t cap = 0;             // blocks val can hold
   T *dscale = nullptr;         // nb * nnodes, D = |diag J|^{-1/2}
   T *dscinv = nullptr;         // nb * nnodes, D^{-1} = |diag J|^{1/2} (multiplied, not divided by D)
@@ -441,15 +444,17 @@ void linsys_free(LinSys<T> &S);
 template <typename T>
 int linsys_reserve(Ctx &c, LinSys<T> &S);           // val for nnzb_cap blocks
 template <typename T>
-void run_scale_system(Ctx &c, LinSys<T> &S, const double *R);  // scales val, rhs = -D R
+void run_scale_system(Ctx &c, LinSys<T> &S, const double *R);  // D (val stays unscaled), rhs = -D R
 template <typename T>
 void run_block_jacobi(Ctx &c, LinSys<T> &S);
 template <typename T>
 int run_fgmres(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters);  // S.x from S.rhs
 template <typename T>
-void run_precond(Ctx &c, LinSys<T> &S, const T *v, T *z);  // z = M^{-1} v (scaled system)
+void run_precond(Ctx &c, LinSys<T> &S, const T *v, T *z);  // v of the scaled system, z = D M^{-1} v
 template <typename T>
-void run_unscale_add(Ctx &c, const LinSys<T> &S, double *X);  // X += D x
+void run_add_solution(Ctx &c, const LinSys<T> &S, double *X);  // X += x
+template <typename T>
+void run_to_scaled(Ctx &c, const LinSys<T> &S, T *z);  // z = D^-1 z
 
 // |x| and the device error word (waits for both); an MPM_ERR_* code of the latter
 int run_norm(Ctx &c, const double *x, double *norm);
@@ -463,7 +468,7 @@ template <typename T>
 int schur_setup(Ctx &c, LinSys<T> &S, bool coarse = true);  // before run_scale_system (unscaled val);
                                                              // coarse = false: the finest levels only
 template <typename T>
-void schur_apply(Ctx &c, LinSys<T> &S, const T *v, T *z);  // z = M^{-1} v
+void schur_apply(Ctx &c, LinSys<T> &S, const T *v, T *z);  // v of the scaled system, z = D M^{-1} v
 int batch_slices(Ctx &c, const std::vector<int32_t> &node_inst);  // bn_* of a batched context
 // its parts, for a caller that captures them: the split's buffers as they are
 // before the core, and the core (results in *zu, *zp)

@@ -213,9 +213,11 @@ __global__ void k_schur_lump(int64_t nnodes, const int32_t *__restrict__ row_ptr
 
 // ------------------------------------------------------------ Schur apply
 // The Krylov solver works on D J D (D = dsc); the blocks below are the
-// unscaled physical ones, so the preconditioner of D J D is D^-1 M^-1 D^-1,
-// applied with the stored D^-1 (dsi = |diag J|^{1/2}: products instead of
-// FP64 divisions, which run long on the narrow FP64 pipe).
+// unscaled physical ones, so the preconditioner of D J D is D^-1 M^-1 D^-1.  The
+// split applies the right D^-1 (dsi = |diag J|^{1/2}, stored: products instead of
+// FP64 divisions, which run long on the narrow FP64 pipe); the left one is left
+// out: z = M^-1 D^-1 v, the vector in the unscaled unknowns that the product
+// y = D J z and the solution take.
 // v_u, v_p of the unscaled system; v_p is the S-cycle's level-0 rhs, whose
 // first smoothing sweep from zero (x = omega Dinv b, pointwise) is done here.
 template <int D>
@@ -351,12 +353,12 @@ __global__ void k_b2c_update(int64_t nnodes, const int32_t *__restrict__ row_ptr
 
 template <int D>
 __global__ void k_merge(int64_t nnodes, const real *__restrict__ zu, const real *__restrict__ zp,
-                        const real *__restrict__ dsi, real *__restrict__ z) {
+                        real *__restrict__ z) {
   pdl_enter();
   const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (a >= nnodes) return;
-  for (int k = 0; k < D; ++k) z[a * (D + 1) + k] = zu[a * D + k] * dsi[a * (D + 1) + k];
-  z[a * (D + 1) + D] = zp[a] * dsi[a * (D + 1) + D];
+  for (int k = 0; k < D; ++k) z[a * (D + 1) + k] = zu[a * D + k];
+  z[a * (D + 1) + D] = zp[a];
 }
 
 // ------------------------------------------------------------ multigrid
@@ -1645,9 +1647,8 @@ void schur_core(Ctx &c, LinSys<MG_REAL> &S) {
 void schur_merge(Ctx &c, LinSys<MG_REAL> &S, const MG_REAL *zu, const MG_REAL *zp, MG_REAL *z) {
   const int64_t nn = c.g.nnodes;
   const Geom g = geom(c, nn);
-  const real *dsc = S.dscinv;  // D^-1: the unscaled v is D^-1 times the scaled one
-  if (c.d == 2) launch_pdl(c, k_merge<2>, g.blocks, g.tpb, 0, nn, zu, zp, dsc, z);
-  else launch_pdl(c, k_merge<3>, g.blocks, g.tpb, 0, nn, zu, zp, dsc, z);
+  if (c.d == 2) launch_pdl(c, k_merge<2>, g.blocks, g.tpb, 0, nn, zu, zp, z);
+  else launch_pdl(c, k_merge<3>, g.blocks, g.tpb, 0, nn, zu, zp, z);
 }
 }  // namespace MG_NS
 
