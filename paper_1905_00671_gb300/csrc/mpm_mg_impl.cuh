@@ -266,14 +266,8 @@ __global__ void k_extract_B2(int64_t nnzb, const real *__restrict__ J, real *__r
 }
 
 // w_p = v_p - B2 z_u with the compact unscaled B2: the S-cycle's level-0 rhs,
-// with its first smoothing sweep from zero (x = omega Dinv_S w_p).  B1C_LANES
-// lanes per row.
-template <int D>
-__global__ void k_b2c_update(int64_t nnodes, const int32_t *__restrict__ row_ptr,
-                             const int32_t *__restrict__ col, const real *__restrict__ B2,
-                             const real *__restrict__ zu, const real *__restrict__ vp,
-                             real *__restrict__ bs0, real *__restrict__ xs0,
-                             const real *__restrict__ dinvs0, real omega);
+// with its first smoothing sweep from zero (x = omega Dinv_S w_p).  LN lanes per
+// row (LN_ below).
 
 // Compact unscaled B1 (column D of the u rows of the unscaled J): D values
 // per block instead of the whole (D+1)^2 block.
@@ -286,17 +280,15 @@ __global__ void k_extract_B1(int64_t nnzb, const real *__restrict__ J, real *__r
 }
 
 // w_u = v_u - B1 z_p with the compact unscaled B1: the A-cycle's level-0 rhs,
-// with its first smoothing sweep from zero (x = omega Dinv w_u).  B1C_LANES
-// lanes per row.
-constexpr int B1C_LANES = 8;
-template <int D>
+// with its first smoothing sweep from zero (x = omega Dinv w_u).  LN lanes per
+// row (LN_ below).
+template <int D, int LN>
 __global__ void k_b1c_update(int64_t nnodes, const int32_t *__restrict__ row_ptr,
                              const int32_t *__restrict__ col, const real *__restrict__ B1,
                              const real *__restrict__ zp, const real *__restrict__ vu,
                              real *__restrict__ ba0, real *__restrict__ xa0,
                              const real *__restrict__ dinva0, real omega) {
   pdl_enter();
-  constexpr int LN = B1C_LANES;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t a = t / LN;
   const int lane = (int)(t % LN);
@@ -324,14 +316,13 @@ __global__ void k_b1c_update(int64_t nnodes, const int32_t *__restrict__ row_ptr
   xa0[a * D + lane] = omega * s;
 }
 
-template <int D>
+template <int D, int LN>
 __global__ void k_b2c_update(int64_t nnodes, const int32_t *__restrict__ row_ptr,
                              const int32_t *__restrict__ col, const real *__restrict__ B2,
                              const real *__restrict__ zu, const real *__restrict__ vp,
                              real *__restrict__ bs0, real *__restrict__ xs0,
                              const real *__restrict__ dinvs0, real omega) {
   pdl_enter();
-  constexpr int LN = B1C_LANES;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t a = t / LN;
   const int lane = (int)(t % LN);
@@ -388,10 +379,17 @@ __device__ inline real free_w(const LevelDev &L, int64_t a, int i) {
 // fine block-CSR in 2D, 125 in 3D, 5^d slots of a coarse stencil).  Eight
 // lanes keep the shuffle reduction (log2 LN steps per block row) small next to
 // the row's FMAs on GB300's narrow FP64 pipe; FP32 3D rows take 16 (latency).
+// Large FP64 levels take 4 lanes: on the FP64 pipe a warp instruction costs the
+// same with any number of lanes, and 4 lanes spend fewer of them on a row's
+// reduction, epilogue and last partial round: one application on the 4.2M-point
+// slope 4.9 -> 4.4 ms, on 64 batched columns 389 -> 333 us (both with the branch-free
+// restriction below).
 template <int D>
 struct LN_ {
   static constexpr int v = (sizeof(real) == sizeof(double) || D == 2) ? 8 : 16;
+  static constexpr int large = sizeof(real) == sizeof(double) ? 4 : v;
 };
+constexpr int64_t LN_LARGE_ROWS = 1 << 16;
 
 // Component `lane` (< B) of a B-vector held in registers, without indexing
 // the register array by a run-time value.
@@ -426,7 +424,7 @@ __device__ inline void row_partial(const LevelDev &L, int64_t a, int lane, const
     // rows without coupling (grid nodes outside the material: half of the
     // slope's coarse grids) are skipped whole
     if (L.nslot[a] == 0) return;
-#pragma unroll
+#pragma unroll 16
     for (int k = 0; k < (NS + LN - 1) / LN; ++k) {
       const int s = lane + k * LN;
       const int o0 = s % 5 - 2, o1 = (s / 5) % 5 - 2, o2 = D == 3 ? s / 25 - 2 : 0;
@@ -477,11 +475,10 @@ __global__ void k_mg_dinv(LevelDev L, int *err) {
 
 // One damped block-Jacobi sweep: xo = xi + w Dinv (b - A xi); zero_init: xi = 0.
 // LN lanes per row.
-template <int B, int D, bool ST>
+template <int B, int D, bool ST, int LN>
 __global__ void k_mg_smooth(LevelDev L, const real *__restrict__ xi, real *__restrict__ xo,
                             const real *__restrict__ b, real omega, int zero_init) {
   pdl_enter();
-  constexpr int LN = LN_<D>::v;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t a = t / LN;
   const int lane = (int)(t % LN);
@@ -541,11 +538,10 @@ __global__ void k_mg_csr_row(LevelDev L, const real *__restrict__ x, real *__res
   out[a * B + r] = x[a * B + r] + omega * sum;
 }
 
-template <int B, int D, bool ST>
+template <int B, int D, bool ST, int LN>
 __global__ void k_mg_resid(LevelDev L, const real *__restrict__ x, const real *__restrict__ b,
                            real *__restrict__ r) {
   pdl_enter();
-  constexpr int LN = LN_<D>::v;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t a = t / LN;
   const int lane = (int)(t % LN);
@@ -751,17 +747,26 @@ __global__ void k_mg_restrict(LevelDev F, LevelDev Cl, const real *__restrict__ 
   grid_xyz(Cl.nn[0], Cl.nn[1], (int)I, Ic);
   real acc[B];
   for (int i = 0; i < B; ++i) acc[i] = 0.0;
-  const int lo2 = D == 3 ? -1 : 0, hi2 = D == 3 ? 1 : 0;
-  for (int d2 = lo2; d2 <= hi2; ++d2)
-    for (int d1 = -1; d1 <= 1; ++d1)
-      for (int d0 = -1; d0 <= 1; ++d0) {
-        const int a0 = 2 * Ic[0] + d0, a1 = 2 * Ic[1] + d1, a2 = D == 3 ? 2 * Ic[2] + d2 : 0;
-        if (a0 < 0 || a0 >= F.nn[0] || a1 < 0 || a1 >= F.nn[1] || a2 < 0 || a2 >= F.nn[2]) continue;
-        const real wgt = pw(a0, Ic[0]) * pw(a1, Ic[1]) * (D == 3 ? pw(a2, Ic[2]) : 1.0);
-        const int64_t a = a0 + (int64_t)F.nn[0] * (a1 + (int64_t)F.nn[1] * a2);
-        if (F.inst && F.inst[a] != Cl.inst[I]) continue;
-        for (int i = 0; i < B; ++i) acc[i] += wgt * free_w(F, a, i) * rf[a * B + i];
-      }
+  // all children's loads without branches between them (a child outside the
+  // grid, of another instance or fixed contributes a selected zero), so that the
+  // loads of the 3^d children are in flight together: one application on the
+  // 80k-point footing 112 -> 104 us (a third of its kernels restrict)
+  const int inst_c = Cl.inst ? Cl.inst[I] : 0;
+#pragma unroll
+  for (int ch = 0; ch < (D == 3 ? 27 : 9); ++ch) {
+    const int d0 = ch % 3 - 1, d1 = ch / 3 % 3 - 1, d2 = D == 3 ? ch / 9 - 1 : 0;
+    const int a0 = 2 * Ic[0] + d0, a1 = 2 * Ic[1] + d1, a2 = 2 * Ic[2] + d2;
+    const bool in = a0 >= 0 && a0 < F.nn[0] && a1 >= 0 && a1 < F.nn[1] && (D == 2 || (a2 >= 0 && a2 < F.nn[2]));
+    const int64_t a = in ? a0 + (int64_t)F.nn[0] * (a1 + (int64_t)F.nn[1] * a2) : 0;
+    const bool ok = in && (!F.inst || F.inst[a] == inst_c);
+    const real wgt = (d0 ? real(0.5) : real(1)) * (d1 ? real(0.5) : real(1)) * (d2 ? real(0.5) : real(1));
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const real r = rf[a * B + i];
+      const bool use = ok && !(F.fixed && F.fixed[a * F.mstride + F.moff + i]);
+      acc[i] = fma(wgt, use ? r : real(0), acc[i]);
+    }
+  }
   for (int i = 0; i < B; ++i) bc[I * B + i] = acc[i];
   if (xc)
     for (int i = 0; i < B; ++i) {
@@ -1290,13 +1295,15 @@ void sweep(Ctx &c, MGHier<real> &H, int l) {
     launch_pdl(c, k_mg_csr_row<B, SPL, true>, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l],
                (const real *)H.b[l], mg_omega(c));
   } else {
-    const Geom g = geom(c, L.nnodes * LN_<D>::v);
-    if (l == 0)
-      launch_pdl(c, k_mg_smooth<B, D, false>, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l],
-                 (const real *)H.b[l], mg_omega(c), 0);
-    else
-      launch_pdl(c, k_mg_smooth<B, D, true>, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l],
-                 (const real *)H.b[l], mg_omega(c), 0);
+    const bool large = L.nnodes >= LN_LARGE_ROWS;
+    constexpr int LV = LN_<D>::v, LL = LN_<D>::large;
+    const Geom g = geom(c, L.nnodes * (large ? LL : LV));
+    auto go = [&](auto kernel) {
+      launch_pdl(c, kernel, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l], (const real *)H.b[l], mg_omega(c),
+                 0);
+    };
+    if (l == 0) large ? go(k_mg_smooth<B, D, false, LL>) : go(k_mg_smooth<B, D, false, LV>);
+    else large ? go(k_mg_smooth<B, D, true, LL>) : go(k_mg_smooth<B, D, true, LV>);
   }
   std::swap(H.x[l], H.x2[l]);
 }
@@ -1318,18 +1325,21 @@ void vcycle_t(Ctx &c, MGHier<real> &H, int l) {
   LevelDev &L = H.L[l], &Ln = H.L[l + 1];
   real *xn_first = l + 1 == H.tail ? nullptr : H.x[l + 1];
   for (int k = 1; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // pre-smoothing after the first
-  const Geom gr = geom(c, L.nnodes * LN_<D>::v), gc = geom(c, Ln.nnodes), gf = geom(c, L.nnodes);
+  const bool large = L.nnodes >= LN_LARGE_ROWS;
+  constexpr int LV = LN_<D>::v, LL = LN_<D>::large;
+  const Geom gr = geom(c, L.nnodes * (large ? LL : LV)), gc = geom(c, Ln.nnodes), gf = geom(c, L.nnodes);
+  auto resid = [&](auto kernel) {
+    launch_pdl(c, kernel, gr.blocks, gr.tpb, 0, L, (const real *)H.x[l], (const real *)H.b[l], H.r[l]);
+  };
   if (l == 0 && B <= 2) {
     constexpr int SPL = B <= 2 ? 4 / B : 1;
     const Geom g0 = geom(c, L.nnodes * B * SPL);
     launch_pdl(c, k_mg_csr_row<B, SPL, false>, g0.blocks, g0.tpb, 0, L, (const real *)H.x[l], H.r[l],
                (const real *)H.b[l], mg_omega(c));
   } else if (l == 0) {
-    launch_pdl(c, k_mg_resid<B, D, false>, gr.blocks, gr.tpb, 0, L, (const real *)H.x[l], (const real *)H.b[l],
-               H.r[l]);
+    large ? resid(k_mg_resid<B, D, false, LL>) : resid(k_mg_resid<B, D, false, LV>);
   } else {
-    launch_pdl(c, k_mg_resid<B, D, true>, gr.blocks, gr.tpb, 0, L, (const real *)H.x[l], (const real *)H.b[l],
-               H.r[l]);
+    large ? resid(k_mg_resid<B, D, true, LL>) : resid(k_mg_resid<B, D, true, LV>);
   }
   launch_pdl(c, k_mg_restrict<B, D>, gc.blocks, gc.tpb, 0, L, Ln, (const real *)H.r[l], H.b[l + 1], xn_first,
              mg_omega(c));
@@ -1622,25 +1632,29 @@ MG_REAL *schur_first_x0(Ctx &c, LinSys<MG_REAL> &S) { return c.schur_lower() ? S
 void schur_core(Ctx &c, LinSys<MG_REAL> &S) {
   const int64_t nn = c.g.nnodes;
   MGHier<real> &HS = *S.mgS, &HA = *S.mgA;
-  const Geom g = geom(c, nn * B1C_LANES);
+  const bool large = nn >= LN_LARGE_ROWS;
+  constexpr int LV = 8, LL = sizeof(real) == sizeof(double) ? 4 : 8;
+  const Geom g = geom(c, nn * (large ? LL : LV));
   const int32_t *rp = c.row_ptr, *cl = c.col;
   const real om = mg_omega(c);
   if (c.schur_lower()) {
     mg_vcycle(c, HA);
     const real *b2 = S.B2c, *zu = HA.x[0], *vp = S.vp, *dinv = HS.L[0].dinv;
-    if (c.d == 2)
-      launch_pdl(c, k_b2c_update<2>, g.blocks, g.tpb, 0, nn, rp, cl, b2, zu, vp, HS.b[0], HS.x[0], dinv, om);
-    else
-      launch_pdl(c, k_b2c_update<3>, g.blocks, g.tpb, 0, nn, rp, cl, b2, zu, vp, HS.b[0], HS.x[0], dinv, om);
+    auto go = [&](auto kernel) {
+      launch_pdl(c, kernel, g.blocks, g.tpb, 0, nn, rp, cl, b2, zu, vp, HS.b[0], HS.x[0], dinv, om);
+    };
+    if (c.d == 2) large ? go(k_b2c_update<2, LL>) : go(k_b2c_update<2, LV>);
+    else large ? go(k_b2c_update<3, LL>) : go(k_b2c_update<3, LV>);
     mg_vcycle(c, HS);
     return;
   }
   mg_vcycle(c, HS);
   const real *b1 = S.B1c, *zp = HS.x[0], *vu = S.vu, *dinv = HA.L[0].dinv;
-  if (c.d == 2)
-    launch_pdl(c, k_b1c_update<2>, g.blocks, g.tpb, 0, nn, rp, cl, b1, zp, vu, HA.b[0], HA.x[0], dinv, om);
-  else
-    launch_pdl(c, k_b1c_update<3>, g.blocks, g.tpb, 0, nn, rp, cl, b1, zp, vu, HA.b[0], HA.x[0], dinv, om);
+  auto go = [&](auto kernel) {
+    launch_pdl(c, kernel, g.blocks, g.tpb, 0, nn, rp, cl, b1, zp, vu, HA.b[0], HA.x[0], dinv, om);
+  };
+  if (c.d == 2) large ? go(k_b1c_update<2, LL>) : go(k_b1c_update<2, LV>);
+  else large ? go(k_b1c_update<3, LL>) : go(k_b1c_update<3, LV>);
   mg_vcycle(c, HA);
 }
 
