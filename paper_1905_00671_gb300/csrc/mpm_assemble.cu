@@ -340,46 +340,42 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
   constexpr int NB = D + 1;
   const int64_t nn = g.nnodes;
   const double dt = s.dt, b = s.beta, gm = s.gamma;
-  const int packed = v.sh_cnt[p];
-  int f[3], cn[3];
-  for (int k = 0; k < 3; ++k) {
-    f[k] = v.sh_first[k * n + p];
-    cn[k] = unpack_cnt(packed, k);
-  }
-  double dF[9] = {0}, gPn[3] = {0, 0, 0}, gVn[9] = {0}, ah[3] = {0, 0, 0};
+  // Sums over the support box.  What is linear in the nodal values is summed
+  // first and combined with the time-stepping coefficients once per point: a
+  // division per (point, node) is as many FP64 instructions as the rest of the
+  // node's work (with the hoisted basis factors: POINTTIMES).
+  double dF[9] = {0}, gPn[3] = {0, 0, 0}, gVn[9] = {0}, ah[3] = {0, 0, 0};  // dF - 1 until after the loop
+  double vh[3] = {0, 0, 0}, uh[3] = {0, 0, 0};
   double ph = 0.0, pdev = 0.0;
-  for (int k = 0; k < D; ++k) dF[k * D + k] = 1.0;
-  for (int s2 = 0; s2 < cn[2]; ++s2)
-    for (int s1 = 0; s1 < cn[1]; ++s1)
-      for (int s0 = 0; s0 < cn[0]; ++s0) {
-        const int off[3] = {s0, s1, s2};
-        const int nc3[3] = {f[0] + s0, f[1] + s1, f[2] + s2};
-        const int64_t a = node_index(g, nc3);
-        double Sa, S0a, Gn[3];
-        basis_at<D>(v, p, off, a, Sa, S0a, Gn);
-        const double P = X[a * NB + D];
-        for (int i = 0; i < D; ++i) {
-          const double dU = X[a * NB + i];
-          for (int k = 0; k < D; ++k) dF[i * D + k] += dU * Gn[k];
-        }
-        ph += Sa * P;
-        for (int k = 0; k < D; ++k) gPn[k] += P * Gn[k];
-        if (DYN) {
-          for (int i = 0; i < D; ++i) {
-            const double dU = X[a * NB + i];
-            const double vn = v.vn[i * nn + a], an = v.an[i * nn + a];
-            const double aa = dU / (b * dt * dt) - vn / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * an;
-            const double va = gm / (b * dt) * dU + (1.0 - gm / b) * vn + (1.0 - gm / (2.0 * b)) * dt * an;
-            ah[i] += Sa * aa;
-            for (int k = 0; k < D; ++k) gVn[i * D + k] += va * Gn[k];
-          }
-          const double pda = gm / (b * dt) * (P - v.Pn[a]) + (1.0 - gm / b) * v.pdn[a] +
-                             (1.0 - gm / (2.0 * b)) * dt * v.pddn[a];
-          pdev += (Sa - S0a) * pda;
-        } else {
-          pdev += (Sa - S0a) * (P - v.Pn[a]) / dt;
-        }
+  const double cvu = gm / (b * dt), cvv = 1.0 - gm / b, cva = (1.0 - gm / (2.0 * b)) * dt;
+  for_box_nodes<D>(g, v, p, [&](int64_t a, double Sa, double S0a, const double Gn[3]) {
+    const double P = X[a * NB + D], dP = P - v.Pn[a];
+    for (int i = 0; i < D; ++i) {
+      const double dU = X[a * NB + i];
+      for (int k = 0; k < D; ++k) dF[i * D + k] = fma(dU, Gn[k], dF[i * D + k]);
+      if (DYN) {
+        const double vn = v.vn[i * nn + a], an = v.an[i * nn + a];
+        const double q = fma(cvv, vn, cva * an);
+        for (int k = 0; k < D; ++k) gVn[i * D + k] = fma(q, Gn[k], gVn[i * D + k]);
+        uh[i] = fma(Sa, dU, uh[i]);
+        vh[i] = fma(Sa, vn, vh[i]);
+        ah[i] = fma(Sa, an, ah[i]);
       }
+    }
+    ph = fma(Sa, P, ph);
+    for (int k = 0; k < D; ++k) gPn[k] = fma(P, Gn[k], gPn[k]);
+    if (DYN) pdev = fma(Sa - S0a, fma(cvu, dP, fma(cvv, v.pdn[a], cva * v.pddn[a])), pdev);
+    else pdev = fma(Sa - S0a, dP, pdev);
+  });
+  if (DYN) {  // acceleration and velocity gradient (Eq. newmark) at the point
+    for (int i = 0; i < D; ++i) {
+      ah[i] = uh[i] / (b * dt * dt) - vh[i] / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * ah[i];
+      for (int k = 0; k < D; ++k) gVn[i * D + k] = fma(cvu, dF[i * D + k], gVn[i * D + k]);
+    }
+  } else {
+    pdev /= dt;
+  }
+  for (int k = 0; k < D; ++k) dF[k * D + k] += 1.0;
   const double dJ = det_d<D>(dF);
   if (!(dJ > 0.0)) {
     atomicOr(v.err, DE_NEG_J);
@@ -400,7 +396,7 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
     atomicOr(v.err, DE_NEG_J);
     return;
   }
-  const double lnJ = log(J);
+  const double lnJ = log(J), lndJ = DYN ? 0.0 : log(dJ);
   for (int i = 0; i < D; ++i)
     for (int j = 0; j < D; ++j) {
       double acc = 0.0;
@@ -492,7 +488,7 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
         }
     }
   } else {
-    divv = log(dJ) / dt;
+    divv = lndJ / dt;
   }
   const double m = v.m[p];
   for (int j = 0; j < D; ++j) {
@@ -516,7 +512,7 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
   put(RC_CST, (DYN ? tau * gm / (b * dt) : tau / dt) * Vn);
   put(RC_RST, tau * Vn * pdev);
   put(RC_DIVV, vol * divv);
-  put(RC_B2, DYN ? vol * (gm / (b * dt) + divv) : vol * (1.0 + log(dJ)) / dt);
+  put(RC_B2, DYN ? vol * (gm / (b * dt) + divv) : vol * (1.0 + lndJ) / dt);
   put(RC_MS, DYN ? m / (b * dt * dt) : 0.0);
   // The residual's per-point factors.  With g = Gn dF^-1 (Gn the gradient of
   // the basis in the configuration of t_n), the momentum term of a node,

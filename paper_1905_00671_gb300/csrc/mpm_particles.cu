@@ -374,45 +374,40 @@ __global__ void k_g2p(GridP g, StepP s, DevView v, const double *__restrict__ X)
   if (p >= n) return;
   constexpr int NB = D + 1;
   const int64_t nn = g.nnodes;
-  const int packed = v.sh_cnt[p];
-  int f[3], cn[3];
-  for (int k = 0; k < 3; ++k) {
-    f[k] = v.sh_first[k * n + p];
-    cn[k] = unpack_cnt(packed, k);
-  }
-  double dF[9] = {0}, du[3] = {0, 0, 0}, ph = 0.0;
-  double anew[3] = {0, 0, 0}, vinc[3] = {0, 0, 0}, pdh = 0.0, pddh = 0.0;
-  for (int k = 0; k < D; ++k) dF[k * D + k] = 1.0;
+  // sums over the support box; the nodal accelerations and rates are linear in
+  // nodal values, which are summed first (as in k_point_eval)
+  double dF[9] = {0}, du[3] = {0, 0, 0}, ph = 0.0;  // dF - 1 until after the loop
+  double vh[3] = {0, 0, 0}, ah[3] = {0, 0, 0}, dph = 0.0, pdh = 0.0, pddh = 0.0;
   const double b = s.beta, gm = s.gamma, dt = s.dt;
-  for (int s2 = 0; s2 < cn[2]; ++s2)
-    for (int s1 = 0; s1 < cn[1]; ++s1)
-      for (int s0 = 0; s0 < cn[0]; ++s0) {
-        const int sl[3] = {s0, s1, s2};
-        const int nc3[3] = {f[0] + s0, f[1] + s1, f[2] + s2};
-        const int64_t a = node_index(g, nc3);
-        double Sa, S0a, Gn[3];
-        basis_at<D>(v, p, sl, a, Sa, S0a, Gn);
-        for (int i = 0; i < D; ++i) {
-          const double dU = X[a * NB + i];
-          du[i] += Sa * dU;
-          for (int k = 0; k < D; ++k) dF[i * D + k] += dU * Gn[k];
-        }
-        const double P = X[a * NB + D];
-        ph += Sa * P;
-        if (DYN) {
-          for (int i = 0; i < D; ++i) {
-            const double dU = X[a * NB + i];
-            const double vn = v.vn[i * nn + a], an = v.an[i * nn + a];
-            const double aa = dU / (b * dt * dt) - vn / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * an;
-            anew[i] += Sa * aa;
-            vinc[i] += Sa * ((1.0 - gm) * an + gm * aa);
-          }
-          const double dP = P - v.Pn[a];
-          const double pdn = v.pdn[a], pddn = v.pddn[a];
-          pdh += Sa * (gm / (b * dt) * dP + (1.0 - gm / b) * pdn + (1.0 - gm / (2.0 * b)) * dt * pddn);
-          pddh += Sa * (dP / (b * dt * dt) - pdn / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * pddn);
-        }
+  for_box_nodes<D>(g, v, p, [&](int64_t a, double Sa, double, const double Gn[3]) {
+    for (int i = 0; i < D; ++i) {
+      const double dU = X[a * NB + i];
+      du[i] = fma(Sa, dU, du[i]);
+      for (int k = 0; k < D; ++k) dF[i * D + k] = fma(dU, Gn[k], dF[i * D + k]);
+      if (DYN) {
+        vh[i] = fma(Sa, v.vn[i * nn + a], vh[i]);
+        ah[i] = fma(Sa, v.an[i * nn + a], ah[i]);
       }
+    }
+    const double P = X[a * NB + D];
+    ph = fma(Sa, P, ph);
+    if (DYN) {
+      dph = fma(Sa, P - v.Pn[a], dph);
+      pdh = fma(Sa, v.pdn[a], pdh);
+      pddh = fma(Sa, v.pddn[a], pddh);
+    }
+  });
+  double anew[3] = {0, 0, 0}, vinc[3] = {0, 0, 0};
+  if (DYN) {
+    for (int i = 0; i < D; ++i) {
+      anew[i] = du[i] / (b * dt * dt) - vh[i] / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * ah[i];
+      vinc[i] = (1.0 - gm) * ah[i] + gm * anew[i];
+    }
+    const double pd = gm / (b * dt) * dph + (1.0 - gm / b) * pdh + (1.0 - gm / (2.0 * b)) * dt * pddh;
+    pddh = dph / (b * dt * dt) - pdh / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * pddh;
+    pdh = pd;
+  }
+  for (int k = 0; k < D; ++k) dF[k * D + k] += 1.0;
   const double dJ = det_d<D>(dF);
   if (!(dJ > 0.0)) {
     atomicOr(v.err, DE_NEG_J);
