@@ -222,33 +222,38 @@ __global__ void k_initial_guess(GridP g, double phi_min, DevView v, double *__re
 // renormalised over the active box nodes (see basis_at).
 // Fixed-stress term of the pressure Schur complement, lumped per node:
 // fsd_a = sum_p S_ap b2_p vol_p / (cs_p K_p), K = lambda + 2 (G - lambda ln J) / d
-// (the drained bulk modulus of the current records).  Node-centric gather in
-// (cell, id) order: these gathers read many record fields per point, and the
-// cells' contiguous runs of points serve them better than the first-node bins.
-template <int D, bool GIMP>
-__global__ void k_fs_diag(GridP g, DevView v, double *__restrict__ out) {
+// (the drained bulk modulus of the current records): the points' factors once
+// per point, then a node-centric gather over the first-node bins (a division per
+// (point, node) over the cells' candidates took 4.0 ms on the 4.2M-point slope).
+template <int D>
+__global__ void k_fs_point(int64_t n, const double *__restrict__ rec, double *__restrict__ fsp) {
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (q >= n) return;
+  const double K = rec[RC_LAM * n + q] + 2.0 * rec[RC_MUP * n + q] / D;
+  fsp[q] = rec[RC_B2 * n + q] * rec[RC_VOL * n + q] / (rec[RC_CS * n + q] * K);
+}
+
+template <int D>
+__global__ void k_fs_diag(GridP g, DevView v, const double *__restrict__ fsp, double *__restrict__ out) {
   const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (a >= g.nnodes) return;
-  const int64_t n = v.n;
-  int ac[3];
+  int ac[3], lo[3], hi[3];
   node_coords(g, a, ac);
-  int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
-  for (int k = 0; k < D; ++k) cand_range<GIMP>(ac[k], g.nc[k], lo[k], hi[k]);
-  const double *rec = v.rec;
+  fb_window<D>(v.fb_cmax, ac, ac, lo, hi);
   double acc = 0.0;
-  for (int c2 = lo[2]; c2 <= hi[2]; ++c2)
-    for (int c1 = lo[1]; c1 <= hi[1]; ++c1)
-      for (int c0 = lo[0]; c0 <= hi[0]; ++c0) {
-        const int64_t cid = cell_index(g, c0, c1, c2);
-        for (int32_t q = v.cell_start[cid]; q < v.cell_start[cid + 1]; ++q) {
-          int off[3];
-          if (!in_box<D>(v, q, ac, off)) continue;
-          double Sa, S0a, Gn[3];
-          basis_at<D>(v, q, off, a, Sa, S0a, Gn);
-          const double K = rec[RC_LAM * n + q] + 2.0 * rec[RC_MUP * n + q] / D;
-          acc += Sa * rec[RC_B2 * n + q] * rec[RC_VOL * n + q] / (rec[RC_CS * n + q] * K);
-        }
+  for (int f2 = lo[2]; f2 <= hi[2]; ++f2)
+    for (int f1 = lo[1]; f1 <= hi[1]; ++f1) {
+      int32_t b, e;
+      fb_run(g, v.fb_start, lo[0], hi[0], f1, f2, b, e);
+      for (int32_t i = b; i < e; ++i) {
+        const int32_t q = v.fb_perm[i];
+        int off[3];
+        if (!in_box4<D>(v.sh_box[q], ac, off)) continue;
+        double Sa, S0a, Gn[3];
+        basis_at<D>(v, q, off, a, Sa, S0a, Gn);
+        acc = fma(Sa, fsp[q], acc);
       }
+    }
   out[a] = acc;
 }
 
@@ -2012,15 +2017,15 @@ void run_initial_guess(Ctx &c) {
 void run_fs_diag(Ctx &c) {
   const DevView v = c.view();
   const int nbk = nblk(c.g.nnodes, 128);
-  const bool gimp = c.shape == MPM_SHAPE_GIMP;
+  double *fsp = c.stage;  // (read-back staging, free during a step)
   if (c.d == 2) {
-    if (gimp) k_fs_diag<2, true><<<nbk, 128, 0, c.st>>>(c.g, v, c.fsd);
-    else k_fs_diag<2, false><<<nbk, 128, 0, c.st>>>(c.g, v, c.fsd);
+    k_fs_point<2><<<nblk(c.n), TPB, 0, c.st>>>(c.n, c.rec, fsp);
+    k_fs_diag<2><<<nbk, 128, 0, c.st>>>(c.g, v, fsp, c.fsd);
   } else {
-    if (gimp) k_fs_diag<3, true><<<nbk, 128, 0, c.st>>>(c.g, v, c.fsd);
-    else k_fs_diag<3, false><<<nbk, 128, 0, c.st>>>(c.g, v, c.fsd);
+    k_fs_point<3><<<nblk(c.n), TPB, 0, c.st>>>(c.n, c.rec, fsp);
+    k_fs_diag<3><<<nbk, 128, 0, c.st>>>(c.g, v, fsp, c.fsd);
   }
-  UPMPM_LAUNCH(c);
+  c.launches += 2;
 }
 
 void run_count_terms(Ctx &c) {

@@ -25,6 +25,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "mpm_internal.cuh"
