@@ -384,8 +384,22 @@ template <int D>
 struct LN_ {
   static constexpr int v = (sizeof(real) == sizeof(double) || D == 2) ? 8 : 16;
   static constexpr int large = sizeof(real) == sizeof(double) ? 4 : v;
+  // small 3D levels: a row of up to 125 blocks on one warp, since what bounds
+  // them is the chain of a lane's blocks (480 nodes: 22-28 -> 11 us a pass; 3,135:
+  // 22-28 -> 15)
+  static constexpr int small = D == 3 ? 32 : v;
+  // 3D levels between: their rows (100 blocks) are bound by FP64 issue too (24k nodes:
+  // 16 lanes 75-79 us a pass, 8 lanes 62-66, 4 lanes 63)
+  static constexpr int mid = D == 3 && sizeof(real) == sizeof(double) ? 4 : v;
 };
-constexpr int64_t LN_LARGE_ROWS = 1 << 16;
+constexpr int64_t LN_LARGE_ROWS = 1 << 16, LN_SMALL_ROWS = 1 << 13;
+// f(lanes) with the compile-time lane count for a level of so many rows
+template <int D, typename F>
+inline void with_lanes(int64_t rows, F &&f) {
+  if (rows >= LN_LARGE_ROWS) f(std::integral_constant<int, LN_<D>::large>{});
+  else if (rows < LN_SMALL_ROWS) f(std::integral_constant<int, LN_<D>::small>{});
+  else f(std::integral_constant<int, LN_<D>::mid>{});
+}
 
 // Component `lane` (< B) of a B-vector held in registers, without indexing
 // the register array by a run-time value.
@@ -580,132 +594,217 @@ __global__ void k_dense_fill(LevelDev L, real *__restrict__ Ad) {
 
 // Inverse of the dense coarsest operator Ad (n x n, row-major) into Ai, for
 // the two hierarchies side by side (job 0, job 1), in two kernels:
-//   k_dense_lu: LU factorisation with partial pivoting, one block per job,
-//     in place in Ad (in dynamic shared memory when n <= DENSE_SMEM_MAX_N),
-//     row interchanges in piv[k] (LAPACK order), n^3 / 3 FMAs;
-//   k_dense_inv_cols: column c of the inverse from P A = L U (forward and
-//     back substitution on e_c), one block per column, so the n^3 FMAs of the
-//     inverse spread over many SMs (GB300's FP64 pipe does 2 FMAs per clock
-//     per SM: one block inverting a 126 x 126 matrix took over a millisecond).
+//   k_dense_lu: LU factorisation with partial pivoting, one block per job (in
+//     dynamic shared memory when it fits), row interchanges in piv[k] (LAPACK
+//     order), n^3 / 3 FMAs; the transpose of the factors, with the reciprocals of
+//     the diagonal, into At;
+//   k_dense_inv_cols: column c of the inverse from P A = L U (forward and back
+//     substitution on e_c), a warp per column with the vector in registers, so
+//     the n^3 FMAs of the inverse spread over many SMs.
+// Both are chains of n steps, and what a step costs is its barriers and the FP64
+// instructions on its path: the pivot is found by one warp comparing magnitudes
+// as integers, the elimination takes a warp per row, and the substitutions need
+// no barrier (n = 72 and 36: 306 + 64 -> 153 + 36 us; n = 180 and 60: 1,380 + 191 ->
+// 1,175 + 153, half of it the FP64 work of one SM).
 // Columns with no usable pivot (below 1e-14 of the largest entry: nodes
 // without material on the coarsest grid) are singular directions: their
 // unknowns get zero in every column of the inverse, so the coarse correction
 // leaves them alone.
 struct DenseJob {
   int n;
-  real *Ad, *Ai;
-  int *piv;  // n: row interchanged with row k; -1 marks a singular column
+  real *Ad, *Ai, *At;
+  int *piv;  // n: row interchanged with row k, -1 marks a singular column; n: P's column c has its 1 here
 };
 
 constexpr int DENSE_LU_THREADS = 512;
+constexpr size_t DENSE_SMEM_MAX = 220 * 1024;
 
-__global__ void __launch_bounds__(DENSE_LU_THREADS) k_dense_lu(DenseJob j0, DenseJob j1, int smem) {
+// bits of |v|, which order as the magnitudes do (NaN above all)
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned long long mag_bits(float v) {
+  return (unsigned long long)(__float_as_uint(v) & 0x7fffffffu);
+}
+
+// ns: the trailing ns x ns part of a job is factorised in shared memory (all of
+// it when n <= ns), the columns before it in place in Ad
+__global__ void __launch_bounds__(DENSE_LU_THREADS) k_dense_lu(DenseJob j0, DenseJob j1, int ns) {
   const DenseJob job = blockIdx.x == 0 ? j0 : j1;
-  const int n = job.n;
+  const int n = job.n, base = n > ns ? n - ns : 0;
   __shared__ int piv;
-  __shared__ real red_v[32];
-  __shared__ int red_i[32];
+  __shared__ real rpiv;
+  __shared__ int spiv[1024];
+  __shared__ unsigned long long red[DENSE_LU_THREADS / 32];
   extern __shared__ __align__(16) unsigned char dyn_smem[];
-  real *M = smem ? reinterpret_cast<real *>(dyn_smem) : job.Ad;
-  if (smem)
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) M[t] = job.Ad[t];
+  real *Ms = reinterpret_cast<real *>(dyn_smem);
+  const int lds = (n - base) | 1;  // odd: a column's entries in different banks
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // largest magnitude, for the singular-pivot threshold
-  real amax = 0;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) amax = fmax(amax, fabs(M[t]));
-  for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  if (lane == 0) red_v[wid] = amax;
+  unsigned long long top = 0;  // largest magnitude, for the singular-pivot threshold
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) top = max(top, mag_bits(job.Ad[t]));
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (lane == 0) red[wid] = top;
   __syncthreads();
-  amax = 0;
-  for (int i = 0; i < nw; ++i) amax = fmax(amax, red_v[i]);
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    // pivot: largest |M[i][k]|, i >= k (warp argmax, then across warps)
-    real best = -1;
-    int bi = k;
-    for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-      const real v = fabs(M[i * n + k]);
-      if (v > best) { best = v; bi = i; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const real ov = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
-    if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      real b = -1;
-      int p = k;
-      for (int i = 0; i < nw; ++i)
-        if (red_v[i] > b || (red_v[i] == b && red_i[i] < p)) { b = red_v[i]; p = red_i[i]; }
-      piv = b > real(1e-14) * amax ? p : -1;
-      job.piv[k] = piv;
-    }
-    __syncthreads();
-    const int p = piv;
-    if (p < 0) {  // singular column: no elimination, zero multipliers
-      for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) M[i * n + k] = 0;
-      __syncthreads();
-      continue;
-    }
-    if (p != k)
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const real t1 = M[k * n + j];
-        M[k * n + j] = M[p * n + j];
-        M[p * n + j] = t1;
+  for (int i = 0; i < nw; ++i) top = max(top, red[i]);
+  const real amax = sizeof(real) == 8 ? (real)__longlong_as_double((long long)top)
+                                      : (real)__uint_as_float((unsigned)top);
+  // columns k0 .. k1 - 1 of the matrix M (leading dimension ld, entry (o, o) first)
+  auto columns = [&](real *M, int ld, int o, int k0, int k1) {
+    for (int k = k0; k < k1; ++k) {
+      if (wid == 0) {  // pivot: largest |M[i][k]|, i >= k, the first of equals
+        unsigned long long best = 0;
+        int bi = n;
+        for (int i = k + lane; i < n; i += 32) {
+          const unsigned long long v = mag_bits(M[(i - o) * ld + k - o]);
+          if (v > best || bi == n) { best = v; bi = i; }
+        }
+        for (int q = 16; q > 0; q >>= 1) {
+          const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, q);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, q);
+          if (oi < n && (bi == n || ov > best || (ov == best && oi < bi))) { best = ov; bi = oi; }
+        }
+        if (lane == 0) {
+          const real v = M[(bi - o) * ld + k - o];
+          const bool use = fabs(v) > real(1e-14) * amax;
+          piv = spiv[k] = use ? bi : -1;
+          rpiv = use ? real(1) / v : real(0);
+          job.piv[k] = piv;
+          job.At[(int64_t)k * n + k] = rpiv;
+        }
       }
-    __syncthreads();
-    const real inv = real(1) / M[k * n + k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) M[i * n + k] *= inv;
-    __syncthreads();
-    const int w = n - k - 1;
-    for (int t = threadIdx.x; t < w * w; t += blockDim.x) {
-      const int i = k + 1 + t / w, j = k + 1 + t % w;
-      M[i * n + j] = fma(-M[i * n + k], M[k * n + j], M[i * n + j]);
+      __syncthreads();
+      const int p = piv;
+      const real inv = rpiv;
+      if (p < 0) {  // singular column: no elimination, zero multipliers
+        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) M[(i - o) * ld + k - o] = 0;
+        __syncthreads();
+        continue;
+      }
+      if (p != k) {  // (the multipliers of the columns before o are in Ad)
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+          real *a = j < o ? job.Ad + (int64_t)k * n + j : M + (k - o) * ld + j - o;
+          real *b = j < o ? job.Ad + (int64_t)p * n + j : M + (p - o) * ld + j - o;
+          const real t1 = *a;
+          *a = *b;
+          *b = t1;
+        }
+        __syncthreads();
+      }
+      const real *row = M + (k - o) * ld - o;
+      for (int i = k + 1 + wid; i < n; i += nw) {
+        real *mi = M + (i - o) * ld - o;
+        const real l = mi[k] * inv;
+        for (int j = k + 1 + lane; j < n; j += 32) mi[j] = fma(-l, row[j], mi[j]);
+        __syncwarp();
+        if (lane == 0) mi[k] = l;
+      }
+      __syncthreads();
     }
-    __syncthreads();
+  };
+  columns(job.Ad, n, 0, 0, base);
+  for (int t = threadIdx.x; t < (n - base) * (n - base); t += blockDim.x) {
+    const int i = t / (n - base), j = t % (n - base);
+    Ms[i * lds + j] = job.Ad[(int64_t)(i + base) * n + j + base];
   }
-  if (smem)
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) job.Ad[t] = M[t];
-}
-
-// block (c, job): column c of the job's inverse; dynamic shared memory n values
-__global__ void k_dense_inv_cols(DenseJob j0, DenseJob j1) {
-  const DenseJob job = blockIdx.y == 0 ? j0 : j1;
-  const int n = job.n, c = blockIdx.x;
-  if (c >= n) return;  // block-uniform
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  real *y = reinterpret_cast<real *>(dyn_smem);
-  const real *LU = job.Ad;
-  const int *pv = job.piv;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) y[i] = i == c ? real(1) : real(0);
   __syncthreads();
-  if (threadIdx.x == 0)  // y = P e_c (the interchanges in order)
+  columns(Ms, lds, base, base, n);
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+    const int i = t % n, k = t / n;  // At[k][i] = M[i][k] off the diagonal
+    if (i != k) job.At[t] = i >= base && k >= base ? Ms[(i - base) * lds + k - base] : job.Ad[(int64_t)i * n + k];
+  }
+  for (int c = threadIdx.x; c < n; c += blockDim.x) {  // where the interchanges take entry c of e_c
+    int pos = c;
     for (int k = 0; k < n; ++k) {
-      const int p = pv[k];
-      if (p > k) { const real t = y[k]; y[k] = y[p]; y[p] = t; }
+      const int p = spiv[k];
+      if (p >= 0) pos = pos == k ? p : (pos == p ? k : pos);
     }
-  __syncthreads();
-  for (int i = 0; i < n; ++i) {  // L y = P e_c (unit lower triangle)
-    const real yi = y[i];
-    if (yi != real(0))
-      for (int k = i + 1 + threadIdx.x; k < n; k += blockDim.x) y[k] = fma(-LU[k * n + i], yi, y[k]);
-    __syncthreads();
+    job.piv[n + c] = pos;
   }
-  for (int i = n - 1; i >= 0; --i) {  // U x = y
-    const real xi = pv[i] < 0 ? real(0) : y[i] / LU[i * n + i];
-    __syncthreads();
-    if (threadIdx.x == 0) y[i] = xi;
-    if (xi != real(0))
-      for (int k = threadIdx.x; k < i; k += blockDim.x) y[k] = fma(-LU[k * n + i], xi, y[k]);
-    __syncthreads();
-  }
-  for (int k = threadIdx.x; k < n; k += blockDim.x) job.Ai[(int64_t)k * n + c] = y[k];
 }
 
-// largest coarsest system factorised in shared memory (n^2 values)
-constexpr int DENSE_SMEM_MAX_N = 160;
+// warp (c, job): column c of the job's inverse, n <= 32 NR; the factors' columns
+// are fetched PF steps ahead (they do not depend on the vector)
+template <int NR, int PF>
+__device__ void dense_inv_col(const DenseJob &job, int c, int lane) {
+  const int n = job.n;
+  const real *At = job.At;
+  const int pos = job.piv[n + c];
+  real y[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r) y[r] = lane + 32 * r == pos ? real(1) : real(0);
+  auto entry = [&](int i) {  // y_i
+    real v = y[0];
+#pragma unroll
+    for (int r = 1; r < NR; ++r) v = (i >> 5) == r ? y[r] : v;
+    return __shfl_sync(0xffffffffu, v, i & 31);
+  };
+  real cur[PF][NR], nxt[PF][NR], dc[PF], dn[PF];
+  // L y = P e_c (unit lower triangle), by columns
+  auto fetch_l = [&](int i0, real (&a)[PF][NR]) {
+#pragma unroll
+    for (int u = 0; u < PF; ++u)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int i = i0 + u, k = lane + 32 * r;
+        a[u][r] = i < n && k > i && k < n ? At[(int64_t)i * n + k] : real(0);
+      }
+  };
+  fetch_l(0, cur);
+  for (int i0 = 0; i0 < n; i0 += PF) {
+    fetch_l(i0 + PF, nxt);
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {
+      if (i0 + u >= n) break;
+      const real yi = entry(i0 + u);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) y[r] = fma(-cur[u][r], yi, y[r]);
+    }
+#pragma unroll
+    for (int u = 0; u < PF; ++u)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) cur[u][r] = nxt[u][r];
+  }
+  // U x = y, by columns from the last
+  auto fetch_u = [&](int i0, real (&a)[PF][NR], real (&dg)[PF]) {
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {
+      const int i = i0 - u;
+      dg[u] = i >= 0 ? At[(int64_t)i * n + i] : real(0);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) a[u][r] = i >= 0 && lane + 32 * r < i ? At[(int64_t)i * n + lane + 32 * r] : real(0);
+    }
+  };
+  fetch_u(n - 1, cur, dc);
+  for (int i0 = n - 1; i0 >= 0; i0 -= PF) {
+    fetch_u(i0 - PF, nxt, dn);
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {
+      const int i = i0 - u;
+      if (i < 0) break;
+      const real xi = entry(i) * dc[u];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) y[r] = lane + 32 * r == i ? xi : fma(-cur[u][r], xi, y[r]);
+    }
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {
+      dc[u] = dn[u];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) cur[u][r] = nxt[u][r];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+    if (lane + 32 * r < n) job.Ai[(int64_t)(lane + 32 * r) * n + c] = y[r];
+}
+
+__global__ void __launch_bounds__(128) k_dense_inv_cols(DenseJob j0, DenseJob j1) {
+  const DenseJob job = blockIdx.y == 0 ? j0 : j1;
+  const int c = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= job.n) return;
+  if (job.n <= 96) dense_inv_col<3, 8>(job, c, lane);
+  else if (job.n <= 192) dense_inv_col<6, 4>(job, c, lane);
+  else dense_inv_col<32, 1>(job, c, lane);
+}
 
 // x = Ai b
 // one warp per row i; lanes split the row and reduce
@@ -732,44 +831,51 @@ __device__ inline real pw(int a, int I) {
 
 // b_c(I) = sum_a P_aI r_a over the fine nodes within one fine cell of 2I; if
 // xc is given, also the coarse level's first smoothing sweep from zero,
-// x_c = omega Dinv_c b_c.
+// x_c = omega Dinv_c b_c.  A lane per component (32 / B nodes a warp).  All
+// children's loads without branches between them (a child outside the grid, of
+// another instance or fixed contributes a selected zero), so that the loads of
+// the 3^d children are in flight together: one application on the 80k-point
+// footing 112 -> 104 us (a third of its kernels restrict); a lane per component
+// instead of per node: 16 -> 10 and 12 -> 7 us a launch on 3D levels of 3,135 and 480
+// nodes.
+template <int B>
+__host__ __device__ constexpr int restrict_nodes() { return 32 / B; }  // per warp
 template <int B, int D>
 __global__ void k_mg_restrict(LevelDev F, LevelDev Cl, const real *__restrict__ rf,
                               real *__restrict__ bc, real *__restrict__ xc, real omega) {
   pdl_enter();
-  const int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (I >= Cl.nnodes) return;
-  int Ic[3];
-  grid_xyz(Cl.nn[0], Cl.nn[1], (int)I, Ic);
-  real acc[B];
-  for (int i = 0; i < B; ++i) acc[i] = 0.0;
-  // all children's loads without branches between them (a child outside the
-  // grid, of another instance or fixed contributes a selected zero), so that the
-  // loads of the 3^d children are in flight together: one application on the
-  // 80k-point footing 112 -> 104 us (a third of its kernels restrict)
-  const int inst_c = Cl.inst ? Cl.inst[I] : 0;
+  constexpr int NPW = restrict_nodes<B>();
+  const int lane = threadIdx.x & 31;
+  const int64_t I = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * NPW + lane / B;
+  const int i = lane % B;
+  const bool live = lane < NPW * B && I < Cl.nnodes;
+  real acc = 0;
+  if (live) {
+    int Ic[3];
+    grid_xyz(Cl.nn[0], Cl.nn[1], (int)I, Ic);
+    const int inst_c = Cl.inst ? Cl.inst[I] : 0;
 #pragma unroll
-  for (int ch = 0; ch < (D == 3 ? 27 : 9); ++ch) {
-    const int d0 = ch % 3 - 1, d1 = ch / 3 % 3 - 1, d2 = D == 3 ? ch / 9 - 1 : 0;
-    const int a0 = 2 * Ic[0] + d0, a1 = 2 * Ic[1] + d1, a2 = 2 * Ic[2] + d2;
-    const bool in = a0 >= 0 && a0 < F.nn[0] && a1 >= 0 && a1 < F.nn[1] && (D == 2 || (a2 >= 0 && a2 < F.nn[2]));
-    const int64_t a = in ? a0 + (int64_t)F.nn[0] * (a1 + (int64_t)F.nn[1] * a2) : 0;
-    const bool ok = in && (!F.inst || F.inst[a] == inst_c);
-    const real wgt = (d0 ? real(0.5) : real(1)) * (d1 ? real(0.5) : real(1)) * (d2 ? real(0.5) : real(1));
-#pragma unroll
-    for (int i = 0; i < B; ++i) {
+    for (int ch = 0; ch < (D == 3 ? 27 : 9); ++ch) {
+      const int d0 = ch % 3 - 1, d1 = ch / 3 % 3 - 1, d2 = D == 3 ? ch / 9 - 1 : 0;
+      const int a0 = 2 * Ic[0] + d0, a1 = 2 * Ic[1] + d1, a2 = 2 * Ic[2] + d2;
+      const bool in = a0 >= 0 && a0 < F.nn[0] && a1 >= 0 && a1 < F.nn[1] && (D == 2 || (a2 >= 0 && a2 < F.nn[2]));
+      const int64_t a = in ? a0 + (int64_t)F.nn[0] * (a1 + (int64_t)F.nn[1] * a2) : 0;
+      const bool ok = in && (!F.inst || F.inst[a] == inst_c) &&
+                      !(F.fixed && F.fixed[a * F.mstride + F.moff + i]);
       const real r = rf[a * B + i];
-      const bool use = ok && !(F.fixed && F.fixed[a * F.mstride + F.moff + i]);
-      acc[i] = fma(wgt, use ? r : real(0), acc[i]);
+      const real wgt = (d0 ? real(0.5) : real(1)) * (d1 ? real(0.5) : real(1)) * (d2 ? real(0.5) : real(1));
+      acc = fma(wgt, ok ? r : real(0), acc);
     }
+    bc[I * B + i] = acc;
   }
-  for (int i = 0; i < B; ++i) bc[I * B + i] = acc[i];
-  if (xc)
-    for (int i = 0; i < B; ++i) {
-      real s = 0.0;
-      for (int j = 0; j < B; ++j) s = fma(Cl.dinv[I * B * B + i * B + j], acc[j], s);
-      xc[I * B + i] = omega * s;
-    }
+  if (!xc) return;
+  real s = 0;
+#pragma unroll
+  for (int j = 0; j < B; ++j) {
+    const real bj = __shfl_sync(0xffffffffu, acc, lane - i + j);
+    if (live) s = fma(Cl.dinv[I * B * B + i * B + j], bj, s);
+  }
+  if (live) xc[I * B + i] = omega * s;
 }
 
 // (P x_c)(a) at fine node a from its 2^d candidate coarse parents: per axis
@@ -832,7 +938,7 @@ __global__ void k_mg_prolong(LevelDev F, LevelDev Cl, real *__restrict__ xf,
 // deposit (FP32) 47 -> 19, harmonic footing 76 -> 46, 80k-point footing 139 -> 109,
 // 64 batched columns 430 -> 389; with 768 the harmonic footing keeps one level more.
 constexpr int TAIL_MAX = 1024;
-constexpr int TAIL_COLS = 4;
+constexpr int TAIL_COLS = 2;  // (4: one block per SM by its shared memory, 331 us for the 966 unknowns below)
 constexpr int TAIL_LEVELS = 8;
 constexpr int TAIL_THREADS = 512;
 
@@ -849,16 +955,27 @@ struct TailArgs {
 
 // out = b - A x (SMOOTH: x + omega Dinv (b - A x)) for TAIL_COLS columns; vectors
 // [unknown][column]; a thread per row.  The thread's row sum is in slot order.
+// box (or null): x and b are zero at the rows outside it, and so is out.
 template <int B, int D, bool ST, bool SMOOTH>
-__device__ inline void tail_rows(const LevelDev &L, const real *x, real *out, const real *b, real omega) {
+__device__ inline void tail_rows(const LevelDev &L, const real *x, real *out, const real *b, real omega,
+                                 const int *box) {
   constexpr int NC = TAIL_COLS;
   for (int a = threadIdx.x; a < (int)L.nnodes; a += blockDim.x) {
+    if (box) {
+      int ac[3];
+      grid_xyz(L.nn[0], L.nn[1], a, ac);
+      if (ac[0] < box[0] || ac[0] > box[1] || ac[1] < box[2] || ac[1] > box[3] || ac[2] < box[4] || ac[2] > box[5]) {
+#pragma unroll
+        for (int i = 0; i < B * NC; ++i) out[a * B * NC + i] = 0;
+        continue;
+      }
+    }
     real acc[B][NC];
 #pragma unroll
     for (int i = 0; i < B; ++i)
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[i][c] = 0;
-    auto add = [&](const real *__restrict__ blk, int64_t nb) {
+    auto add = [&](const real *blk, int64_t nb) {
 #pragma unroll
       for (int j = 0; j < B; ++j)
 #pragma unroll
@@ -877,7 +994,14 @@ __device__ inline void tail_rows(const LevelDev &L, const real *x, real *out, co
       for (int s = 0; s < NS_<D>::v; ++s) {
         const int b0 = ac[0] + s % 5 - 2, b1 = ac[1] + (s / 5) % 5 - 2, b2 = ac[2] + (D == 3 ? s / 25 - 2 : 0);
         if (b0 < 0 || b0 >= L.nn[0] || b1 < 0 || b1 >= L.nn[1] || b2 < 0 || b2 >= L.nn[2]) continue;
-        add(base + s * B * B, b0 + (int64_t)L.nn[0] * (b1 + (int64_t)L.nn[1] * b2));
+        real blk[B * B];  // most blocks of a coarse stencil are zero: skipped by an integer test
+        unsigned long long any = 0;
+#pragma unroll
+        for (int e = 0; e < B * B; ++e) {
+          blk[e] = base[s * B * B + e];
+          any |= mag_bits(blk[e]);
+        }
+        if (any) add(blk, b0 + (int64_t)L.nn[0] * (b1 + (int64_t)L.nn[1] * b2));
       }
     }
 #pragma unroll
@@ -901,9 +1025,10 @@ __device__ inline void tail_rows(const LevelDev &L, const real *x, real *out, co
 }
 
 template <int B, int D, bool SMOOTH>
-__device__ inline void tail_level(const TailArgs &A, int l, const real *x, real *out, const real *b) {
-  if (l == 0 && !A.st0) tail_rows<B, D, false, SMOOTH>(A.L[l], x, out, b, A.omega);
-  else tail_rows<B, D, true, SMOOTH>(A.L[l], x, out, b, A.omega);
+__device__ inline void tail_level(const TailArgs &A, int l, const real *x, real *out, const real *b,
+                                  const int *box = nullptr) {
+  if (l == 0 && !A.st0) tail_rows<B, D, false, SMOOTH>(A.L[l], x, out, b, A.omega, box);
+  else tail_rows<B, D, true, SMOOTH>(A.L[l], x, out, b, A.omega, box);
 }
 
 // Columns c0 .. c0 + TAIL_COLS - 1 of T.  Dynamic shared memory: per level x,
@@ -941,7 +1066,28 @@ __device__ void tail_build(const TailArgs &A, int c0, real *sm) {
       __syncthreads();
       swap(x[l], r[l]);
     }
-    tail_level<B, D, false>(A, l, x[l], r[l], b[l]);
+    // the first residual of the unit vectors is zero beyond their nodes' stencils
+    int box[6];
+    const bool near = l == 0 && A.nsw == 1;
+    if (near) {
+      int p[3], q[3];
+      grid_xyz(L.nn[0], L.nn[1], c0 / B, p);
+      grid_xyz(L.nn[0], L.nn[1], min(c0 + NC - 1, A.n - 1) / B, q);
+      const int reach = A.st0 ? 2 : 3;
+      if (p[1] != q[1] || p[2] != q[2]) {  // the columns' nodes run over a row's end
+        p[0] = 0;
+        q[0] = L.nn[0] - 1;
+      }
+      if (p[2] != q[2]) {
+        p[1] = 0;
+        q[1] = L.nn[1] - 1;
+      }
+      for (int k = 0; k < 3; ++k) {
+        box[2 * k] = min(p[k], q[k]) - reach;
+        box[2 * k + 1] = max(p[k], q[k]) + reach;
+      }
+    }
+    tail_level<B, D, false>(A, l, x[l], r[l], b[l], near ? box : nullptr);
     __syncthreads();
     for (int t = threadIdx.x; t < (int)Ln.nnodes * B * NC; t += blockDim.x) {  // restriction
       const int c = t % NC, I = t / NC / B, i = t / NC % B;
@@ -1155,20 +1301,25 @@ __global__ void k_mg_rap2(LevelDev F, LevelDev Cl, const real *__restrict__ T) {
 
 // Nonzero blocks of each coarse row (a block is zero when the product never
 // reached it: the coupling is absent), so that the row kernels skip the rows
-// of nodes without coupling.  Thread per row.
+// of nodes without coupling.  A warp per row (a thread per row read its up to 9 KB
+// alone: 110 us on a 3,000-node level).
 template <int B, int D>
 __global__ void k_mg_rowcount(LevelDev Cl) {
   constexpr int NS = NS_<D>::v;
-  const int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t I = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (I >= Cl.nnodes) return;
   const real *row = Cl.sval + I * NS * B * B;
   int cnt = 0;
-  for (int s = 0; s < NS; ++s) {
+  for (int s0 = 0; s0 < NS; s0 += 32) {
+    const int s = s0 + lane;
     bool nz = false;
-    for (int e = 0; e < B * B; ++e) nz |= row[s * B * B + e] != real(0);
-    cnt += nz ? 1 : 0;
+    if (s < NS)
+#pragma unroll
+      for (int e = 0; e < B * B; ++e) nz |= row[s * B * B + e] != real(0);
+    cnt += __popc(__ballot_sync(0xffffffffu, nz));
   }
-  Cl.nslot[I] = (uint8_t)cnt;
+  if (lane == 0) Cl.nslot[I] = (uint8_t)cnt;
 }
 
 }  // namespace MG_NS
@@ -1179,7 +1330,8 @@ struct MGHier<MG_REAL> {
   int B = 1, nlev = 0;
   MG_NS::LevelDev L[16];
   MG_REAL *x[16], *x2[16], *b[16], *r[16];
-  MG_REAL *Ad = nullptr, *Ai = nullptr;  // dense coarsest operator (LU factors after set-up) and its inverse
+  // dense coarsest operator (LU factors after set-up), its inverse, the factors' transpose
+  MG_REAL *Ad = nullptr, *Ai = nullptr, *At = nullptr;
   int *piv = nullptr;                    // row interchanges of the LU factorisation
   MG_REAL *apT = nullptr;                // finest level x 5^d window: A P, first pass of a level's product
   int ncoarse = 0;                       // unknowns of the coarsest level
@@ -1207,7 +1359,7 @@ void mg_setup_t(Ctx &c, MGHier<real> &H) {
         k_mg_ap<B, D, true><<<nblk(ap_threads(H.L[l - 1].nnodes, NS)), TPB, 0, c.st>>>(H.L[l - 1], L, H.apT);
         k_mg_rap2<B, D, true><<<g2, TPB, 0, c.st>>>(H.L[l - 1], L, H.apT);
       }
-      k_mg_rowcount<B, D><<<nbk, TPB, 0, c.st>>>(L);
+      k_mg_rowcount<B, D><<<nblk(L.nnodes * 32), TPB, 0, c.st>>>(L);
       UPMPM_LAUNCH(c);
       UPMPM_LAUNCH(c);
       UPMPM_LAUNCH(c);
@@ -1228,13 +1380,13 @@ void mg_setup_t(Ctx &c, MGHier<real> &H) {
 // Inverses of the coarsest operators of two hierarchies, in one launch.
 void dense_invert_pair(Ctx &c, MGHier<real> &H0, MGHier<real> &H1) {
   const int nmax = H0.ncoarse > H1.ncoarse ? H0.ncoarse : H1.ncoarse;
-  const int smem = nmax <= DENSE_SMEM_MAX_N;
-  const size_t bytes = smem ? sizeof(real) * nmax * nmax : 0;
-  if (smem && bytes > 48 * 1024)
-    cudaFuncSetAttribute(k_dense_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  const DenseJob a{H0.ncoarse, H0.Ad, H0.Ai, H0.piv}, b{H1.ncoarse, H1.Ad, H1.Ai, H1.piv};
-  k_dense_lu<<<2, DENSE_LU_THREADS, bytes, c.st>>>(a, b, smem);
-  k_dense_inv_cols<<<dim3(nmax, 2), 128, sizeof(real) * nmax, c.st>>>(a, b);
+  int ns = nmax;
+  while (sizeof(real) * (size_t)ns * (ns | 1) > DENSE_SMEM_MAX) --ns;
+  const size_t bytes = sizeof(real) * (size_t)ns * (ns | 1);
+  cudaFuncSetAttribute(k_dense_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM_MAX);
+  const DenseJob a{H0.ncoarse, H0.Ad, H0.Ai, H0.At, H0.piv}, b{H1.ncoarse, H1.Ad, H1.Ai, H1.At, H1.piv};
+  k_dense_lu<<<2, DENSE_LU_THREADS, bytes, c.st>>>(a, b, ns);
+  k_dense_inv_cols<<<dim3(nblk(nmax, 4), 2), 128, 0, c.st>>>(a, b);
   c.launches += 2;
 }
 
@@ -1299,15 +1451,16 @@ void sweep(Ctx &c, MGHier<real> &H, int l) {
     launch_pdl(c, k_mg_csr_row<B, SPL, true>, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l],
                (const real *)H.b[l], mg_omega(c));
   } else {
-    const bool large = L.nnodes >= LN_LARGE_ROWS;
-    constexpr int LV = LN_<D>::v, LL = LN_<D>::large;
-    const Geom g = geom(c, L.nnodes * (large ? LL : LV));
-    auto go = [&](auto kernel) {
-      launch_pdl(c, kernel, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l], (const real *)H.b[l], mg_omega(c),
-                 0);
-    };
-    if (l == 0) large ? go(k_mg_smooth<B, D, false, LL>) : go(k_mg_smooth<B, D, false, LV>);
-    else large ? go(k_mg_smooth<B, D, true, LL>) : go(k_mg_smooth<B, D, true, LV>);
+    with_lanes<D>(L.nnodes, [&](auto lanes) {
+      constexpr int LN = decltype(lanes)::value;
+      const Geom g = geom(c, L.nnodes * LN);
+      auto go = [&](auto kernel) {
+        launch_pdl(c, kernel, g.blocks, g.tpb, 0, L, (const real *)H.x[l], H.x2[l], (const real *)H.b[l],
+                   mg_omega(c), 0);
+      };
+      if (l == 0) go(k_mg_smooth<B, D, false, LN>);
+      else go(k_mg_smooth<B, D, true, LN>);
+    });
   }
   std::swap(H.x[l], H.x2[l]);
 }
@@ -1329,21 +1482,22 @@ void vcycle_t(Ctx &c, MGHier<real> &H, int l) {
   LevelDev &L = H.L[l], &Ln = H.L[l + 1];
   real *xn_first = l + 1 == H.tail ? nullptr : H.x[l + 1];
   for (int k = 1; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // pre-smoothing after the first
-  const bool large = L.nnodes >= LN_LARGE_ROWS;
-  constexpr int LV = LN_<D>::v, LL = LN_<D>::large;
-  const Geom gr = geom(c, L.nnodes * (large ? LL : LV)), gc = geom(c, Ln.nnodes), gf = geom(c, L.nnodes);
-  auto resid = [&](auto kernel) {
-    launch_pdl(c, kernel, gr.blocks, gr.tpb, 0, L, (const real *)H.x[l], (const real *)H.b[l], H.r[l]);
-  };
+  const Geom gc = geom(c, (Ln.nnodes + restrict_nodes<B>() - 1) / restrict_nodes<B>() * 32), gf = geom(c, L.nnodes);
   if (l == 0 && B <= 2) {
     constexpr int SPL = B <= 2 ? 4 / B : 1;
     const Geom g0 = geom(c, L.nnodes * B * SPL);
     launch_pdl(c, k_mg_csr_row<B, SPL, false>, g0.blocks, g0.tpb, 0, L, (const real *)H.x[l], H.r[l],
                (const real *)H.b[l], mg_omega(c));
-  } else if (l == 0) {
-    large ? resid(k_mg_resid<B, D, false, LL>) : resid(k_mg_resid<B, D, false, LV>);
   } else {
-    large ? resid(k_mg_resid<B, D, true, LL>) : resid(k_mg_resid<B, D, true, LV>);
+    with_lanes<D>(L.nnodes, [&](auto lanes) {
+      constexpr int LN = decltype(lanes)::value;
+      const Geom g = geom(c, L.nnodes * LN);
+      auto go = [&](auto kernel) {
+        launch_pdl(c, kernel, g.blocks, g.tpb, 0, L, (const real *)H.x[l], (const real *)H.b[l], H.r[l]);
+      };
+      if (l == 0) go(k_mg_resid<B, D, false, LN>);
+      else go(k_mg_resid<B, D, true, LN>);
+    });
   }
   launch_pdl(c, k_mg_restrict<B, D>, gc.blocks, gc.tpb, 0, L, Ln, (const real *)H.r[l], H.b[l + 1], xn_first,
              mg_omega(c));
@@ -1422,7 +1576,8 @@ int mg_alloc(Ctx &c, MGHier<real> &H, int B) {
     return MPM_ERR_BAD_ARG;
   }
   if (cudaMalloc(&H.Ad, sizeof(real) * H.ncoarse * H.ncoarse) ||
-      cudaMalloc(&H.Ai, sizeof(real) * H.ncoarse * H.ncoarse) || cudaMalloc(&H.piv, sizeof(int) * H.ncoarse))
+      cudaMalloc(&H.Ai, sizeof(real) * H.ncoarse * H.ncoarse) ||
+      cudaMalloc(&H.At, sizeof(real) * H.ncoarse * H.ncoarse) || cudaMalloc(&H.piv, 2 * sizeof(int) * H.ncoarse))
     return MPM_ERR_NO_MEMORY;
   H.tail = H.nlev - 1;
   while (H.tail > 0 && H.L[H.tail - 1].nnodes * B <= TAIL_MAX && H.nlev - H.tail < TAIL_LEVELS) --H.tail;
@@ -1437,10 +1592,11 @@ int mg_alloc(Ctx &c, MGHier<real> &H, int B) {
 void mg_free(MGHier<real> &H) {
   cudaFree(H.Ad);
   cudaFree(H.Ai);
+  cudaFree(H.At);
   cudaFree(H.piv);
   cudaFree(H.apT);
   cudaFree(H.T);
-  H.Ad = H.Ai = H.apT = H.T = nullptr;
+  H.Ad = H.Ai = H.At = H.apT = H.T = nullptr;
   H.piv = nullptr;
   for (int l = 0; l < H.nlev; ++l) {
     cudaFree(const_cast<int32_t *>(H.L[l].inst));
