@@ -522,7 +522,7 @@ void free_all(Ctx &c) {
   for (float *p : fptrs)
     if (p) cudaFree(p);
   void *ptrs[] = {c.pf, c.pf_alt, c.pid, c.pid_alt, c.surf, c.surf_alt, c.cell, c.cell_tmp,
-                  c.cell_start, c.cell_cursor, c.perm, c.sh_first, c.sh_cnt, c.sh_box, c.fb_key, c.fb_start, c.fb_cursor, c.fb_perm, c.fb_cmax, c.jb, c.jb_cnt, c.pn_cnt, c.pn_base, c.sh_S, c.sh_dS,
+                  c.cell_start, c.cell_cursor, c.perm, c.sh_first, c.sh_cnt, c.sh_box, c.fb_key, c.fb_start, c.fb_cursor, c.fb_perm, c.fb_cmax, c.jb, c.jb_cnt, c.rb, c.rb_cnt, c.pn_cnt, c.pn_base, c.sh_S, c.sh_dS,
                   c.sh_S0, c.m, c.rec, c.pn, c.M, c.Pn, c.vn, c.an, c.pdn, c.pddn, c.phi, c.act, c.fsd, c.sh_nrm, c.fixed, c.u_fixed,
                   c.p_fixed, c.u_value, c.p_value, c.trac, c.trac_raw, c.flux, c.err, c.row_nnz,
                   c.row_ptr, c.row_of, c.col, c.row_mask, c.X, c.R, c.dX, c.stage, c.H, c.gvec,

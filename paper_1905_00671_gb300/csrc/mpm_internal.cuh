@@ -363,6 +363,10 @@ struct Ctx {
   int32_t *jb_cnt = nullptr;
   int jb_ring = 0;
   bool jb_short = false;                 // memory was short of the ring asked for
+  // residual by first-node bins: the bins' sums and box extents
+  double *rb = nullptr;
+  int64_t rb_cap = 0;
+  int32_t *rb_cnt = nullptr;
   int *h_cmax = nullptr;                 // pinned: the step's largest box extent per axis
   unsigned long long *h_terms = nullptr; // pinned copy
   // Jacobian kernel configuration per precision ([0] FP64, [1] FP32): the
