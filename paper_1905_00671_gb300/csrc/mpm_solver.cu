@@ -279,6 +279,25 @@ __global__ void k_bj_apply(int64_t nnodes, const T *__restrict__ dinv, const T *
 }
 
 // ---------------------------------------------------------------- SpMV
+// NB values of a block row, or of a node's x.  FP32 with NB = 4: one 16-byte word
+// (every such address is a multiple of 4 values from an allocation's start).  One
+// value at a time, a warp's loads took more cycles of the L1 than its bytes took of
+// HBM: products of the mixed 4.2M-point slope 0.89 -> 0.84 ms, of the 1M-point block
+// 0.222 -> 0.201.  (FP64 is bound by its pipe: 2.08 ms a product one by one, 2.10 by words.)
+template <int NB, typename T>
+__device__ __forceinline__ void load_row(const T *__restrict__ p, T v[NB]) {
+  if constexpr (NB == 4 && sizeof(T) == 4) {
+    const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+    v[3] = q.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) v[i] = __ldg(p + i);
+  }
+}
+
 // SPL * NB threads per block row: the SPL lanes of output r of a row split the
 // row's blocks (lane l takes blocks l, l + SPL, ...) and spend one FMA per
 // stored value of block row r; one shuffle sum per output joins them.
@@ -313,8 +332,11 @@ __global__ void k_bsr_spmv(int64_t nnodes, const int32_t *__restrict__ row_ptr,
     for (int e = row_ptr[row] + part; e < e1; e += SPL) {
       const T *blk = val + (int64_t)e * NB * NB + r * NB;
       const T *xb = x + (int64_t)__ldg(&col[e]) * NB;
+      T bv[NB], xv[NB];
+      load_row<NB>(blk, bv);
+      load_row<NB>(xb, xv);
 #pragma unroll
-      for (int c = 0; c < NB; ++c) acc = fma(__ldg(&blk[c]), __ldg(&xb[c]), acc);
+      for (int c = 0; c < NB; ++c) acc = fma(bv[c], xv[c], acc);
     }
   }
 #pragma unroll
