@@ -337,11 +337,18 @@ __global__ void k_renorm(GridP g, DevView v) {
 }
 
 // ---------------------------------------------------------------- points
+// The walk over the support boxes takes a block's points in the order of
+// point_by_extent and hands its sums over in shared memory, so that everything
+// else, the records' stores above all, stays in the points' own order.
 template <int D, bool DYN>
-__global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restrict__ X) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__host__ __device__ constexpr int point_block() { return D == 3 && DYN ? 128 : 256; }
+template <int D, bool DYN>
+__global__ void __launch_bounds__(256) k_point_eval(GridP g, StepP s, DevView v, const double *__restrict__ X) {
+  constexpr int TP = point_block<D, DYN>();
+  constexpr int NF = D * D + D + 2 + (DYN ? D * D + 3 * D : 0);
+  __shared__ double sums[NF][TP];
+  const int64_t p0 = blockIdx.x * (int64_t)TP, p = p0 + threadIdx.x;
   const int64_t n = v.n;
-  if (p >= n) return;
   constexpr int NB = D + 1;
   const int64_t nn = g.nnodes;
   const double dt = s.dt, b = s.beta, gm = s.gamma;
@@ -355,7 +362,8 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
   double vh[3] = {0, 0, 0}, uh[3] = {0, 0, 0};
   double ph = 0.0, pdev = 0.0;
   const double cvu = gm / (b * dt), cvv = 1.0 - gm / b, cva = (1.0 - gm / (2.0 * b)) * dt;
-  for_box_nodes<D>(g, v, p, [&](int64_t a, double Sa, double S0a, const double Gn[3]) {
+  const int walk = point_by_extent<D, TP>(v, p0);
+  if (p0 + walk < n) for_box_nodes<D>(g, v, p0 + walk, [&](int64_t a, double Sa, double S0a, const double Gn[3]) {
     const double P = X[a * NB + D], dP = P - v.Pn[a];
     for (int i = 0; i < D; ++i) {
       const double dU = X[a * NB + i];
@@ -374,6 +382,25 @@ __global__ void k_point_eval(GridP g, StepP s, DevView v, const double *__restri
     if (DYN) pdev = fma(Sa - S0a, fma(cvu, dP, fma(cvv, v.pdn[a], cva * v.pddn[a])), pdev);
     else pdev = fma(Sa - S0a, dP, pdev);
   });
+  {
+    auto each = [&](auto &&f) {
+      int o = 0;
+      for (int i = 0; i < D * D; ++i) f(o++, dF[i]);
+      for (int i = 0; i < D; ++i) f(o++, gPn[i]);
+      f(o++, ph);
+      f(o++, pdev);
+      if (DYN) {
+        for (int i = 0; i < D * D; ++i) f(o++, gVn[i]);
+        for (int i = 0; i < D; ++i) f(o++, ah[i]);
+        for (int i = 0; i < D; ++i) f(o++, vh[i]);
+        for (int i = 0; i < D; ++i) f(o++, uh[i]);
+      }
+    };
+    each([&](int o, double &x) { sums[o][walk] = x; });
+    __syncthreads();
+    if (p >= n) return;
+    each([&](int o, double &x) { x = sums[o][threadIdx.x]; });
+  }
   if (DYN) {  // acceleration and velocity gradient (Eq. newmark) at the point
     for (int i = 0; i < D; ++i) {
       ah[i] = uh[i] / (b * dt * dt) - vh[i] / (b * dt) + (1.0 - 1.0 / (2.0 * b)) * ah[i];
@@ -2214,14 +2241,10 @@ void run_renorm(Ctx &c) {
 void run_point_eval(Ctx &c, const double *X) {
   prof_begin(c, MPM_PROF_POINT);
   const DevView v = c.view();
-  const int nbk = nblk(c.n);
-  if (c.d == 2) {
-    if (c.dyn) k_point_eval<2, true><<<nbk, TPB, 0, c.st>>>(c.g, c.s, v, X);
-    else k_point_eval<2, false><<<nbk, TPB, 0, c.st>>>(c.g, c.s, v, X);
-  } else {
-    if (c.dyn) k_point_eval<3, true><<<nbk, TPB, 0, c.st>>>(c.g, c.s, v, X);
-    else k_point_eval<3, false><<<nbk, TPB, 0, c.st>>>(c.g, c.s, v, X);
-  }
+#define POINTS(D, Y) k_point_eval<D, Y><<<nblk(c.n, point_block<D, Y>()), point_block<D, Y>(), 0, c.st>>>(c.g, c.s, v, X)
+  if (c.d == 2) { if (c.dyn) POINTS(2, true); else POINTS(2, false); }
+  else { if (c.dyn) POINTS(3, true); else POINTS(3, false); }
+#undef POINTS
   UPMPM_LAUNCH(c);
   prof_end(c, MPM_PROF_POINT);
 }

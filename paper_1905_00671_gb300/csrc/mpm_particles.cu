@@ -369,17 +369,20 @@ __device__ inline void stretch_diag(const double *F, double *Ud) {
 
 template <int D, bool DYN>
 __global__ void k_g2p(GridP g, StepP s, DevView v, const double *__restrict__ X) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  constexpr int NF = D * D + D + 1 + (DYN ? 2 * D + 3 : 0);
+  __shared__ double sums[NF][TPB];
+  const int64_t p0 = blockIdx.x * (int64_t)TPB, p = p0 + threadIdx.x;
   const int64_t n = v.n;
-  if (p >= n) return;
   constexpr int NB = D + 1;
   const int64_t nn = g.nnodes;
-  // sums over the support box; the nodal accelerations and rates are linear in
-  // nodal values, which are summed first (as in k_point_eval)
+  // sums over the support box, in the order of point_by_extent; the nodal
+  // accelerations and rates are linear in nodal values, which are summed first (as
+  // in k_point_eval)
   double dF[9] = {0}, du[3] = {0, 0, 0}, ph = 0.0;  // dF - 1 until after the loop
   double vh[3] = {0, 0, 0}, ah[3] = {0, 0, 0}, dph = 0.0, pdh = 0.0, pddh = 0.0;
   const double b = s.beta, gm = s.gamma, dt = s.dt;
-  for_box_nodes<D>(g, v, p, [&](int64_t a, double Sa, double, const double Gn[3]) {
+  const int walk = point_by_extent<D, TPB>(v, p0);
+  if (p0 + walk < n) for_box_nodes<D>(g, v, p0 + walk, [&](int64_t a, double Sa, double, const double Gn[3]) {
     for (int i = 0; i < D; ++i) {
       const double dU = X[a * NB + i];
       du[i] = fma(Sa, dU, du[i]);
@@ -397,6 +400,25 @@ __global__ void k_g2p(GridP g, StepP s, DevView v, const double *__restrict__ X)
       pddh = fma(Sa, v.pddn[a], pddh);
     }
   });
+  {
+    auto each = [&](auto &&f) {
+      int o = 0;
+      for (int i = 0; i < D * D; ++i) f(o++, dF[i]);
+      for (int i = 0; i < D; ++i) f(o++, du[i]);
+      f(o++, ph);
+      if (DYN) {
+        for (int i = 0; i < D; ++i) f(o++, vh[i]);
+        for (int i = 0; i < D; ++i) f(o++, ah[i]);
+        f(o++, dph);
+        f(o++, pdh);
+        f(o++, pddh);
+      }
+    };
+    each([&](int o, double &x) { sums[o][walk] = x; });
+    __syncthreads();
+    if (p >= n) return;
+    each([&](int o, double &x) { x = sums[o][threadIdx.x]; });
+  }
   double anew[3] = {0, 0, 0}, vinc[3] = {0, 0, 0};
   if (DYN) {
     for (int i = 0; i < D; ++i) {
