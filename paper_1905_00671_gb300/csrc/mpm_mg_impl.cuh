@@ -880,45 +880,208 @@ __global__ void k_mg_restrict(LevelDev F, LevelDev Cl, const real *__restrict__ 
 
 // (P x_c)(a) at fine node a from its 2^d candidate coarse parents: per axis
 // I = a/2 (weight 1 if a is even, 1/2 if odd) and I + 1 (weight 1/2 if a is
-// odd and I + 1 exists, else 0, with its index clamped), so all loads are
-// issued without branches.
-template <int B, int D>
-__device__ inline void prolong_at(const LevelDev &Cl, const real *__restrict__ xc, const int ac[3],
-                                  int inst_a, real out[B]) {
-  int i0[3], i1[3];
-  real w0[3], w1[3];
-  for (int k = 0; k < 3; ++k) {
-    const int odd = ac[k] & 1;
-    i0[k] = ac[k] >> 1;
-    const bool up = odd && i0[k] + 1 < Cl.nn[k];
-    i1[k] = up ? i0[k] + 1 : i0[k];
-    w0[k] = odd ? 0.5 : 1.0;
-    w1[k] = up ? 0.5 : 0.0;
+// odd and I + 1 exists, else 0, with its index clamped).  Components i0 .. i0 + NE - 1,
+// the loads (prolong_load) apart from the sum, so that a caller can issue other loads
+// between them.
+template <int D>
+__device__ inline int64_t prolong_parent(const LevelDev &Cl, const int ac[3], int cmb, real &wgt) {
+  int64_t I = 0, stride = 1;
+  wgt = 1;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const int odd = ac[k] & 1, i0 = ac[k] >> 1;
+    const bool up = odd && i0 + 1 < Cl.nn[k], far = (cmb >> k) & 1;
+    I += stride * (far && up ? i0 + 1 : i0);
+    stride *= Cl.nn[k];
+    wgt = far ? (up ? wgt * real(0.5) : real(0)) : (odd ? wgt * real(0.5) : wgt);
   }
-  for (int i = 0; i < B; ++i) out[i] = 0.0;
+  return I;
+}
+template <int B, int NE, int D>
+__device__ inline void prolong_load(const LevelDev &Cl, const real *__restrict__ xc, const int ac[3], int i0,
+                                    real pv[1 << D][NE]) {
 #pragma unroll
   for (int cmb = 0; cmb < (1 << D); ++cmb) {
-    const int s0 = cmb & 1, s1 = (cmb >> 1) & 1, s2 = (cmb >> 2) & 1;
-    const real wgt = (s0 ? w1[0] : w0[0]) * (s1 ? w1[1] : w0[1]) * (D == 3 ? (s2 ? w1[2] : w0[2]) : 1.0);
-    const int64_t I = (s0 ? i1[0] : i0[0]) +
-                      (int64_t)Cl.nn[0] * ((s1 ? i1[1] : i0[1]) + (int64_t)Cl.nn[1] * (D == 3 ? (s2 ? i1[2] : i0[2]) : 0));
-    const real w = (!Cl.inst || Cl.inst[I] == inst_a) ? wgt : real(0);
-    for (int i = 0; i < B; ++i) out[i] = fma(w, xc[I * B + i], out[i]);
+    real wgt;
+    const int64_t I = prolong_parent<D>(Cl, ac, cmb, wgt);
+#pragma unroll
+    for (int i = 0; i < NE; ++i) pv[cmb][i] = xc[I * B + i0 + i];
+  }
+}
+template <int NE, int D>
+__device__ inline void prolong_sum(const LevelDev &Cl, const int ac[3], int inst_a, const real pv[1 << D][NE],
+                                   real out[NE]) {
+#pragma unroll
+  for (int i = 0; i < NE; ++i) out[i] = 0;
+#pragma unroll
+  for (int cmb = 0; cmb < (1 << D); ++cmb) {
+    real w;
+    const int64_t I = prolong_parent<D>(Cl, ac, cmb, w);
+    if (Cl.inst && Cl.inst[I] != inst_a) w = 0;
+#pragma unroll
+    for (int i = 0; i < NE; ++i) out[i] = fma(w, pv[cmb][i], out[i]);
   }
 }
 
-// x_f(a) += sum_I P_aI x_c(I)
-template <int B, int D>
-__global__ void k_mg_prolong(LevelDev F, LevelDev Cl, real *__restrict__ xf,
-                             const real *__restrict__ xc) {
+// Window of coarse nodes that a fine row reaches: floor(a / 2) + WIN0 .. + WIN0 + W - 1
+// per axis, W = 3, 4 or 5 for couplings up to 1, 2 or 3 nodes apart.  The Galerkin
+// product keeps a reach of 1 at 1, and brings 2 and 3 to 2.
+template <int W>
+constexpr int WIN0 = W == 5 ? -2 : -1;
+// whether a row of that parity reaches slot d of its window
+template <int W>
+__device__ __forceinline__ bool win_reaches(int a, int d) {
+  return W == 3 ? !(d == -1 && (a & 1)) : W == 4 ? !(d == 2 && !(a & 1)) : true;
+}
+
+// A fine row that contributes nothing to the Galerkin product: a stencil row
+// without coupling, or a finest-level row whose DOFs are all fixed (its
+// transfers are masked).  On levels of VOID_ROWS rows and more k_mg_ap leaves such a
+// row's T unwritten and its readers skip the row (on the slope, the grid nodes
+// outside the material); on smaller ones it writes zeros, so that k_mg_post need not
+// wait for the test before it loads.
+constexpr int64_t VOID_ROWS = 1 << 16;
+template <int B, bool FST>
+__device__ inline bool row_void(const LevelDev &F, int64_t a) {
+  if (FST) return F.nslot[a] == 0;
+  if (!F.fixed) return false;
+  for (int i = 0; i < B; ++i)
+    if (!F.fixed[a * F.mstride + F.moff + i]) return false;
+  return true;
+}
+
+// A level's rows are split into parts until it has POST_THREADS threads: about three
+// warps for each of the chip's 608 SM quarters, so that their FP64 pipes share the work.
+constexpr int64_t POST_THREADS = 1 << 16;
+constexpr int POST_WARPS = 16;  // warps of a block at most
+
+// Coarse correction and first post-smoothing sweep in one pass.  With r = b - A x
+// from before the restriction and T = A P from the set-up,
+//   x + P e + omega Dinv (b - A (x + P e)) = x + P e + omega Dinv (r - T e):
+// a row of T holds at most 3 (even) or 4 (odd) coarse nodes per axis, 43 blocks on
+// average in 3D, where a row of A holds about 110 (125 on a coarse level), and
+// neither the neighbours' x nor a prolongation kernel is needed.
+// A lane per row, 32 consecutive rows a warp (T is stored by rows, so every load
+// of it is one line).  Where a level has few rows (SPLIT), `parts` warps share the
+// rows' (z, y) window lines; their sums are joined in a tree and the rows finished a
+// component a warp, since a warp's FP64 instruction holds its SM quarter's pipe for
+// 64 cycles and what a small level costs is its longest warp.  What the row's end
+// reads is then loaded before T (its use would hold up T's loads), and in FP32; on
+// large FP64 levels, bound by the pipe (90% busy), the registers cost more than that
+// gives (slope: 217 against 261 ms a step).  Where the pipe is not the bound, the loads
+// of a window line go out together (finest FP32 level of a 110k-node block: 175 us with
+// the compiler's order, 77 warps stalled on loads per issue).
+// Preconditioner per step, against a prolongation kernel and a sweep over A (GB300):
+// 4.2M-point slope 271 -> 209 ms, mixed 141 -> 113; 163k-point block 18.6 -> 16.7, 1M-point
+// block mixed 22.9 -> 18.7; 80k-point footing 5.5 -> 5.1; steps of 64 batched columns
+// 53 -> 48 ms.  On the smallest level it serves (1,681 nodes) it costs what the two
+// kernels did.
+template <int B, int D, bool FST, int W, bool SPLIT>
+__global__ void k_mg_post(LevelDev F, LevelDev Cl, const real *__restrict__ T, const real *__restrict__ x,
+                          const real *__restrict__ e, const real *__restrict__ r, real *__restrict__ out,
+                          real omega, int parts) {
   pdl_enter();
-  const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (a >= F.nnodes) return;
-  int ac[3];
-  grid_xyz(F.nn[0], F.nn[1], (int)a, ac);
-  real acc[B];
-  prolong_at<B, D>(Cl, xc, ac, F.inst ? F.inst[a] : 0, acc);
-  for (int i = 0; i < B; ++i) xf[a * B + i] += free_w(F, a, i) * acc[i];
+  __shared__ real sm[SPLIT ? POST_WARPS : 1][B][32];
+  constexpr bool EARLY = SPLIT || sizeof(real) == sizeof(float);
+  constexpr int NE = SPLIT ? 1 : B;  // components a lane finishes
+  constexpr int BATCH = EARLY ? W : 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int part = SPLIT ? wid % parts : 0, grp = SPLIT ? wid / parts : wid;
+  const int64_t a = ((int64_t)blockIdx.x * ((blockDim.x >> 5) / (SPLIT ? parts : 1)) + grp) * 32 + lane;
+  const bool valid = a < F.nnodes;
+  const bool ends = valid && (!SPLIT || part < B);
+  const int i0 = SPLIT ? part : 0;
+  real te[B], rv[B], xv[NE], di[NE * B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) te[i] = 0;
+  int ac[3] = {0, 0, 0};
+  bool live = valid;  // T holds the row
+  real pv[1 << D][NE];
+  bool fx[NE];
+  auto load_end = [&]() {  // loads alone: a use of one would hold up those after it
+    prolong_load<B, NE, D>(Cl, e, ac, i0, pv);
+#pragma unroll
+    for (int j = 0; j < B; ++j) rv[j] = r[a * B + j];
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+      xv[i] = x[a * B + i0 + i];
+      fx[i] = F.fixed && F.fixed[a * F.mstride + F.moff + i0 + i];
+#pragma unroll
+      for (int j = 0; j < B; ++j) di[i * B + j] = F.dinv[a * B * B + (i0 + i) * B + j];
+    }
+  };
+  auto sum_end = [&]() {
+    real pe[NE];
+    prolong_sum<NE, D>(Cl, ac, F.inst ? F.inst[a] : 0, pv, pe);
+#pragma unroll
+    for (int i = 0; i < NE; ++i) xv[i] += fx[i] ? real(0) : pe[i];
+  };
+  if (valid) {
+    grid_xyz(F.nn[0], F.nn[1], (int)a, ac);
+    if (F.nnodes >= VOID_ROWS) live = !row_void<B, FST>(F, a);
+    if (EARLY && ends) {
+      load_end();
+      if (!SPLIT) sum_end();
+    }
+  }
+  if (live) {
+    constexpr int NL = D == 2 ? W : W * W;
+    for (int l = part; l < NL; l += SPLIT ? parts : 1) {
+      const int d1 = l % W + WIN0<W>, d2 = D == 3 ? l / W + WIN0<W> : 0;
+      if (!win_reaches<W>(ac[1], d1) || (D == 3 && !win_reaches<W>(ac[2], d2))) continue;
+      const int j1 = (ac[1] >> 1) + d1, j2 = D == 3 ? (ac[2] >> 1) + d2 : 0;
+      if (j1 < 0 || j1 >= Cl.nn[1] || j2 < 0 || j2 >= Cl.nn[2]) continue;
+      const int64_t jrow = (int64_t)Cl.nn[0] * (j1 + (int64_t)Cl.nn[1] * j2);
+      const real *t0 = T + (int64_t)(l * W) * (B * B) * F.nnodes + a;
+#pragma unroll
+      for (int q = 0; q < W; q += BATCH) {
+        real tv[BATCH][B * B], ev[BATCH][B];  // the loads of a batch go out together
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+          const int j0 = (ac[0] >> 1) + q + u + WIN0<W>;
+          const bool in = j0 >= 0 && j0 < Cl.nn[0];
+          const real *ej = e + (jrow + (in ? j0 : 0)) * B;
+#pragma unroll
+          for (int k = 0; k < B * B; ++k) tv[u][k] = __ldg(t0 + (int64_t)((q + u) * B * B + k) * F.nnodes);
+#pragma unroll
+          for (int j = 0; j < B; ++j) {
+            const real v = __ldg(ej + j);
+            ev[u][j] = in ? v : real(0);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u)
+#pragma unroll
+          for (int i = 0; i < B; ++i)
+#pragma unroll
+            for (int j = 0; j < B; ++j) te[i] = fma(tv[u][i * B + j], ev[u][j], te[i]);
+      }
+    }
+  }
+  if constexpr (SPLIT) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) sm[wid][i][lane] = te[i];
+    __syncthreads();
+    for (int h = parts / 2; h >= 2; h /= 2) {
+      if (part < h)
+#pragma unroll
+        for (int i = 0; i < B; ++i) sm[wid][i][lane] = te[i] = te[i] + sm[wid + h][i][lane];
+      __syncthreads();
+    }
+    if (ends)
+#pragma unroll
+      for (int i = 0; i < B; ++i) te[i] = sm[wid - part][i][lane] + sm[wid - part + 1][i][lane];
+  }
+  if (!ends) return;
+  if (!EARLY) load_end();
+  if (!EARLY || SPLIT) sum_end();
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    real s = 0;
+#pragma unroll
+    for (int j = 0; j < B; ++j) s = fma(di[i * B + j], rv[j] - te[j], s);
+    out[a * B + i0 + i] = fma(omega, s, xv[i]);
+  }
 }
 
 // ---- coarse tail of a V-cycle as one dense operator
@@ -1167,9 +1330,9 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail_build(TailArgs A, Tail
 // Galerkin product P^T A P in two passes, from the block-CSR finest level
 // (couplings up to 3 apart per axis) or a stencil level (up to 2 apart):
 //   k_mg_ap:   T_a(J) = sum_b w_bJ A_ab over the children b of J, for every
-//              fine row a and coarse node J of the 5^d window centred on
-//              floor(a / 2) (the coarse nodes a row can reach); thread per
-//              (window slot, a), T stored slot-major;
+//              fine row a and coarse node J of the W^d window of the coarse
+//              nodes a row can reach (WIN0); thread per (window slot, a).  T is
+//              kept: k_mg_post applies it;
 //   k_mg_rap2: A_c(I, J) = sum_a w_aI T_a(J) over the 3^d children a of I;
 //              thread per (stencil slot, I).
 // Dirichlet DOFs are masked out of the finest level's transfers only, and
@@ -1177,25 +1340,12 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail_build(TailArgs A, Tail
 // entry costs a few lookups and 3^d FMA blocks instead of one per (a, b) pair
 // (measured on the slope's stencil levels: the one-pass product took 20 ms
 // per set-up).
-// A fine row that contributes nothing to the Galerkin product: a stencil row
-// without coupling, or a finest-level row whose DOFs are all fixed (its
-// transfers are masked).  k_mg_ap leaves such a row's T unwritten and
-// k_mg_rap2 skips it (on the slope, the grid nodes outside the material).
-template <int B, bool FST>
-__device__ inline bool row_void(const LevelDev &F, int64_t a) {
-  if (FST) return F.nslot[a] == 0;
-  if (!F.fixed) return false;
-  for (int i = 0; i < B; ++i)
-    if (!F.fixed[a * F.mstride + F.moff + i]) return false;
-  return true;
-}
-
-template <int B, int D, bool FST>
+template <int B, int D, bool FST, int W>
 __global__ void k_mg_ap(LevelDev F, LevelDev Cl, real *__restrict__ T) {
-  constexpr int NS = NS_<D>::v;
+  constexpr int NS = D == 2 ? W * W : W * W * W;  // window slots
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   // the lanes of a warp take one window slot of consecutive fine rows (the same
-  // loop bounds up to the parity of a), and T is stored slot-major ([s][a]) so
+  // loop bounds up to the parity of a), and T is stored [slot][value][row] so
   // that their results are written side by side; a tile of AP_ROWS rows takes all
   // its slots before the next one, so that the row's blocks are read from DRAM
   // once and not once per slot that reaches them (the set-up class of the
@@ -1206,15 +1356,16 @@ __global__ void k_mg_ap(LevelDev F, LevelDev Cl, real *__restrict__ T) {
   const int64_t a = tile * AP_ROWS + rem % AP_ROWS;
   const int s = rem / AP_ROWS;
   if (a >= F.nnodes) return;
-  if (row_void<B, FST>(F, a)) return;
+  const bool none = row_void<B, FST>(F, a);
+  if (none && F.nnodes >= VOID_ROWS) return;
   int fa[3], Jc[3];
   grid_xyz(F.nn[0], F.nn[1], (int)a, fa);
-  Jc[0] = (fa[0] >> 1) + s % 5 - 2;
-  Jc[1] = (fa[1] >> 1) + (s / 5) % 5 - 2;
-  Jc[2] = D == 3 ? (fa[2] >> 1) + s / 25 - 2 : 0;
+  Jc[0] = (fa[0] >> 1) + s % W + WIN0<W>;
+  Jc[1] = (fa[1] >> 1) + (s / W) % W + WIN0<W>;
+  Jc[2] = D == 3 ? (fa[2] >> 1) + s / (W * W) + WIN0<W> : 0;
   real acc[B * B];
   for (int i = 0; i < B * B; ++i) acc[i] = 0.0;
-  if (Jc[0] >= 0 && Jc[0] < Cl.nn[0] && Jc[1] >= 0 && Jc[1] < Cl.nn[1] && Jc[2] >= 0 && Jc[2] < Cl.nn[2]) {
+  if (!none && Jc[0] >= 0 && Jc[0] < Cl.nn[0] && Jc[1] >= 0 && Jc[1] < Cl.nn[1] && Jc[2] >= 0 && Jc[2] < Cl.nn[2]) {
     const int64_t Jn = Jc[0] + (int64_t)Cl.nn[0] * (Jc[1] + (int64_t)Cl.nn[1] * Jc[2]);
     int blo[3], bhi[3];  // children of J within reach of a (and inside the grid)
     for (int k = 0; k < 3; ++k) {
@@ -1237,7 +1388,7 @@ __global__ void k_mg_ap(LevelDev F, LevelDev Cl, real *__restrict__ T) {
           } else {     // stencil level: the 5^d slot of b - a
             const int d0 = b0 - fa[0], d1 = b1 - fa[1], d2 = b2 - fa[2];
             if (d0 < -2 || d0 > 2 || d1 < -2 || d1 > 2 || d2 < -2 || d2 > 2) continue;
-            blk = F.sval + (a * NS + (d0 + 2) + 5 * (d1 + 2) + (D == 3 ? 25 * (d2 + 2) : 0)) * B * B;
+            blk = F.sval + (a * NS_<D>::v + (d0 + 2) + 5 * (d1 + 2) + (D == 3 ? 25 * (d2 + 2) : 0)) * B * B;
           }
           const real w = pw(b0, Jc[0]) * pw(b1, Jc[1]) * (D == 3 ? pw(b2, Jc[2]) : 1.0);
           for (int j = 0; j < B; ++j) {
@@ -1246,10 +1397,10 @@ __global__ void k_mg_ap(LevelDev F, LevelDev Cl, real *__restrict__ T) {
           }
         }
   }
-  for (int i = 0; i < B * B; ++i) T[((int64_t)s * F.nnodes + a) * B * B + i] = acc[i];
+  for (int i = 0; i < B * B; ++i) T[((int64_t)s * (B * B) + i) * F.nnodes + a] = acc[i];
 }
 
-template <int B, int D, bool FST>
+template <int B, int D, bool FST, int W>
 __global__ void k_mg_rap2(LevelDev F, LevelDev Cl, const real *__restrict__ T) {
   constexpr int NS = NS_<D>::v;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1278,7 +1429,8 @@ __global__ void k_mg_rap2(LevelDev F, LevelDev Cl, const real *__restrict__ T) {
             continue;
           // slot of J in a's window; outside it, T_a(J) is zero (J out of reach)
           const int d0 = Jc[0] - (fa[0] >> 1), d1 = Jc[1] - (fa[1] >> 1), d2 = D == 3 ? Jc[2] - (fa[2] >> 1) : 0;
-          if (d0 < -2 || d0 > 2 || d1 < -2 || d1 > 2 || d2 < -2 || d2 > 2) continue;
+          constexpr int lo = WIN0<W>, hi = lo + W - 1;
+          if (d0 < lo || d0 > hi || d1 < lo || d1 > hi || (D == 3 && (d2 < lo || d2 > hi))) continue;
           const int64_t a = fa[0] + (int64_t)F.nn[0] * (fa[1] + (int64_t)F.nn[1] * fa[2]);
           if (F.inst && F.inst[a] != Cl.inst[I]) continue;
           const real wa = pw(fa[0], Ic[0]) * pw(fa[1], Ic[1]) * (D == 3 ? pw(fa[2], Ic[2]) : 1.0);
@@ -1290,10 +1442,11 @@ __global__ void k_mg_rap2(LevelDev F, LevelDev Cl, const real *__restrict__ T) {
           }
           // a row without contribution (row_void): T_a was not written
           if (FST ? F.nslot[a] == 0 : !any) continue;
-          const int sl = (d0 + 2) + 5 * (d1 + 2) + (D == 3 ? 25 * (d2 + 2) : 0);
-          const real *ta = T + ((int64_t)sl * F.nnodes + a) * B * B;
+          const int sl = (d0 - lo) + W * (d1 - lo) + (D == 3 ? W * W * (d2 - lo) : 0);
+          const real *ta = T + (int64_t)sl * (B * B) * F.nnodes + a;
           for (int i = 0; i < B; ++i)
-            for (int j = 0; j < B; ++j) acc[i * B + j] = fma(wi[i], ta[i * B + j], acc[i * B + j]);
+            for (int j = 0; j < B; ++j)
+              acc[i * B + j] = fma(wi[i], ta[(int64_t)(i * B + j) * F.nnodes], acc[i * B + j]);
         }
   }
   for (int i = 0; i < B * B; ++i) Cl.sval[(I * NS + s) * B * B + i] = acc[i];
@@ -1333,13 +1486,23 @@ struct MGHier<MG_REAL> {
   // dense coarsest operator (LU factors after set-up), its inverse, the factors' transpose
   MG_REAL *Ad = nullptr, *Ai = nullptr, *At = nullptr;
   int *piv = nullptr;                    // row interchanges of the LU factorisation
-  MG_REAL *apT = nullptr;                // finest level x 5^d window: A P, first pass of a level's product
+  MG_REAL *ap[16] = {};                  // A P of a level and the next one, on its window (k_mg_ap)
+  int win = 4, cwin = 4;                 // windows of the finest level and of the coarse levels
+  bool ap_wide = false;                  // ap[0] has room for a window of 5
   int ncoarse = 0;                       // unknowns of the coarsest level
   int tail = 15;                         // first level of the dense tail (nlev - 1: the coarsest alone)
   MG_REAL *T = nullptr;                  // its operator
 };
 
 namespace MG_NS {
+
+// f(W) with the compile-time window
+template <typename F>
+inline void with_window(int win, F &&f) {
+  if (win == 3) f(std::integral_constant<int, 3>{});
+  else if (win == 5) f(std::integral_constant<int, 5>{});
+  else f(std::integral_constant<int, 4>{});
+}
 
 template <int B, int D>
 void mg_setup_t(Ctx &c, MGHier<real> &H) {
@@ -1349,16 +1512,18 @@ void mg_setup_t(Ctx &c, MGHier<real> &H) {
     if (l > 0) {
       constexpr int NS = NS_<D>::v;
       const int g2 = nblk(ap_threads(L.nnodes, NS));
-      // two passes, P^T (A P), on every level (the intermediate of the finest
-      // level is the largest): on the stencil levels a few lookups and 3^d
-      // FMA blocks per coarse entry instead of 3^d x 3^d in one pass
-      if (l == 1) {
-        k_mg_ap<B, D, false><<<nblk(ap_threads(H.L[0].nnodes, NS)), TPB, 0, c.st>>>(H.L[0], L, H.apT);
-        k_mg_rap2<B, D, false><<<g2, TPB, 0, c.st>>>(H.L[0], L, H.apT);
-      } else {
-        k_mg_ap<B, D, true><<<nblk(ap_threads(H.L[l - 1].nnodes, NS)), TPB, 0, c.st>>>(H.L[l - 1], L, H.apT);
-        k_mg_rap2<B, D, true><<<g2, TPB, 0, c.st>>>(H.L[l - 1], L, H.apT);
-      }
+      const int64_t nf = H.L[l - 1].nnodes;
+      real *T = H.ap[l - 1];
+      with_window(l == 1 ? H.win : H.cwin, [&](auto win) {
+        constexpr int W = decltype(win)::value, N = D == 2 ? W * W : W * W * W;
+        if (l == 1) {
+          k_mg_ap<B, D, false, W><<<nblk(ap_threads(nf, N)), TPB, 0, c.st>>>(H.L[0], L, T);
+          k_mg_rap2<B, D, false, W><<<g2, TPB, 0, c.st>>>(H.L[0], L, T);
+        } else if constexpr (W < 5) {
+          k_mg_ap<B, D, true, W><<<nblk(ap_threads(nf, N)), TPB, 0, c.st>>>(H.L[l - 1], L, T);
+          k_mg_rap2<B, D, true, W><<<g2, TPB, 0, c.st>>>(H.L[l - 1], L, T);
+        }
+      });
       k_mg_rowcount<B, D><<<nblk(L.nnodes * 32), TPB, 0, c.st>>>(L);
       UPMPM_LAUNCH(c);
       UPMPM_LAUNCH(c);
@@ -1482,7 +1647,7 @@ void vcycle_t(Ctx &c, MGHier<real> &H, int l) {
   LevelDev &L = H.L[l], &Ln = H.L[l + 1];
   real *xn_first = l + 1 == H.tail ? nullptr : H.x[l + 1];
   for (int k = 1; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // pre-smoothing after the first
-  const Geom gc = geom(c, (Ln.nnodes + restrict_nodes<B>() - 1) / restrict_nodes<B>() * 32), gf = geom(c, L.nnodes);
+  const Geom gc = geom(c, (Ln.nnodes + restrict_nodes<B>() - 1) / restrict_nodes<B>() * 32);
   if (l == 0 && B <= 2) {
     constexpr int SPL = B <= 2 ? 4 / B : 1;
     const Geom g0 = geom(c, L.nnodes * B * SPL);
@@ -1502,8 +1667,21 @@ void vcycle_t(Ctx &c, MGHier<real> &H, int l) {
   launch_pdl(c, k_mg_restrict<B, D>, gc.blocks, gc.tpb, 0, L, Ln, (const real *)H.r[l], H.b[l + 1], xn_first,
              mg_omega(c));
   vcycle_t<B, D>(c, H, l + 1);
-  launch_pdl(c, k_mg_prolong<B, D>, gf.blocks, gf.tpb, 0, L, Ln, H.x[l], (const real *)H.x[l + 1]);
-  for (int k = 0; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // post-smoothing sweeps
+  // coarse correction and first post-smoothing sweep
+  int parts = 1;
+  while (parts < (D == 2 ? 4 : 16) && L.nnodes * parts < POST_THREADS) parts *= parts == 1 ? D + D - 2 : 2;
+  const int warps = parts < 4 ? 4 : parts, rows = warps / parts * 32;
+  auto post = [&](auto kernel) {
+    launch_pdl(c, kernel, nblk(L.nnodes, rows), 32 * warps, 0, L, Ln, (const real *)H.ap[l], (const real *)H.x[l],
+               (const real *)H.x[l + 1], (const real *)H.r[l], H.x2[l], mg_omega(c), parts);
+  };
+  with_window(l == 0 ? H.win : H.cwin, [&](auto win) {
+    constexpr int W = decltype(win)::value;
+    if (l == 0) parts > 1 ? post(k_mg_post<B, D, false, W, true>) : post(k_mg_post<B, D, false, W, false>);
+    else if constexpr (W < 5) parts > 1 ? post(k_mg_post<B, D, true, W, true>) : post(k_mg_post<B, D, true, W, false>);
+  });
+  std::swap(H.x[l], H.x2[l]);
+  for (int k = 1; k < c.mg_sweeps(); ++k) sweep<B, D>(c, H, l);  // post-smoothing sweeps after it
 }
 
 // Allocate a hierarchy for block size B over the grid's node lattice; level 0
@@ -1585,7 +1763,8 @@ int mg_alloc(Ctx &c, MGHier<real> &H, int B) {
     const int64_t n = H.L[H.tail].nnodes * B;
     if (cudaMalloc(&H.T, sizeof(real) * n * n)) return MPM_ERR_NO_MEMORY;
   }
-  if (H.nlev > 1 && cudaMalloc(&H.apT, sizeof(real) * H.L[0].nnodes * NS * B * B)) return MPM_ERR_NO_MEMORY;
+  for (int k = 0; k + 1 < H.nlev; ++k)
+    if (cudaMalloc(&H.ap[k], sizeof(real) * H.L[k].nnodes * (D == 2 ? 16 : 64) * B * B)) return MPM_ERR_NO_MEMORY;
   return MPM_OK;
 }
 
@@ -1594,9 +1773,12 @@ void mg_free(MGHier<real> &H) {
   cudaFree(H.Ai);
   cudaFree(H.At);
   cudaFree(H.piv);
-  cudaFree(H.apT);
+  for (real *&p : H.ap) {
+    cudaFree(p);
+    p = nullptr;
+  }
   cudaFree(H.T);
-  H.Ad = H.Ai = H.At = H.apT = H.T = nullptr;
+  H.Ad = H.Ai = H.At = H.T = nullptr;
   H.piv = nullptr;
   for (int l = 0; l < H.nlev; ++l) {
     cudaFree(const_cast<int32_t *>(H.L[l].inst));
@@ -1612,10 +1794,18 @@ void mg_free(MGHier<real> &H) {
   H.nlev = 0;
 }
 
-// The finest level's block-Jacobi inverses only: the coarse levels keep the
+// The finest level's block-Jacobi inverses and A P only: the coarse levels keep the
 // Galerkin product of an earlier set-up (mpm_options.precond_reuse).
 template <int B, int D>
 void mg_refresh_t(Ctx &c, MGHier<real> &H) {
+  if (H.nlev > 1) {
+    const int64_t nf = H.L[0].nnodes;
+    with_window(H.win, [&](auto win) {
+      constexpr int W = decltype(win)::value, N = D == 2 ? W * W : W * W * W;
+      k_mg_ap<B, D, false, W><<<nblk(ap_threads(nf, N)), TPB, 0, c.st>>>(H.L[0], H.L[1], H.ap[0]);
+    });
+    UPMPM_LAUNCH(c);
+  }
   k_mg_dinv<B, D, false><<<nblk(H.L[0].nnodes), TPB, 0, c.st>>>(H.L[0], c.err);
   UPMPM_LAUNCH(c);
 }
@@ -1711,6 +1901,31 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
     }
     S.sub_cap = cap;
   }
+  const bool full = coarse || !S.coarse_built;
+  // the window of A P from the step's largest support
+  int win = 3;
+  for (int k = 0; k < d; ++k) win = std::max(win, std::min(c.h_cmax[k], 4) + 1);
+  for (MGHier<real> *H : {S.mgA, S.mgS}) {
+    // (coarse levels kept from an earlier set-up keep their window)
+    const int cwin = !full ? H->cwin : win == 3 ? 3 : 4;
+    if (H->win != win || H->cwin != cwin) {  // the captured graphs hold the other window's kernels
+      if (S.gexec) cudaGraphExecDestroy(S.gexec);
+      if (S.itexec) cudaGraphExecDestroy(S.itexec);
+      S.gexec = S.itexec = nullptr;
+      H->win = win;
+      H->cwin = cwin;
+    }
+    if (win == 5 && !H->ap_wide && H->nlev > 1) {
+      cudaFree(H->ap[0]);
+      H->ap[0] = nullptr;
+      if (cudaMalloc(&H->ap[0], sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B)) {
+        cudaGetLastError();
+        c.last_error = "device allocation of the block preconditioner failed";
+        return MPM_ERR_NO_MEMORY;
+      }
+      H->ap_wide = true;
+    }
+  }
   // B1 serves the upper order's coupling update and the DIAG_A product, B2 the
   // lower order's
   const int64_t nsl = d == 2 ? 49 : 343;
@@ -1736,10 +1951,9 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
   };
   if (d == 2) setup_blocks(std::integral_constant<int, 2>{});
   else setup_blocks(std::integral_constant<int, 3>{});
-  // the coarse levels and the coarsest inverses: a new Galerkin product, or
-  // (coarse = false, after one exists) the product of an earlier set-up kept,
-  // the finest levels' values and block-Jacobi inverses refreshed
-  const bool full = coarse || !S.coarse_built;
+  // the coarse levels and the coarsest inverses: a new Galerkin product, or (not
+  // full) the product of an earlier set-up kept, the finest levels' values,
+  // block-Jacobi inverses and A P refreshed
   mg_setup(c, *S.mgA, c.row_ptr, c.col, S.Aval, 0, full);
   mg_setup(c, *S.mgS, c.row_ptr, c.col, S.Sval, d, full);
   if (full) {
