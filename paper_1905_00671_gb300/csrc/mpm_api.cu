@@ -529,11 +529,7 @@ void free_all(Ctx &c) {
                   c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i, c.bk_post, c.bn_nodes, c.bn_s0, c.bn_slices, c.bn_part, c.bn_npart};
   for (void *p : ptrs)
     if (p) cudaFree(p);
-  if (c.h_inorm) cudaFreeHost(c.h_inorm);
-  if (c.h_scalar) cudaFreeHost(c.h_scalar);
-  if (c.h_terms) cudaFreeHost(c.h_terms);
-  if (c.h_cmax) cudaFreeHost(c.h_cmax);
-  if (c.h_slot) cudaFreeHost(c.h_slot);
+  if (c.h_slot) cudaFreeHost(c.h_slot);  // with all other pinned words
   if (c.own_stream && c.st) cudaStreamDestroy(c.st);
   c.st = nullptr;
 }
@@ -777,16 +773,18 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   }
   if (!rc) rc = linsys_alloc<double>(c, c.L64, !c.have32);
   if (!rc && c.have32) rc = linsys_alloc<float>(c, c.L32, true);
-  if (!rc && (cudaHostAlloc((void **)&c.h_slot, SLOTS * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+  // all pinned words in one allocation (each took about 50 us of the creation)
+  if (!rc && (cudaHostAlloc((void **)&c.h_slot, sizeof(double) * (SLOTS + 12 + c.ninst), cudaHostAllocMapped) !=
+                  cudaSuccess ||
               cudaHostGetDevicePointer((void **)&c.d_slot, c.h_slot, 0) != cudaSuccess))
     rc = MPM_ERR_NO_MEMORY;
-  if (!rc && cudaHostAlloc((void **)&c.h_scalar, 8 * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
-    rc = MPM_ERR_NO_MEMORY;
-  if (!rc && (cudaMalloc((void **)&c.terms, 2 * sizeof(unsigned long long)) != cudaSuccess ||
-              cudaHostAlloc((void **)&c.h_cmax, 4 * sizeof(int), cudaHostAllocDefault) != cudaSuccess ||
-              cudaHostAlloc((void **)&c.h_terms, 2 * sizeof(unsigned long long), cudaHostAllocDefault) !=
-                  cudaSuccess))
-    rc = MPM_ERR_NO_MEMORY;
+  if (!rc) {
+    c.h_scalar = c.h_slot + SLOTS;
+    c.h_terms = reinterpret_cast<unsigned long long *>(c.h_scalar + 8);
+    c.h_cmax = reinterpret_cast<int *>(c.h_scalar + 10);
+    c.h_inorm = c.h_scalar + 12;
+  }
+  A(&c.terms, 2);
   A(&c.inst, c.ninst);
   A(&c.inorm, c.ninst);
   A(&c.node_inst, nn);
@@ -799,8 +797,6 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
     A(&c.bk_post, 1);
     if (!rc) cudaMemset(c.bk_post, 0, sizeof(BatchPost));
   }
-  if (!rc && cudaHostAlloc((void **)&c.h_inorm, sizeof(double) * c.ninst, cudaHostAllocDefault) != cudaSuccess)
-    rc = MPM_ERR_NO_MEMORY;
   if (rc) {
     free_all(c);
     return create_abort(h, rc, "device or pinned host memory allocation failed");
