@@ -1906,6 +1906,17 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
   int win = 3;
   for (int k = 0; k < d; ++k) win = std::max(win, std::min(c.h_cmax[k], 4) + 1);
   for (MGHier<real> *H : {S.mgA, S.mgS}) {
+    if (win == 5 && !H->ap_wide && H->nlev > 1) {
+      real *p = nullptr;  // (the narrower buffer stays if there is no room)
+      if (cudaMalloc(&p, sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B) != cudaSuccess) {
+        cudaGetLastError();
+        c.last_error = "device allocation of the block preconditioner failed";
+        return MPM_ERR_NO_MEMORY;
+      }
+      cudaFree(H->ap[0]);
+      H->ap[0] = p;
+      H->ap_wide = true;
+    }
     // (coarse levels kept from an earlier set-up keep their window)
     const int cwin = !full ? H->cwin : win == 3 ? 3 : 4;
     if (H->win != win || H->cwin != cwin) {  // the captured graphs hold the other window's kernels
@@ -1914,16 +1925,6 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
       S.gexec = S.itexec = nullptr;
       H->win = win;
       H->cwin = cwin;
-    }
-    if (win == 5 && !H->ap_wide && H->nlev > 1) {
-      cudaFree(H->ap[0]);
-      H->ap[0] = nullptr;
-      if (cudaMalloc(&H->ap[0], sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B)) {
-        cudaGetLastError();
-        c.last_error = "device allocation of the block preconditioner failed";
-        return MPM_ERR_NO_MEMORY;
-      }
-      H->ap_wide = true;
     }
   }
   // B1 serves the upper order's coupling update and the DIAG_A product, B2 the
