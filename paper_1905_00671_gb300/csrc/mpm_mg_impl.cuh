@@ -969,8 +969,8 @@ constexpr int POST_WARPS = 16;  // warps of a block at most
 // reads is then loaded before T (its use would hold up T's loads), and in FP32; on
 // large FP64 levels, bound by the pipe (90% busy), the registers cost more than that
 // gives (slope: 217 against 261 ms a step).  Where the pipe is not the bound, the loads
-// of a window line go out together (finest FP32 level of a 110k-node block: 175 us with
-// the compiler's order, 77 warps stalled on loads per issue).
+// of a window line go out together (finest FP32 level of a 110k-node block: 175 us in
+// the compiler's order, 48 so).
 // Preconditioner per step, against a prolongation kernel and a sweep over A (GB300):
 // 4.2M-point slope 271 -> 209 ms, mixed 141 -> 113; 163k-point block 18.6 -> 16.7, 1M-point
 // block mixed 22.9 -> 18.7; 80k-point footing 5.5 -> 5.1; steps of 64 batched columns
