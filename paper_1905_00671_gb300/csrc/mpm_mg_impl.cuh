@@ -1104,6 +1104,14 @@ constexpr int TAIL_MAX = 1024;
 constexpr int TAIL_COLS = 2;  // (4: one block per SM by its shared memory, 331 us for the 966 unknowns below)
 constexpr int TAIL_LEVELS = 8;
 constexpr int TAIL_THREADS = 512;
+// Shared memory of the largest tail: three vectors per level and column, under 2
+// TAIL_MAX unknowns over all levels (while a level is coarsened, every axis has
+// at least 3 nodes and keeps at most 2/3 of them, so a level has at most 4/9 of the
+// unknowns of the one before it).  The limit is set to this constant and not to a
+// tail's own size: it belongs to the kernel, which contexts of other host threads
+// launch at the same time.
+constexpr size_t TAIL_SMEM_MAX = sizeof(real) * 3 * TAIL_COLS * 2 * TAIL_MAX;
+static_assert(TAIL_SMEM_MAX <= 227 * 1024, "a tail's vectors fit a block's shared memory");
 
 struct TailArgs {
   int nl;  // levels of the tail, the last one the dense coarsest level
@@ -1584,13 +1592,12 @@ void tail_build_pair(Ctx &c, MGHier<real> &HA, MGHier<real> &HS, bool finest_onl
   const TailArgs A = args(HA, &smem), S = args(HS, &smem);
   const int na = nblk(A.n, TAIL_COLS), ns = nblk(S.n, TAIL_COLS);
   if (na + ns == 0) return;
-  if (c.d == 2) {
-    cudaFuncSetAttribute(k_mg_tail_build<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_mg_tail_build<2><<<na + ns, TAIL_THREADS, smem, c.st>>>(A, S, na);
-  } else {
-    cudaFuncSetAttribute(k_mg_tail_build<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_mg_tail_build<3><<<na + ns, TAIL_THREADS, smem, c.st>>>(A, S, na);
-  }
+  auto build = [&](auto kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX);
+    kernel<<<na + ns, TAIL_THREADS, smem, c.st>>>(A, S, na);
+  };
+  if (c.d == 2) build(k_mg_tail_build<2>);
+  else build(k_mg_tail_build<3>);
   UPMPM_LAUNCH(c);
 }
 
