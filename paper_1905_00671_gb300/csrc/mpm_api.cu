@@ -790,10 +790,9 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   A(&c.node_inst, nn);
   if (c.ninst > 1) {
     // batched FGMRES state per instance: H ((m+1) m), g, cs, sn (m+1 each), h1,
-    // h2 (PSTR each), target, residual; the column it is frozen at, columns,
-    // second-pass mark
+    // h2 (PSTR each), target, residual; the column it is frozen at, columns
     A(&c.bk, (int64_t)c.ninst * ((int64_t)(m + 1) * m + 3 * (m + 1) + 2 * 129 + 2));
-    A(&c.bk_i, 3 * (int64_t)c.ninst);
+    A(&c.bk_i, 2 * (int64_t)c.ninst);
     A(&c.bk_post, 1);
     if (!rc) cudaMemset(c.bk_post, 0, sizeof(BatchPost));
   }

@@ -94,7 +94,7 @@ struct KrylovCtl {
 };
 // Reports of a batched iteration's instances (mpm_solver.cu).
 struct BatchPost {
-  unsigned arrived, active, again;
+  unsigned arrived, active;
   unsigned long long ratio;  // bits of the largest estimate / target
 };
 

@@ -493,9 +493,11 @@ __global__ void k_update_x(T *__restrict__ x, const T *__restrict__ Z, const dou
 // one seen is far above the target (SPEC_MARGIN), so that the GPU does not wait
 // for it.  An iteration launched past convergence is not counted and leaves
 // the solution alone (it writes column j + 1 and later words only).
-// In FP64 the second Gram-Schmidt pass is rare (REORTH_THETA): the finishing
-// kernel then only raises ctl->halt, which stops what was launched ahead, and
-// the host launches the second pass.
+// In FP64 the second Gram-Schmidt pass of a single system depends on the first
+// (REORTH_THETA): where it is needed the finishing kernel leaves the column
+// unfinished and sets ctl->next.y.  Of an iteration launched ahead only the
+// preconditioner's core then runs, and what it overwrites the second pass's finish
+// writes anew.  The host launches that pass.  Batches take both passes always.
 // Against kernels launched one by one with a reduction kernel per pass and a
 // copy and stream synchronisation per iteration (GB300, whole steps): column 2.40 ->
 // 1.61 ms (25 iterations), 17 x 17 deposit in FP32 6.45 -> 4.52 (70), harmonic
@@ -508,7 +510,7 @@ constexpr double SPEC_MARGIN = 16.0;
 constexpr double EST_REORTH = -2.0;  // posted instead of an estimate: second pass needed
 constexpr int GS_SLICE = 512;        // vector elements per block of the inner products
 
-// part[b * PSTR + i] = block (b, .)'s part of V_i . w, i < cnt (= ctl->j + 1), and
+// part[b * PSTR + i] = block (b, .)'s part of V_i . w, i < cnt (= ctl->cur.x + 1), and
 // of w . w at i = cnt (with_norm): a warp per product and slice, all of them side
 // by side (the grid has blocks for m products; those past cnt leave at once)
 template <typename T>
@@ -825,9 +827,11 @@ double read_scalar(Ctx &c, const double *dptr) {
 // of 4,200 nodes and three passes an iteration.)  The iteration is a graph, as
 // for one instance; frozen_at holds the first column an instance skips, so that
 // the blocks of an instance agree on it while its first block moves it on.
-// Measured (GB300, 64 instances, whole steps): columns 74.8 -> 56.4 ms (95
-// iterations), footings 140 -> 120 ms (125); the Gram-Schmidt kernels then run at
-// the FP64 rate of their products.
+// Both passes of classical Gram-Schmidt run in every iteration, in FP64 as in FP32:
+// an instance's basis is as orthogonal as two passes leave it, whatever the others
+// need.  (With the second pass only where one instance's first had lost 99% of its
+// norm, a step of 64 columns took 53.3 ms against 59.2, of 64 footings 84.0 against
+// 88.2.)  The Gram-Schmidt kernels run at the FP64 rate of their products.
 constexpr int BG_NODES = 256;
 
 struct BatchK {  // device pointers of the batched solve, by value
@@ -835,7 +839,7 @@ struct BatchK {  // device pointers of the batched solve, by value
   const int32_t *nodes, *s0;  // node lists by slice; first slice of every instance (ni + 1)
   const int4 *slices;         // (instance or -1, start in nodes, count, -)
   double *H, *g, *cs, *sn, *h1, *h2, *tgt, *res;
-  int32_t *frozen_at, *jc, *again;
+  int32_t *frozen_at, *jc;
   double *part, *npart;
   BatchPost *post;
   KrylovCtl *ctl;
@@ -849,25 +853,24 @@ __device__ inline double slices_sum(const BatchK &K, int i, const double *__rest
   return block_sum(acc);
 }
 
-// An instance's first block reports (thread 0): whether it goes on, how far its
-// estimate is from its target, whether it needs a second pass; the last report
-// of the kernel posts the largest ratio (0: all done) and moves the control word
-__device__ inline void batch_report(const BatchK &K, int j, double *slot, bool active, double ratio, bool again) {
+// An instance's first block reports (thread 0): whether it goes on and how far
+// its estimate is from its target; the last report of the kernel posts the largest
+// ratio (0: all done) and moves the control word
+__device__ inline void batch_report(const BatchK &K, int j, double *slot, bool active, double ratio) {
   BatchPost *q = K.post;
   if (active) {
     atomicAdd(&q->active, 1u);
     atomicMax(&q->ratio, (unsigned long long)__double_as_longlong(ratio));
   }
-  if (again) atomicAdd(&q->again, 1u);
   __threadfence();
   if (atomicAdd(&q->arrived, 1u) != (unsigned)K.ni - 1) return;
   __threadfence();
-  const unsigned act = atomicAdd(&q->active, 0u), ag = atomicAdd(&q->again, 0u);
+  const unsigned act = atomicAdd(&q->active, 0u);
   const double worst = __longlong_as_double((long long)atomicMax(&q->ratio, 0ull));
-  q->active = q->again = q->arrived = 0;
+  q->active = q->arrived = 0;
   q->ratio = 0;
-  K.ctl->next = make_int2(ag ? j : j + 1, ag ? 1 : 0);
-  slot_write(slot, ag ? EST_REORTH : (act ? worst : 0.0));
+  K.ctl->next = make_int2(j + 1, 0);
+  slot_write(slot, act ? worst : 0.0);
 }
 
 template <int NB, typename T>
@@ -904,7 +907,7 @@ __global__ void k_bgs_start(BatchK K, const T *__restrict__ r, T *__restrict__ V
         g[0] = beta;
         K.jc[i] = 0;
         K.frozen_at[i] = done ? 0 : 0x7fffffff;
-        batch_report(K, -1, K.slot + SLOT_BETA, !done, beta / tgt, false);
+        batch_report(K, -1, K.slot + SLOT_BETA, !done, beta / tgt);
       }
     }
   }
@@ -914,16 +917,14 @@ __global__ void k_bgs_start(BatchK K, const T *__restrict__ r, T *__restrict__ V
 
 // products of a slice, a warp each; summed in FP64
 template <int NB, typename T>
-__global__ void k_bgs_dots(BatchK K, const T *__restrict__ V, const T *__restrict__ w, int64_t n, int with_norm,
-                           int force) {
+__global__ void k_bgs_dots(BatchK K, const T *__restrict__ V, const T *__restrict__ w, int64_t n) {
   pdl_enter();
-  const int2 it = K.ctl->cur;
-  const int cnt = it.x + 1, lane = threadIdx.x & 31;
+  const int j = K.ctl->cur.x, lane = threadIdx.x & 31;
   const int k = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (k >= cnt + with_norm || (it.y && !force)) return;
+  if (k > j) return;
   const int4 sl = K.slices[blockIdx.x];
-  if (K.frozen_at[sl.x] <= it.x || (force && !K.again[sl.x])) return;
-  const T *vk = k < cnt ? V + (int64_t)k * n : w;
+  if (K.frozen_at[sl.x] <= j) return;
+  const T *vk = V + (int64_t)k * n;
   double s = 0.0;
 #pragma unroll 4
   for (int e = lane; e < sl.z; e += 32) {
@@ -938,27 +939,26 @@ __global__ void k_bgs_dots(BatchK K, const T *__restrict__ V, const T *__restric
 // w -= sum_k h_k V_k on a slice, h its instance's sums over the slices (kept in
 // h by the instance's first block); npart: the slice's squared norm after
 template <int NB, typename T>
-__global__ void k_bgs_update(BatchK K, T *__restrict__ w, const T *__restrict__ V, int64_t n, int with_norm,
-                             int force, double *__restrict__ h, int want_norm) {
+__global__ void k_bgs_update(BatchK K, T *__restrict__ w, const T *__restrict__ V, int64_t n,
+                             double *__restrict__ h, int want_norm) {
   pdl_enter();
-  const int2 it = K.ctl->cur;
-  if (it.y && !force) return;
+  const int j = K.ctl->cur.x;
   const int4 sl = K.slices[blockIdx.x];
-  const int i = sl.x, cnt = it.x + 1;
-  if (K.frozen_at[i] <= it.x || (force && !K.again[i])) return;
+  const int i = sl.x, cnt = j + 1;
+  if (K.frozen_at[i] <= j) return;
   __shared__ T hs[PSTR];
   {
-    const int nh = cnt + with_norm, b1 = K.s0[i + 1];
+    const int b1 = K.s0[i + 1];
     int lg = 5;
-    while (lg > 0 && (nh << lg) > (int)blockDim.x) --lg;
+    while (lg > 0 && (cnt << lg) > (int)blockDim.x) --lg;
     const int G = 1 << lg, k = threadIdx.x >> lg, sub = threadIdx.x & (G - 1);
     double s = 0.0;
-    if (k < nh) {
+    if (k < cnt) {
 #pragma unroll 4
       for (int b = K.s0[i] + sub; b < b1; b += G) s += K.part[(int64_t)b * PSTR + k];
     }
     for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (k < nh && sub == 0) {
+    if (k < cnt && sub == 0) {
       hs[k] = (T)s;
       if ((int)blockIdx.x == K.s0[i]) h[(int64_t)i * PSTR + k] = s;
     }
@@ -986,50 +986,35 @@ __global__ void k_bgs_update(BatchK K, T *__restrict__ w, const T *__restrict__ 
   }
 }
 
-// Arnoldi column j of every active instance (its first block): H(:, j) = h1
-// (+ h2), the rotations, g, the estimate; V_{j+1} = w / |w| with its split (all
-// blocks), zero for a frozen instance and between instances.  theta as in
-// k_gs_finish, per instance: one that needs a second pass is marked in again
-// and finished by the forced call after it.
+// Arnoldi column j of every active instance (its first block): H(:, j) = h1 + h2,
+// the rotations, g, the estimate; V_{j+1} = w / |w| with its split (all blocks),
+// zero for a frozen instance and between instances.
 template <int NB, typename T>
-__global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ V, int64_t n, double theta,
-                             int force, int two, SplitP<T> P) {
+__global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ V, int64_t n, SplitP<T> P) {
   pdl_enter();
-  const int2 it = K.ctl->cur;
-  if (it.y && !force) return;
-  const int j = it.x;
+  const int j = K.ctl->cur.x;
   const int4 sl = K.slices[blockIdx.x];
   const int i = sl.x;
   const bool lead = i >= 0 && (int)blockIdx.x == K.s0[i];
-  const bool live = i >= 0 && K.frozen_at[i] > j && (!force || K.again[i]);
+  const bool live = i >= 0 && K.frozen_at[i] > j;
   __shared__ double sh_scale;
-  __shared__ int sh_skip;
   __shared__ double col[PSTR], sc[PSTR], ss[PSTR];
   double n2 = 0.0;
   if (live) {
     if (lead)
       for (int k = threadIdx.x; k <= j; k += blockDim.x) {
         const int64_t hk = (int64_t)i * PSTR + k, rk = (int64_t)i * (K.m + 1) + k;
-        col[k] = K.h1[hk] + (two ? K.h2[hk] : 0.0);
+        col[k] = K.h1[hk] + K.h2[hk];
         sc[k] = K.cs[rk];
         ss[k] = K.sn[rk];
       }
     n2 = slices_sum(K, i, K.npart);
   }
   if (threadIdx.x == 0) {
-    sh_scale = 0.0;
-    sh_skip = i >= 0 && force && !live;  // its vector is in place from the first pass
-    double hn = 0.0;
-    bool again = false;
-    if (live) {
-      hn = sqrt(n2);
-      sh_scale = hn > 0.0 ? 1.0 / hn : 0.0;
-      again = theta > 0.0 && n2 < theta * theta * K.h1[(int64_t)i * PSTR + j + 1];
-      if (again) sh_skip = 1;
-    }
+    const double hn = live ? sqrt(n2) : 0.0;
+    sh_scale = hn > 0.0 ? 1.0 / hn : 0.0;
     if (lead) {
-      if (!force) K.again[i] = again ? 1 : 0;
-      if (live && !again) {
+      if (live) {
         double *g = K.g + (int64_t)i * (K.m + 1), *H = K.H + (int64_t)i * (K.m + 1) * K.m;
         double below = col[0];
 #pragma unroll 4
@@ -1055,11 +1040,10 @@ __global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ 
         if (res <= K.tgt[i] || !(hn > 0.0)) K.frozen_at[i] = j + 1;
       }
       const bool on = K.frozen_at[i] > j + 1;
-      batch_report(K, j, K.slot + j, on, on ? K.res[i] / K.tgt[i] : 0.0, again);
+      batch_report(K, j, K.slot + j, on, on ? K.res[i] / K.tgt[i] : 0.0);
     }
   }
   __syncthreads();
-  if (sh_skip) return;
   if ((int)threadIdx.x < sl.z)
     scale_split<NB>(K.nodes[sl.y + threadIdx.x], w, sh_scale, V + (int64_t)(j + 1) * n, P);
 }
@@ -1116,7 +1100,6 @@ inline BatchK batch_k(const Ctx &c) {
   K.res = K.tgt + ni;
   K.frozen_at = c.bk_i;
   K.jc = c.bk_i + ni;
-  K.again = c.bk_i + 2 * ni;
   K.part = c.bn_part;
   K.npart = c.bn_npart;
   K.post = c.bk_post;
@@ -1167,26 +1150,23 @@ void enqueue_iteration(Ctx &c, LinSys<T> &S) {
   prof_end(c, MPM_PROF_PRECOND);
   spmv<NB, T>(c, S, S.Z, S.w, ctl, N);
   prof_begin(c, MPM_PROF_ORTH);
-  // FP64: one pass, |w|^2 beside the products for the test of the second;
-  // FP32: always two (one leaves the basis orthogonal to about 1e-6 only)
-  const bool sel = sizeof(T) == sizeof(double);
-  const double *part = c.part;
   // the split goes where the next core reads it: a replayed graph's core is the
   // one captured here, a directly launched one has swapped its buffers
   const SplitP<T> next = c.capturing ? before : next_split<T>(c, S);
   if (c.ninst > 1) {
     const BatchK K = batch_k(c);
-    launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N, sel ? 1 : 0, 0);
-    launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, sel ? 1 : 0, 0, K.h1, sel ? 1 : 0);
-    if (!sel) {
-      launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N, 0, 0);
-      launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, 0, 0, K.h2, 1);
-    }
-    launch_pdl(c, k_bgs_finish<NB, T>, c.bn_all, BG_NODES, 0, K, w, S.V, N, sel ? REORTH_THETA : 0.0, 0,
-               sel ? 0 : 1, next);
+    launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N);
+    launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, K.h1, 0);
+    launch_pdl(c, k_bgs_dots<NB, T>, dim3(c.bn_live, q.ydot), TPB, 0, K, V, w, N);
+    launch_pdl(c, k_bgs_update<NB, T>, c.bn_live, BG_NODES, 0, K, S.w, V, N, K.h2, 1);
+    launch_pdl(c, k_bgs_finish<NB, T>, c.bn_all, BG_NODES, 0, K, w, S.V, N, next);
     prof_end(c, MPM_PROF_ORTH);
     return;
   }
+  // FP64: one pass, |w|^2 beside the products for the test of the second;
+  // FP32: always two (one leaves the basis orthogonal to about 1e-6 only)
+  const bool sel = sizeof(T) == sizeof(double);
+  const double *part = c.part;
   launch_pdl(c, k_gs_dots<T>, dim3(q.ndot, q.ydot), TPB, 0, V, w, N, q.slice, ctl, sel ? 1 : 0, 0, c.part);
   launch_pdl(c, k_gs_update<T>, q.nupd, TPB, 0, S.w, V, N, ctl, part, q.ndot, sel ? 1 : 0, 0, h1,
              sel ? c.npart : (double *)nullptr);
@@ -1200,20 +1180,14 @@ void enqueue_iteration(Ctx &c, LinSys<T> &S) {
   prof_end(c, MPM_PROF_ORTH);
 }
 
-// The second Gram-Schmidt pass of the halted column and its finish (FP64).
+// The second Gram-Schmidt pass of the halted column and its finish (FP64, one
+// instance).
 template <int NB, typename T>
 void enqueue_second_pass(Ctx &c, LinSys<T> &S, const SplitP<T> &next) {
   const int64_t N = c.N(), nn = c.g.nnodes;
   const GsGeom q = gs_geom(c);
   double *h1 = c.hcol, *h2 = c.hcol + PSTR;
   c.launches += 3;
-  if (c.ninst > 1) {
-    const BatchK K = batch_k(c);
-    k_bgs_dots<NB, T><<<dim3(c.bn_live, q.ydot), TPB, 0, c.st>>>(K, S.V, S.w, N, 0, 1);
-    k_bgs_update<NB, T><<<c.bn_live, BG_NODES, 0, c.st>>>(K, S.w, S.V, N, 0, 1, K.h2, 1);
-    k_bgs_finish<NB, T><<<c.bn_all, BG_NODES, 0, c.st>>>(K, S.w, S.V, N, 0.0, 1, 1, next);
-    return;
-  }
   k_gs_dots<T><<<dim3(q.ndot, q.ydot), TPB, 0, c.st>>>(S.V, S.w, N, q.slice, c.ctl, 0, 1, c.part);
   k_gs_update<T><<<q.nupd, TPB, 0, c.st>>>(S.w, S.V, N, c.ctl, c.part, q.ndot, 0, 1, h2, c.npart);
   k_gs_finish<NB, T><<<q.nnode, TPB, 0, c.st>>>(S.w, S.V, nn, c.m_restart, c.ctl, c.npart, q.nupd, h1, h2, 0.0, 1,
@@ -1306,7 +1280,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
       if (launched == j + 1 && launched < m && total + 1 < maxit && seen > SPEC_MARGIN * target) launch(launched++);
       double est;
       if (int rc = slot_wait(c, j, &est)) return rc;
-      if (est == EST_REORTH) {  // what was launched ahead did nothing
+      if (est == EST_REORTH) {  // column j was left unfinished, also by what was launched ahead
         slot_reset(c, j);
         enqueue_second_pass<NB, T>(c, S, split());
         launched = j + 1;

@@ -1,0 +1,42 @@
+"""FGMRES on its less travelled ways."""
+import numpy as np
+import pytest
+
+from paper_1905_00671_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mpm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1905_00671_gb300 import mpm as m
+
+    m.load()
+    return m
+
+
+def columns():
+    return [I.terzaghi_column(ncell_y=30, ncell_x=6, h=0.25, k=1e-10, load=10e3),
+            I.terzaghi_column(ncell_y=24, ncell_x=8, h=0.25, k=1e-11, load=50e3)]
+
+
+def test_batch_takes_both_gram_schmidt_passes(mpm):
+    """A batch's iteration takes as many kernels in FP64 as in FP32, whose
+    iterations always orthogonalise twice.  Kernels per iteration: from two solves
+    of one Newton iteration each, to different tolerances."""
+    per_iteration = []
+    for precision in (mpm.MPM_FP64, mpm.MPM_MIXED):
+        runs = []
+        for rtol in (1e-2, 1e-5):
+            batch = mpm.Batch(columns(), precision=precision, newton_rtol=0.5, krylov_rtol=rtol)
+            st = batch.step()
+            assert st["newton_iters"] == 1
+            runs.append((st["krylov_total"], st["kernel_launches"]))
+            batch.close()
+        (i0, l0), (i1, l1) = runs
+        assert i1 >= i0 + 5
+        per_iteration.append((l1 - l0) / (i1 - i0))
+    assert per_iteration[0] == per_iteration[1], per_iteration
