@@ -44,7 +44,7 @@ enum {
   MPM_ERR_BAD_ARG = -1,          /* invalid argument or size */
   MPM_ERR_OUT_OF_GRID = -2,      /* a material point centre left the background grid */
   MPM_ERR_NEGATIVE_J = -3,       /* det F <= 0 at some material point */
-  MPM_ERR_NONFINITE = -4,        /* NaN / Inf in the residual */
+  MPM_ERR_NONFINITE = -4,        /* NaN / Inf in the residual or the linear solve */
   MPM_ERR_NEWTON_DIVERGED = -5,  /* Newton hit its iteration cap */
   MPM_ERR_KRYLOV_STAGNATED = -6, /* the Krylov solver hit its iteration cap */
   MPM_ERR_TIMEOUT = -7,          /* reserved for bounded device-side waits */

@@ -345,6 +345,11 @@ __global__ void k_bsr_spmv(int64_t nnodes, const int32_t *__restrict__ row_ptr,
 }
 
 // ---------------------------------------------------------------- FGMRES
+// What a solve posts instead of an estimate once a value is not finite (a rotation
+// formed from such a value could leave an estimate of zero): the host returns
+// MPM_ERR_NONFINITE.
+__device__ inline double not_finite() { return __longlong_as_double(0x7ff8000000000000ll); }
+
 // Partial dots of w against V_0..V_{cnt-1}, block (b, i) summing its slice of
 // V_i . w: the cnt products run side by side instead of one after another.
 // A row i = cnt of blocks (grid y = cnt + 1) sums w . w.  With skip set, the
@@ -434,7 +439,9 @@ __global__ void k_arnoldi_finish(const double *__restrict__ part, int np, int j,
   }
   const double r = hypot(col[j], hn);
   double c = 1.0, s = 0.0;
-  if (r > 0.0) {
+  if (!isfinite(r)) {
+    s = not_finite();
+  } else if (r > 0.0) {
     c = col[j] / r;
     s = hn / r;
   }
@@ -660,7 +667,9 @@ __global__ void k_gs_finish(const T *__restrict__ w, T *__restrict__ V, int64_t 
         double r = fma(below, below, hn * hn);
         r = r > 1e-280 && r < 1e280 ? sqrt(r) : hypot(below, hn);
         double c = 1.0, s2 = 0.0;
-        if (r > 0.0) {
+        if (!isfinite(r)) {
+          s2 = not_finite();
+        } else if (r > 0.0) {
           c = below / r;
           s2 = hn / r;
         }
@@ -853,6 +862,12 @@ __device__ inline double slices_sum(const BatchK &K, int i, const double *__rest
   return block_sum(acc);
 }
 
+// How far an estimate is from its target.  Ratios are compared by their bits, where
+// this NaN is above every number.
+__device__ inline double batch_ratio(double res, double tgt) {
+  return isfinite(res) ? res / tgt : not_finite();
+}
+
 // An instance's first block reports (thread 0): whether it goes on and how far
 // its estimate is from its target; the last report of the kernel posts the largest
 // ratio (0: all done) and moves the control word
@@ -898,7 +913,7 @@ __global__ void k_bgs_start(BatchK K, const T *__restrict__ r, T *__restrict__ V
     const double n2 = slices_sum(K, i, K.npart);
     if (threadIdx.x == 0) {
       const double beta = sqrt(n2), tgt = set_target ? rtol * beta : K.tgt[i];
-      const bool done = !(beta > tgt);
+      const bool done = isfinite(beta) && !(beta > tgt);
       sh_scale = !done && beta > 0.0 ? 1.0 / beta : 0.0;
       if ((int)blockIdx.x == K.s0[i]) {
         if (set_target) K.tgt[i] = tgt;
@@ -907,7 +922,7 @@ __global__ void k_bgs_start(BatchK K, const T *__restrict__ r, T *__restrict__ V
         g[0] = beta;
         K.jc[i] = 0;
         K.frozen_at[i] = done ? 0 : 0x7fffffff;
-        batch_report(K, -1, K.slot + SLOT_BETA, !done, beta / tgt);
+        batch_report(K, -1, K.slot + SLOT_BETA, !done, batch_ratio(beta, tgt));
       }
     }
   }
@@ -1025,7 +1040,9 @@ __global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ 
         }
         const double r = hypot(below, hn);
         double c = 1.0, sv = 0.0;
-        if (r > 0.0) {
+        if (!isfinite(r)) {
+          sv = not_finite();
+        } else if (r > 0.0) {
           c = below / r;
           sv = hn / r;
         }
@@ -1037,10 +1054,10 @@ __global__ void k_bgs_finish(BatchK K, const T *__restrict__ w, T *__restrict__ 
         g[j] = c * gj;
         K.res[i] = res;
         K.jc[i] = j + 1;
-        if (res <= K.tgt[i] || !(hn > 0.0)) K.frozen_at[i] = j + 1;
+        if (res <= K.tgt[i] || (isfinite(res) && !(hn > 0.0))) K.frozen_at[i] = j + 1;
       }
       const bool on = K.frozen_at[i] > j + 1;
-      batch_report(K, j, K.slot + j, on, on ? K.res[i] / K.tgt[i] : 0.0);
+      batch_report(K, j, K.slot + j, on, on ? batch_ratio(K.res[i], K.tgt[i]) : 0.0);
     }
   }
   __syncthreads();
@@ -1267,8 +1284,8 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
   *iters = 0;
   double beta0;
   if (int rc = start(b, &beta0, 1)) return rc;
-  if (!(beta0 > 0.0)) return MPM_OK;
   if (!isfinite(beta0)) return MPM_ERR_NONFINITE;
+  if (!(beta0 > 0.0)) return MPM_OK;
   const double target = batch ? 0.5 : rtol * beta0;  // (a batch posts 0 or a ratio above 1)
   int total = 0;
   bool converged = false;
@@ -1312,6 +1329,7 @@ int fgmres_graph_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) 
     UPMPM_LAUNCH(c);
     double br;
     if (int rc = start(w, &br, 0)) return rc;
+    if (!isfinite(br)) return MPM_ERR_NONFINITE;
     if (br <= target) {
       converged = true;
       break;
@@ -1342,8 +1360,8 @@ int fgmres_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
   c.launches += 4;
   const double beta0 = read_scalar(c, c.scal);
   *iters = 0;
-  if (!(beta0 > 0.0)) return MPM_OK;
   if (!isfinite(beta0)) return MPM_ERR_NONFINITE;
+  if (!(beta0 > 0.0)) return MPM_OK;
   const double target = rtol * beta0;
   int total = 0;
   bool converged = false;
@@ -1411,6 +1429,7 @@ int fgmres_impl(Ctx &c, LinSys<T> &S, double rtol, int maxit, int *iters) {
     k_scale_copy<T><<<gN, TPB, 0, c.st>>>(S.V, w, c.scal + 1, N);
     c.launches += 5;
     const double br = read_scalar(c, c.scal);
+    if (!isfinite(br)) return MPM_ERR_NONFINITE;
     if (br <= target) {
       converged = true;
       break;

@@ -1,4 +1,6 @@
 """FGMRES on its less travelled ways."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 
@@ -40,3 +42,29 @@ def test_batch_takes_both_gram_schmidt_passes(mpm):
         assert i1 >= i0 + 5
         per_iteration.append((l1 - l0) / (i1 - i0))
     assert per_iteration[0] == per_iteration[1], per_iteration
+
+
+def overflowing(w):
+    """A few points in the middle so stiff that their blocks are infinite in FP32,
+    while the residual (and the rows of the loaded surface) stay finite."""
+    E = w.E.copy()
+    mid = np.argsort(np.abs(w.x - w.x.mean(axis=0)).sum(axis=1))[:4]
+    E[mid] = 1e42
+    return replace(w, E=E)
+
+
+@pytest.mark.parametrize("kind", ["single", "batch", "large"])
+def test_values_that_are_not_finite_are_an_error(mpm, kind):
+    """Not a solution: a rotation formed from NaN would leave an estimate of zero."""
+    if kind == "batch":
+        ws = columns()
+        x = mpm.Batch([ws[0], overflowing(ws[1])], precision=mpm.MPM_MIXED)
+    else:
+        # ("large": above 2^20 unknowns, where the iterations are not graphs)
+        n = (30, 6) if kind == "single" else (592, 592)
+        x = mpm.Simulation(overflowing(I.terzaghi_column(ncell_y=n[0], ncell_x=n[1])), precision=mpm.MPM_MIXED)
+    with pytest.raises(mpm.MPMError) as e:
+        x.step()
+    assert e.value.code == -4, e.value          # MPM_ERR_NONFINITE
+    assert "FGMRES" in str(e.value)
+    x.close()
