@@ -862,10 +862,12 @@ __device__ inline double slices_sum(const BatchK &K, int i, const double *__rest
   return block_sum(acc);
 }
 
-// How far an estimate is from its target.  Ratios are compared by their bits, where
-// this NaN is above every number.
+// How far an estimate is from its target: finite also for a target of zero or below
+// (a krylov_rtol that no estimate reaches).  Ratios are compared by their bits, where
+// the NaN is above every number.
 __device__ inline double batch_ratio(double res, double tgt) {
-  return isfinite(res) ? res / tgt : not_finite();
+  if (!isfinite(res)) return not_finite();
+  return tgt > 0.0 ? fmin(res / tgt, 1e300) : 1e300;
 }
 
 // An instance's first block reports (thread 0): whether it goes on and how far

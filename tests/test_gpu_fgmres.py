@@ -68,3 +68,14 @@ def test_values_that_are_not_finite_are_an_error(mpm, kind):
     assert e.value.code == -4, e.value          # MPM_ERR_NONFINITE
     assert "FGMRES" in str(e.value)
     x.close()
+
+
+@pytest.mark.parametrize("rtol", [0.0, -1.0, 1e-320])
+def test_a_tolerance_that_nothing_reaches(mpm, rtol):
+    """A batch stops at its iteration cap, as a single system does."""
+    for x in (mpm.Simulation(columns()[0], krylov_rtol=rtol, krylov_max=150),
+              mpm.Batch(columns(), krylov_rtol=rtol, krylov_max=150)):
+        with pytest.raises(mpm.MPMError) as e:
+            x.step()
+        assert e.value.code == -6, e.value      # MPM_ERR_KRYLOV_STAGNATED
+        x.close()
