@@ -328,6 +328,7 @@ int prepare_step(Ctx &c, double dt, const mpm_loads *L, const mpm_bcs *B) {
   if (!rc) rc = upload_bcs(c, B);
   if (rc) return rc;
   c.s.dt = dt;
+  c.jb_refused = c.rb_refused = false;
   prof_begin(c, MPM_PROF_PREP);
   rc = run_binning(c);
   if (rc) return rc;
@@ -681,7 +682,6 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   s.phi_min = opt->min_volume_fraction;
   s.kozeny = opt->permeability == MPM_PERM_KOZENY_CARMAN;
   s.hencky = opt->model == MPM_MODEL_HENCKY;
-  // the FP32 Jacobian's direct form has no Hencky tangent: staged only
   for (int k = 0; k < 3; ++k) s.g[k] = k < c.d ? mat->g[k] : 0.0;
   c.n = P->n;
   c.n_surf = P->n_surf;
@@ -720,8 +720,6 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   A(&c.sh_S0, 3 * MAXS * n);
   A(&c.m, n);
   A(&c.rec, RC_COUNT * n);
-  // the FP64 Jacobian's staging (allocated on first use in a mixed context,
-  // whose Jacobian is FP32 and unstaged)
   A(&c.M, nn);
   A(&c.Pn, nn);
   A(&c.vn, d * nn);

@@ -1962,21 +1962,49 @@ __global__ void k_cm_init(int64_t nn, int K, const double *__restrict__ rhs, con
 }  // namespace
 
 // ============================================================== launchers
+// The bins' sums only make the residual and the Jacobian faster, so they give way
+// where a step needs their memory for what it cannot do without.
+bool shed_scratch(Ctx &c) {
+  if (!c.rb && !c.jb) return false;
+  for (void **p : {(void **)&c.rb, (void **)&c.rb_cnt, &c.jb, (void **)&c.jb_cnt}) {
+    cudaFree(*p);
+    *p = nullptr;
+  }
+  c.rb_cap = c.jb_cap = 0;
+  return true;
+}
+
+int step_malloc(Ctx &c, void **p, size_t bytes) {
+  for (;;) {
+    if (cudaMalloc(p, bytes) == cudaSuccess) return MPM_OK;
+    cudaGetLastError();
+    *p = nullptr;
+    if (!shed_scratch(c)) return MPM_ERR_NO_MEMORY;
+  }
+}
+
+// Most that one of the bins' buffers may take: an eighth of what is free, so that
+// other contexts and the application keep room.
+static int64_t scratch_limit() {
+  size_t avail = 0, total = 0;
+  if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (int64_t)(avail / 8);
+}
+
 // Staging buffer of at least c.pn_total records of `stride` values: kept
 // while large enough, else reallocated with a quarter of headroom (the supports
 // grow and shrink a little from step to step as the points move).
 template <typename R>
-static int grow_staging(R **buf, int64_t *cap, int64_t total, int stride) {
+static int grow_staging(Ctx &c, R **buf, int64_t *cap, int64_t total, int stride) {
   if (*buf && *cap >= total) return MPM_OK;
   cudaFree(*buf);
   *buf = nullptr;
   *cap = 0;
   const int64_t want = total + total / 4 + 1024;
-  if (cudaMalloc(buf, sizeof(R) * want * stride) != cudaSuccess) {
-    cudaGetLastError();
-    *buf = nullptr;
-    return MPM_ERR_NO_MEMORY;
-  }
+  if (const int rc = step_malloc(c, (void **)buf, sizeof(R) * want * stride)) return rc;
   *cap = want;
   return MPM_OK;
 }
@@ -1992,8 +2020,11 @@ static int jac_box(const Ctx &c) {
   return 3;
 }
 
-// Ring of bin planes: as many as JAC_RING_BYTES hold (all of a 2D grid or a
-// small 3D one, so that the two kernels run once), at least LB.
+// Ring of bin planes: as many as JAC_RING_BYTES (and scratch_limit) hold, all of a
+// 2D grid or a small 3D one, so that the two kernels run once; at least LB.  Per
+// assembly with 8 GB, 1 GB and three planes: 4.2M-point slope 90.0, 94.7, 94.7 ms (FP32
+// 18.4, 21.1, 21.1), 1M-point block FP32 3.84, 4.16, 5.48, 163k-point block 3.71, 3.84, 5.74
+// (1.6 GB hold all of its planes).
 constexpr int64_t JAC_RING_BYTES = 8ll << 30;
 template <typename R>
 static int64_t jac_plane_bytes(const Ctx &c, int lb) {
@@ -2006,43 +2037,43 @@ template <typename R>
 static int ensure_jac_ring(Ctx &c, int lb) {
   const int64_t pb = jac_plane_bytes<R>(c, lb);
   const int planes = c.g.nn[c.d - 1];
-  int ring = (int)std::min<int64_t>(planes, std::max<int64_t>(lb, JAC_RING_BYTES / pb));
-  if (c.jb && (c.jb_cap >= pb * ring || (c.jb_short && c.jb_cap >= pb * lb))) {
-    c.jb_ring = (int)std::min<int64_t>(ring, c.jb_cap / pb);
+  if (c.jb && c.jb_cap >= pb * std::min(lb, planes)) {
+    c.jb_ring = (int)std::min<int64_t>(planes, c.jb_cap / pb);
     return MPM_OK;
   }
-  const int asked = ring;
+  if (c.jb_refused) return MPM_ERR_NO_MEMORY;
   cudaFree(c.jb);
   cudaFree(c.jb_cnt);
   c.jb = nullptr;
   c.jb_cnt = nullptr;
   c.jb_cap = 0;
-  for (;; ring = std::max(lb, ring / 2)) {  // a smaller ring where memory is short
-    if (cudaMalloc(&c.jb, pb * ring) == cudaSuccess) break;
+  const int64_t limit = std::min(JAC_RING_BYTES, scratch_limit());
+  int ring = (int)std::min<int64_t>(planes, std::max<int64_t>(lb, limit / pb));
+  for (;;) {  // a smaller ring where memory is short, then the residual's bins in its place
+    if (cudaMalloc(&c.jb, pb * ring) == cudaSuccess) {
+      if (cudaMalloc(&c.jb_cnt, sizeof(int32_t) * c.g.nnodes) == cudaSuccess) break;
+      cudaFree(c.jb);
+    }
     cudaGetLastError();
-    c.jb = nullptr;
-    if (ring <= lb) return MPM_ERR_NO_MEMORY;
-  }
-  if (cudaMalloc(&c.jb_cnt, sizeof(int32_t) * c.g.nnodes) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(c.jb);
     c.jb = nullptr;
     c.jb_cnt = nullptr;
-    return MPM_ERR_NO_MEMORY;
+    if (ring > lb) {
+      ring = std::max(lb, ring / 2);
+    } else if (!shed_scratch(c)) {
+      c.jb_refused = true;
+      return MPM_ERR_NO_MEMORY;
+    }
   }
   c.jb_cap = pb * ring;
   c.jb_ring = ring;
-  c.jb_short = ring < asked;
   return MPM_OK;
 }
 
+// (the per-pair kernel with its staging where not even LB planes fit)
 int ensure_jacobian_staging(Ctx &c) {
-  if (const int lb = jac_box(c)) {
-    const int rc = ensure_jac_ring<double>(c, lb);
-    if (rc) c.last_error = "device allocation of the Jacobian's bin sums failed";
-    return rc;
-  }
-  const int rc = grow_staging(&c.pn, &c.pn_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 8));
+  const int lb = jac_box(c);
+  if (lb && ensure_jac_ring<double>(c, lb) == MPM_OK) return MPM_OK;
+  const int rc = grow_staging(c, &c.pn, &c.pn_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 8));
   if (rc) c.last_error = "device allocation of the Jacobian staging failed";
   return rc;
 }
@@ -2068,7 +2099,7 @@ int run_consistent_p2g(Ctx &c) {
     cudaFree(c.cm_buf);
     c.cm_buf = nullptr;
     c.cm_cap = 0;
-    if (cudaMalloc(&c.cm_buf, sizeof(double) * need) != cudaSuccess) {
+    if (step_malloc(c, (void **)&c.cm_buf, sizeof(double) * need)) {
       c.last_error = "device allocation of the consistent-mass mapping failed";
       return MPM_ERR_NO_MEMORY;
     }
@@ -2082,7 +2113,7 @@ int run_consistent_p2g(Ctx &c) {
     cudaFree(c.mc);
     c.mc = nullptr;
     c.mc_cap = 0;
-    if (cudaMalloc(&c.mc, sizeof(double) * c.nnzb_cap) != cudaSuccess) {
+    if (step_malloc(c, (void **)&c.mc, sizeof(double) * c.nnzb_cap)) {
       c.last_error = "device allocation of the consistent mass failed";
       return MPM_ERR_NO_MEMORY;
     }
@@ -2161,8 +2192,8 @@ int run_pattern(Ctx &c) {
     cudaFree(c.col);
     cudaFree(c.row_of);
     c.col = c.row_of = nullptr;
-    if (cudaMalloc(&c.col, sizeof(int32_t) * cap) != cudaSuccess ||
-        cudaMalloc(&c.row_of, sizeof(int32_t) * cap) != cudaSuccess) {
+    if (step_malloc(c, (void **)&c.col, sizeof(int32_t) * cap) ||
+        step_malloc(c, (void **)&c.row_of, sizeof(int32_t) * cap)) {
       c.nnzb_cap = 0;
       c.last_error = "device allocation of the block-CSR matrix failed";
       return MPM_ERR_NO_MEMORY;
@@ -2255,17 +2286,20 @@ static bool ensure_residual_bins(Ctx &c, int lb) {
   const int nl = c.d == 2 ? lb * lb : lb * lb * lb;
   const int64_t need = c.g.nnodes * nl * c.nb;
   if (c.rb && c.rb_cap >= need) return true;
+  if (c.rb_refused) return false;
   cudaFree(c.rb);
+  cudaFree(c.rb_cnt);
   c.rb = nullptr;
+  c.rb_cnt = nullptr;
   c.rb_cap = 0;
-  if (!c.rb_cnt && cudaMalloc(&c.rb_cnt, sizeof(int32_t) * c.g.nnodes) != cudaSuccess) {
+  if ((int64_t)sizeof(double) * need > scratch_limit() ||
+      cudaMalloc(&c.rb, sizeof(double) * need) != cudaSuccess ||
+      cudaMalloc(&c.rb_cnt, sizeof(int32_t) * c.g.nnodes) != cudaSuccess) {
     cudaGetLastError();
-    c.rb_cnt = nullptr;
-    return false;
-  }
-  if (cudaMalloc(&c.rb, sizeof(double) * need) != cudaSuccess) {
-    cudaGetLastError();
+    cudaFree(c.rb);
     c.rb = nullptr;
+    c.rb_cnt = nullptr;
+    c.rb_refused = true;
     return false;
   }
   c.rb_cap = need;
@@ -2302,8 +2336,12 @@ void run_residual(Ctx &c, const double *X, double *R, int apply_bc) {
 
 // FP32 copy of the staging (allocated for the staged FP32 variant only)
 int ensure_jacobian_staging32(Ctx &c) {
-  if (const int lb = jac_box(c)) return ensure_jac_ring<float>(c, lb);
-  return grow_staging(&c.pn32, &c.pn32_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 4));
+  const int lb = jac_box(c);
+  if (lb) {
+    const int rc = ensure_jac_ring<float>(c, lb);
+    if (!rc || !c.s.hencky) return rc;  // (without room the direct form serves, which has no Hencky tangent)
+  }
+  return grow_staging(c, &c.pn32, &c.pn32_cap, c.pn_total, pn_stride(c.d, c.dyn, c.s.hencky, 4));
 }
 
 // The staged form by first-node bins: chunks of bin planes, each followed by the
@@ -2332,8 +2370,8 @@ void launch_jac_bins(Ctx &c, T *val, int apply_bc, const BasisArrays<T> &BA, con
 }
 
 // One assembly with a given kernel configuration: staged (by first-node bins, or
-// for supports of 4 nodes k_point_nodes then k_jacobian on the per-(point, node)
-// vectors) or direct (k_jacobian_direct), tpb threads per block of the kernel
+// for supports of 4 nodes, or without room for the ring, k_point_nodes then
+// k_jacobian on the per-(point, node) vectors) or direct (k_jacobian_direct), tpb threads per block of the kernel
 // that writes the blocks.  Values in precision T computed
 // in precision T from the FP64 records or their FP32 copies.
 template <typename T>
@@ -2362,8 +2400,8 @@ void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
     BA.nrm = (const R *)c.sh_nrmf; rec = (const R *)c.recf;
     pn = (R *)c.pn32;
   }
-  const int lb = staged ? jac_box(c) : 0;
-  if (staged && !(lb ? c.jb != nullptr : pn != nullptr)) return;  // callers allocate the staging first
+  const int lb = staged && c.jb ? jac_box(c) : 0;
+  if (staged && !lb && !pn) return;  // callers allocate the ring or the staging first
   if (lb) {
 #define BINS(D, LB, Y, H) launch_jac_bins<D, LB, Y, H, T>(c, val, apply_bc, BA, rec, tpb)
 #define BINS_LB(D, Y, H) do { if (lb == 2) BINS(D, 2, Y, H); else BINS(D, 3, Y, H); } while (0)
@@ -2393,7 +2431,7 @@ void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
 #undef PNODES
     UPMPM_LAUNCH(c);
   }
-  // supports of four nodes (GIMP), or the direct form (FP32)
+  // supports of four nodes (GIMP) or no room for the ring, or the direct form (FP32)
 #define JAC_WIDE(D, Y)                                                                                       \
   do {                                                                                                       \
     if (c.s.hencky)                                                                                          \
@@ -2486,14 +2524,15 @@ void run_jacobian(Ctx &c, T *val, int apply_bc) {
   constexpr int pi = sizeof(T) == sizeof(double) ? 0 : 1;
   Ctx::JacCfg &cfg = c.jac_cfg[pi];
   if (c.opt.autotune && !cfg.tuned && !c.capturing) autotune_jacobian<T>(c, val, apply_bc);
-  // without room for the FP32 staging the direct form serves, except for
-  // Hencky (whose Newton loop allocates the staging first and stops on failure)
-  if (pi == 1 && cfg.form != Ctx::JAC_DIRECT && !c.s.hencky && ensure_jacobian_staging32(c) != MPM_OK)
-    cfg.form = Ctx::JAC_DIRECT;
-  c.stats.jac_config[pi] = cfg.tpb + 1000 * cfg.form;
+  // without room for the FP32 ring the direct form serves this assembly, except for
+  // Hencky (whose Newton loop allocates the ring or staging first and stops on failure)
+  int form = cfg.form;
+  if (pi == 1 && form != Ctx::JAC_DIRECT && !c.s.hencky && ensure_jacobian_staging32(c) != MPM_OK)
+    form = Ctx::JAC_DIRECT;
+  c.stats.jac_config[pi] = cfg.tpb + 1000 * form;
   c.stats.jac_tuned[pi] = cfg.tuned;
   prof_begin(c, MPM_PROF_JACOBIAN);
-  launch_jacobian<T>(c, val, apply_bc, cfg.form, cfg.tpb);
+  launch_jacobian<T>(c, val, apply_bc, form, cfg.tpb);
   prof_end(c, MPM_PROF_JACOBIAN);
 }
 

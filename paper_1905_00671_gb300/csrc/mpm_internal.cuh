@@ -362,7 +362,8 @@ struct Ctx {
   int64_t jb_cap = 0;                    // bytes
   int32_t *jb_cnt = nullptr;
   int jb_ring = 0;
-  bool jb_short = false;                 // memory was short of the ring asked for
+  // not tried again before the next step after an allocation that failed
+  bool jb_refused = false, rb_refused = false;
   // residual by first-node bins: the bins' sums and box extents
   double *rb = nullptr;
   int64_t rb_cap = 0;
@@ -428,8 +429,11 @@ void run_g2p(Ctx &c);
 // assembly
 int run_pattern(Ctx &c);                          // builds row_ptr / col / row_of
 int run_consistent_p2g(Ctx &c);  // Stage-1 fields by the consistent mass (after run_pattern)
-int ensure_jacobian_staging(Ctx &c);  // the FP64 Jacobian's staging buffer (allocated by FP64 contexts at create)
-int ensure_jacobian_staging32(Ctx &c);  // the FP32 staged Jacobian's buffer (mixed mode; Hencky always, else when chosen)
+int ensure_jacobian_staging(Ctx &c);  // the FP64 Jacobian's ring of bins, or its staging buffer
+int ensure_jacobian_staging32(Ctx &c);  // the same in FP32 (mixed mode)
+// cudaMalloc for what a step cannot do without: the bins' buffers give way to it
+int step_malloc(Ctx &c, void **p, size_t bytes);
+bool shed_scratch(Ctx &c);  // frees them; false if there were none
 void run_initial_guess(Ctx &c);   // also sets the active flags
 void run_renorm(Ctx &c);          // per-point renormalisation over active box nodes
 int run_pn_layout(Ctx &c);        // first staged Jacobian record of each point (pn_base)

@@ -1899,9 +1899,9 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
     for (MG_REAL *p : ptrs) cudaFree(p);
     S.Aval = S.Sval = S.B1c = S.W = S.B2c = nullptr;
     const int64_t cap = c.nnzb_cap;
-    if (cudaMalloc(&S.Aval, sizeof(real) * cap * d * d) || cudaMalloc(&S.Sval, sizeof(real) * cap) ||
-        cudaMalloc(&S.B1c, sizeof(real) * cap * d) || cudaMalloc(&S.W, sizeof(real) * cap * d) ||
-        (c.schur_lower() && cudaMalloc(&S.B2c, sizeof(real) * cap * d))) {
+    auto get = [&](MG_REAL **p, int64_t vals) { return step_malloc(c, (void **)p, sizeof(real) * vals); };
+    if (get(&S.Aval, cap * d * d) || get(&S.Sval, cap) || get(&S.B1c, cap * d) || get(&S.W, cap * d) ||
+        (c.schur_lower() && get(&S.B2c, cap * d))) {
       S.sub_cap = 0;
       c.last_error = "device allocation of the block preconditioner failed";
       return MPM_ERR_NO_MEMORY;
@@ -1915,8 +1915,7 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
   for (MGHier<real> *H : {S.mgA, S.mgS}) {
     if (win == 5 && !H->ap_wide && H->nlev > 1) {
       real *p = nullptr;  // (the narrower buffer stays if there is no room)
-      if (cudaMalloc(&p, sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B) != cudaSuccess) {
-        cudaGetLastError();
+      if (step_malloc(c, (void **)&p, sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B)) {
         c.last_error = "device allocation of the block preconditioner failed";
         return MPM_ERR_NO_MEMORY;
       }

@@ -1552,7 +1552,7 @@ int linsys_reserve(Ctx &c, LinSys<T> &S) {
   if (S.val) cudaFree(S.val);
   S.val = nullptr;
   S.cap = 0;
-  if (dmalloc(&S.val, c.nnzb_cap * c.nb * c.nb)) {
+  if (step_malloc(c, (void **)&S.val, sizeof(T) * c.nnzb_cap * c.nb * c.nb)) {
     c.last_error = "device allocation of the block-CSR values failed";
     return MPM_ERR_NO_MEMORY;
   }

@@ -1,7 +1,8 @@
 /* Preloaded between libupmpm.so and the CUDA runtime by the tests that need a
  * call to be slow or to fail where on a real machine that is a matter of luck:
  *   SHIM_ATTR_SLEEP_US  microseconds that cudaFuncSetAttribute takes longer,
- *   shim_set_budget(b)  bytes that cudaMalloc may still hand out (negative: any).
+ *   shim_set_budget(b)  bytes that cudaMalloc may still hand out (negative: any),
+ *                       which cudaMemGetInfo then calls free.
  * A refused allocation is passed on as one that no device can serve, so that the
  * runtime's own error state is the one of a real failure. */
 #define _GNU_SOURCE
@@ -64,6 +65,18 @@ int cudaFree(void *p) {
     }
   pthread_mutex_unlock(&lock);
   return f(p);
+}
+
+int cudaMemGetInfo(size_t *avail, size_t *total) {
+  int (*f)(size_t *, size_t *) = (int (*)(size_t *, size_t *))real("cudaMemGetInfo");
+  const int rc = f(avail, total);
+  pthread_mutex_lock(&lock);
+  if (rc == 0 && budget >= 0) {
+    const long long left = budget > used ? budget - used : 0;
+    if ((long long)*avail > left) *avail = (size_t)left;
+  }
+  pthread_mutex_unlock(&lock);
+  return rc;
 }
 
 int cudaFuncSetAttribute(const void *func, int attr, int value) {

@@ -1,0 +1,57 @@
+"""Steps where device memory is short: the sums by first-node bins make the
+residual and the Jacobian faster, and a step must do without them before it fails
+for want of memory.  The thin block's ring of three bin planes (0.3 GB) is larger
+than the records of the per-pair kernel."""
+import pytest
+
+from tests import shim
+
+pytestmark = pytest.mark.gpu
+
+PROGRAM = """
+import numpy as np
+from paper_1905_00671_gb300 import inputs as I, mpm
+
+precision, extra = {precision}, {extra}
+w = I.small_block(seed=11, body=(40, 40, 2), pad=5)
+
+def step():
+    base = shim.shim_used()
+    sim = mpm.Simulation(w, precision=precision)
+    st = sim.step()
+    out = sim.read(("u", "p")), shim.shim_used() - base, sim.stats()
+    sim.close()
+    return out
+
+ref, used, st = step()
+nn = [c + 1 for c in w.ncell]
+nodes, plane, word = nn[0] * nn[1] * nn[2], nn[0] * nn[1], 4 if precision else 8
+pair = 378 * (24 if precision else 22) * word     # values of a bin's pairs, padded to 16 bytes
+ring, bins = nodes * (pair + 4), nodes * (27 * 4 * 8 + 4)
+records = ((st["jac_point_nodes"] + len(w.x)) * 1.25 + 1024) * 22 * 8 if not precision else 0
+others = used - ring - bins
+assert records < 0.8 * 3 * plane * pair, (records, 3 * plane * pair)
+assert others > 0
+shim.shim_set_budget(int(others + eval(extra)))
+got, _, st = step()
+print("refused", shim.shim_refused(), "config", st["jac_config"])
+assert shim.shim_refused() > 0
+for f in ref:
+    assert np.abs(got[f] - ref[f]).max() <= 1e-8 * np.abs(ref[f]).max(), f
+"""
+
+# what is left beside the buffers that a step cannot do without
+CASES = {
+    "fp64-no-room-for-three-planes": (0, "bins + 0.9 * 3 * plane * pair"),
+    "fp64-bins-give-way": (0, "records + 0.4 * bins"),
+    "mixed-bins-give-way": (1, "0.6 * bins"),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_a_step_does_without_the_bins(name, tmp_path):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    precision, extra = CASES[name]
+    shim.run(shim.build(tmp_path), PROGRAM.format(precision=precision, extra=repr(extra)))
