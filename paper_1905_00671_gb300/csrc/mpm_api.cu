@@ -89,7 +89,7 @@ int slot_wait(Ctx &c, int slot, double *value) {
       return MPM_ERR_CUDA;
     }
     if (n % 4096 == 0) {  // a failed launch or kernel never writes it
-      cudaError_t e = cudaPeekAtLastError();
+      cudaError_t e = cudaGetLastError();
       if (e == cudaSuccess) {
         e = cudaStreamQuery(c.st);
         if (e == cudaErrorNotReady) {
