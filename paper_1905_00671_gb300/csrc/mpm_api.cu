@@ -7,8 +7,10 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <new>
 #include <string>
+#include <thread>
 
 #include "mpm_internal.cuh"
 
@@ -94,6 +96,9 @@ int slot_wait(Ctx &c, int slot, double *value) {
         e = cudaStreamQuery(c.st);
         if (e == cudaErrorNotReady) {
           cudaGetLastError();
+          // (the first 4,096 looks take about the time of a few kernels)
+          if (c.wait_sleeps) std::this_thread::sleep_for(std::chrono::microseconds(50));
+          else std::this_thread::yield();
           continue;
         }
       }
@@ -642,6 +647,9 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
       c.nsm = nsm;
+    unsigned flags = 0;
+    if (cudaGetDeviceFlags(&flags) == cudaSuccess)
+      c.wait_sleeps = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   }
   c.st = (cudaStream_t)opt->stream;
   if (!c.st) {

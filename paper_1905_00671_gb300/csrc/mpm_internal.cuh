@@ -402,6 +402,7 @@ struct Ctx {
   // write and the host polls (slot_reset / slot_wait), against a copy and a
   // stream synchronisation each
   double *h_slot = nullptr, *d_slot = nullptr;
+  bool wait_sleeps = false;              // between looks: the application asked for blocking synchronisation
 
   // scan scratch
   int32_t *scan_tmp = nullptr;

@@ -1,5 +1,5 @@
-"""How the library waits for results on the host, in processes of their own (a
-pending error belongs to a thread)."""
+"""How the library waits for results on the host, in processes of their own (the
+way of waiting and a pending error belong to the process and its thread)."""
 import pytest
 
 from tests import shim
@@ -12,6 +12,17 @@ from paper_1905_00671_gb300 import inputs as I, mpm
 
 cudart = ctypes.CDLL("libcudart.so.13")
 w = I.consolidation_block(body=(48, 48, 24), pad=2)
+"""
+
+BLOCKING = HEAD + """
+assert cudart.cudaSetDeviceFlags(4) == 0        # cudaDeviceScheduleBlockingSync
+sim = mpm.Simulation(w)
+sim.step()
+wall, cpu = time.perf_counter(), time.thread_time()
+sim.step()
+wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+print("wall", wall, "cpu", cpu)
+assert cpu <= 0.5 * wall, (cpu, wall)
 """
 
 PENDING = HEAD + """
@@ -32,6 +43,12 @@ def so(tmp_path_factory):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     return shim.build(tmp_path_factory.mktemp("shim"))
+
+
+def test_a_blocking_application_does_not_spin(so):
+    """With blocking synchronisation asked of the runtime, the stepping thread sleeps
+    for most of a step whose kernels take tens of milliseconds."""
+    shim.run(so, BLOCKING)
 
 
 def test_a_pending_error_is_reported_once(so):
