@@ -58,11 +58,12 @@ int scratch_for_current_device(int32_t **out) {
 // floor(d / h) as the correctly rounded quotient gives it.  d * (1 / h) is
 // within 2^-50 of that quotient, relatively, so its floor is the same one unless
 // an integer lies that close; only then (and for zeros, infinities and NaN, where the
-// comparison fails) is the division made.  The FP64 pipe does 2 operations a
-// cycle and SM and a division costs about ten.
+// comparison fails, and next to zero, where a quotient is too small for a relative
+// bound) is the division made.  The FP64 pipe does 2 operations a cycle and SM
+// and a division costs about ten.
 __device__ __forceinline__ double cell_floor(double d, double h, double inv) {
   const double q = d * inv;
-  if (fabs(q - rint(q)) > 0x1p-50 * fabs(q)) return floor(q);
+  if (fabs(q - rint(q)) > fma(0x1p-50, fabs(q), 0x1p-1000)) return floor(q);
   return floor(__ddiv_rn(d, h));
 }
 
