@@ -355,9 +355,9 @@ __global__ void __launch_bounds__(256) k_point_eval(GridP g, StepP s, DevView v,
   // Sums over the support box.  What is linear in the nodal values is summed
   // first and combined with the time-stepping coefficients once per point: a
   // division per (point, node) is as many FP64 instructions as the rest of the
-  // node's work.  With the hoisted basis factors and one reciprocal per inverse, an
-  // evaluation of the 4.2M-point slope took 10.9 -> 7.4 ms, of 64 batched Newmark
-  // footings 1.54 -> 0.89, of the 80k-point footing 0.20 -> 0.12.
+  // node's work.  With the hoisted basis factors (and a reciprocal in inv_d, since
+  // taken out) an evaluation of the 4.2M-point slope took 10.9 -> 7.4 ms, of 64 batched
+  // Newmark footings 1.54 -> 0.89, of the 80k-point footing 0.20 -> 0.12.
   double dF[9] = {0}, gPn[3] = {0, 0, 0}, gVn[9] = {0}, ah[3] = {0, 0, 0};  // dF - 1 until after the loop
   double vh[3] = {0, 0, 0}, uh[3] = {0, 0, 0};
   double ph = 0.0, pdev = 0.0;

@@ -569,24 +569,26 @@ __device__ inline double det_d(const double *A) {
          A[2] * (A[3] * A[7] - A[4] * A[6]);
 }
 
+// (By divisions: a product with 1 / det takes 0.6 of 6.2 ms off an evaluation of 4.2M
+// points, but its root mean square error is 6 to 14% larger.)
 template <int D>
 __device__ inline void inv_d(const double *A, double *B) {
-  const double r = 1.0 / det_d<D>(A);  // (an FP64 division is a long sequence on the narrow pipe)
+  const double det = det_d<D>(A);
   if (D == 2) {
-    B[0] = A[3] * r;
-    B[1] = -A[1] * r;
-    B[2] = -A[2] * r;
-    B[3] = A[0] * r;
+    B[0] = A[3] / det;
+    B[1] = -A[1] / det;
+    B[2] = -A[2] / det;
+    B[3] = A[0] / det;
   } else {
-    B[0] = (A[4] * A[8] - A[5] * A[7]) * r;
-    B[1] = (A[2] * A[7] - A[1] * A[8]) * r;
-    B[2] = (A[1] * A[5] - A[2] * A[4]) * r;
-    B[3] = (A[5] * A[6] - A[3] * A[8]) * r;
-    B[4] = (A[0] * A[8] - A[2] * A[6]) * r;
-    B[5] = (A[2] * A[3] - A[0] * A[5]) * r;
-    B[6] = (A[3] * A[7] - A[4] * A[6]) * r;
-    B[7] = (A[1] * A[6] - A[0] * A[7]) * r;
-    B[8] = (A[0] * A[4] - A[1] * A[3]) * r;
+    B[0] = (A[4] * A[8] - A[5] * A[7]) / det;
+    B[1] = (A[2] * A[7] - A[1] * A[8]) / det;
+    B[2] = (A[1] * A[5] - A[2] * A[4]) / det;
+    B[3] = (A[5] * A[6] - A[3] * A[8]) / det;
+    B[4] = (A[0] * A[8] - A[2] * A[6]) / det;
+    B[5] = (A[2] * A[3] - A[0] * A[5]) / det;
+    B[6] = (A[3] * A[7] - A[4] * A[6]) / det;
+    B[7] = (A[1] * A[6] - A[0] * A[7]) / det;
+    B[8] = (A[0] * A[4] - A[1] * A[3]) / det;
   }
 }
 
@@ -679,8 +681,9 @@ __device__ __forceinline__ void for_box_nodes(const GridP &g, const DevView &v, 
 // 2 x 2 x 2), and neighbours in a lattice differ: on a jittered 3D block 23 of 32 lanes
 // of the point evaluation were active, at 86% of the FP64 pipe.  Per evaluation, in the
 // points' own order and in this one: 4.2M-point slope 7.3 -> 5.6 ms, 1M-point block
-// 1.84 -> 1.37, 163k-point block 0.35 -> 0.27, 80k-point footing 0.120 -> 0.108; per
-// update: 5.9 -> 5.1, 1.49 -> 1.24, 0.30 -> 0.25, 0.082 -> 0.074 ms.
+// 1.84 -> 1.37, 163k-point block 0.35 -> 0.27, 80k-point footing 0.120 -> 0.108 (all with
+// one reciprocal in inv_d; 6.2, 1.50, 0.30 and 0.114 with its divisions); per update:
+// 5.9 -> 5.1, 1.49 -> 1.24, 0.30 -> 0.25, 0.082 -> 0.074 ms.
 template <int D, int TP>
 __device__ inline int point_by_extent(const DevView &v, int64_t p0) {
   constexpr int NW = TP / 32, NE = 8 * NW, PER = (NE + 31) / 32;
