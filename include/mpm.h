@@ -447,7 +447,7 @@ int mpm_debug_jacobian32(mpm_ctx *ctx, const double *X, int32_t form, int32_t tp
  * ordered by (cell, index), without allocating: x_dev (n*dim doubles,
  * point-major), cell_dev (n int32) and order_dev (n int64) are DEVICE pointers
  * owned by the caller; stream is a cudaStream_t (NULL = default stream).  The
- * per-cell counters live in a fixed device array of this library (about 3 MiB
+ * per-cell counters live in a fixed device array of this library (about 2 MiB
  * on every GPU that loads it, held until exit), so the grid may have at most
  * 262,144 cells (also per axis, checked before the cell count is formed);
  * larger grids return MPM_ERR_TOO_LARGE.  A point outside the

@@ -532,7 +532,7 @@ void free_all(Ctx &c) {
                   c.sh_S0, c.m, c.rec, c.pn, c.M, c.Pn, c.vn, c.an, c.pdn, c.pddn, c.phi, c.act, c.fsd, c.sh_nrm, c.fixed, c.u_fixed,
                   c.p_fixed, c.u_value, c.p_value, c.trac, c.trac_raw, c.flux, c.err, c.row_nnz,
                   c.row_ptr, c.row_of, c.col, c.row_mask, c.X, c.R, c.dX, c.stage, c.H, c.gvec,
-                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.node_inst, c.bk, c.bk_i, c.bk_post, c.bn_nodes, c.bn_s0, c.bn_slices, c.bn_part, c.bn_npart};
+                  c.cs, c.sn, c.yv, c.hcol, c.part, c.scal, c.ctl, c.npart, c.mc, c.cm_buf, c.scan_tmp, c.terms, c.inst, c.inorm, c.bk, c.bk_i, c.bk_post, c.bn_nodes, c.bn_s0, c.bn_slices, c.bn_part, c.bn_npart};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (c.h_slot) cudaFreeHost(c.h_slot);  // with all other pinned words
@@ -793,7 +793,6 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
   A(&c.terms, 2);
   A(&c.inst, c.ninst);
   A(&c.inorm, c.ninst);
-  A(&c.node_inst, nn);
   if (c.ninst > 1) {
     // batched FGMRES state per instance: H ((m+1) m), g, cs, sn (m+1 each), h1,
     // h2 (PSTR each), target, residual; the column it is frozen at, columns
@@ -807,7 +806,7 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
     return create_abort(h, rc, "device or pinned host memory allocation failed");
   }
   cudaMemcpyAsync(c.inst, c.inst_h.data(), sizeof(InstDev) * c.ninst, cudaMemcpyHostToDevice, c.st);
-  {  // instance of every node (node boxes of the instances; -1 between them)
+  if (c.ninst > 1) {  // instance of every node (node boxes of the instances; -1 between them)
     std::vector<int32_t> ni(nn, -1);
     for (int i = 0; i < c.ninst; ++i) {
       const InstDev &I = c.inst_h[i];
@@ -817,9 +816,7 @@ int create_impl(const mpm_grid *grid, const mpm_particles *P, const mpm_material
         ni[(i0 + I.off[0]) + (int64_t)g.nn[0] * ((i1 + I.off[1]) + (int64_t)g.nn[1] * (i2 + I.off[2]))] = i;
       }
     }
-    cudaMemcpyAsync(c.node_inst, ni.data(), sizeof(int32_t) * nn, cudaMemcpyHostToDevice, c.st);
-    cudaStreamSynchronize(c.st);  // ni is a host temporary
-    if (c.ninst > 1 && (rc = batch_slices(c, ni))) {
+    if ((rc = batch_slices(c, ni))) {
       free_all(c);
       return create_abort(h, rc, "device memory allocation failed (node slices)");
     }

@@ -9,18 +9,16 @@
 //   gathered per block, with the Newmark linearization of Eq.
 //   newmark-linearization and delta ln J = div u for the quasi-static form.
 //
-// Design: gather, not scatter.  Points are cell-sorted, so the points that
-// can touch node a live in a small box of cells around it; the pattern, the
-// consistent mass and the Jacobian walk instead the first-node bins (the
-// points indexed by the first node of their support box, built per step),
-// whose box around a node (or a pair of nodes) is one narrower per axis,
-// fewer candidates for the kernels that read little per point or stage their
-// reads (the residual, which reads many record fields of each point, keeps the
-// cells' contiguous runs of points).  The residual is
-// computed by one thread per node row and each Jacobian block by one thread,
-// each summing its points in a fixed order: no floating-point atomics, results
-// are deterministic, and every (point, a, b) block term is computed exactly
-// once.  Per-point quantities that do not depend on (a, b) are computed once
+// Design: gather, not scatter.  Points are cell-sorted, and indexed by the
+// first node of their support box (the first-node bins, built per step).  All
+// terms of a bin fall on the nodes, and pairs of nodes, of one small box: the
+// residual and the Jacobian first sum each bin's points on its box, then add, for
+// each node and pair of nodes, the bins whose box holds it.  Supports of four
+// nodes, or no memory for the bins' sums, leave them to a thread per node row and
+// per pair of nodes, which walks the candidate points around it, as the pattern and
+// the consistent mass do.  Every sum runs in a fixed order: no floating-point
+// atomics, results are deterministic, and every (point, a, b) block term is
+// computed exactly once.  Per-point quantities that do not depend on (a, b) are computed once
 // per Newton iterate by k_point_eval and stored as structure-of-arrays
 // records.
 #include <math.h>

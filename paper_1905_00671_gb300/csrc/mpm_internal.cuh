@@ -298,7 +298,6 @@ struct Ctx {
   bool b_has_flux = false;
   double *inorm = nullptr;             // device: per-instance squared residual norms
   double *h_inorm = nullptr;           // pinned copy
-  int32_t *node_inst = nullptr;        // device: instance of every node (-1: between instances)
   // batched FGMRES: per-instance Krylov state (ninst x ...), see mpm_solver.cu
   double *bk = nullptr;                // one block of device doubles, carved below
   int32_t *bk_i = nullptr;             // per-instance flags / column counts

@@ -1637,7 +1637,7 @@ void sweep(Ctx &c, MGHier<real> &H, int l) {
   std::swap(H.x[l], H.x2[l]);
 }
 
-// V(k,k)-cycle on level l (k = c.mg_sweeps(), default 2).  On entry b[l]
+// V(k,k)-cycle on level l (k = c.mg_sweeps(), default 1).  On entry b[l]
 // holds the rhs and x[l] the first pre-smoothing sweep from zero (omega Dinv
 // b, pointwise), done by the kernel that produced b[l]; on return x[l] holds
 // the result.

@@ -9,7 +9,7 @@
 // the two output arrays; the per-cell counters live in the fixed array below.
 //
 // The scratch array is a file-scope __device__ variable: every GPU that loads
-// this library holds it (about 3 MiB) until the process exits, and every call
+// this library holds it (about 2 MiB) until the process exits, and every call
 // on that GPU shares it.  Host code cannot use the array's name as a device
 // address; the first call on each device looks the address up with
 // cudaGetSymbolAddress (with that device current) and keeps it.  Because that
