@@ -568,6 +568,7 @@ int create_fail(int rc, const char *why) {
 // a context that failed part-way: keep its message, free it
 int create_abort(mpm_ctx *h, int rc, const char *fallback) {
   g_create_error = h->c.last_error.empty() ? fallback : h->c.last_error;
+  cudaGetLastError();  // reported here: not again by the thread's next call
   delete h;
   return rc;
 }

@@ -36,6 +36,22 @@ print(rc)
 assert rc[1:] == [0, 0], rc
 """
 
+FAILED_CREATE = HEAD + """
+lib = mpm.load()
+sim = mpm.Simulation(w)
+sim.step()
+for spare in (0, 10 ** 6, 10 ** 8, 10 ** 9):
+    shim.shim_set_budget(spare)
+    try:
+        mpm.Simulation(w)
+        assert False, spare
+    except mpm.MPMError as e:
+        assert e.code == -9, e                  # MPM_ERR_NO_MEMORY
+    shim.shim_set_budget(-1)
+    rc = lib.mpm_step(sim.ctx, ctypes.c_double(w.dt), None, None)
+    assert rc == 0, (spare, rc)
+"""
+
 
 @pytest.fixture(scope="module")
 def so(tmp_path_factory):
@@ -54,3 +70,8 @@ def test_a_blocking_application_does_not_spin(so):
 def test_a_pending_error_is_reported_once(so):
     """An error that another call of the thread left behind fails one step at most."""
     shim.run(so, PENDING)
+
+
+def test_a_failed_creation_leaves_other_contexts_alone(so):
+    """A context that does not fit is refused, and the step of another goes on."""
+    shim.run(so, FAILED_CREATE)
