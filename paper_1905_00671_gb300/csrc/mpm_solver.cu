@@ -5,7 +5,8 @@
 // which brings the momentum rows (stiffness ~ 1e7) and the mass rows (~ 1e-7)
 // to unit diagonal so that the Krylov residual weighs both balance laws; then
 // right-preconditioned restarted FGMRES with classical Gram-Schmidt applied
-// twice (CGS2) solves it.  The Hessenberg matrix and the Givens rotations live
+// twice (in FP64 on single systems: where the first pass needs the second) solves
+// it.  The Hessenberg matrix and the Givens rotations live
 // in device memory (FP64); the host reads one scalar per iteration.  Vectors
 // and matrix values are in the precision T of the solve: FP64, or FP32 in the
 // mixed mode (the Newton residual around it stays FP64).  Reductions use a
