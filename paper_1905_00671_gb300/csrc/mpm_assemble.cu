@@ -1960,10 +1960,17 @@ __global__ void k_cm_init(int64_t nn, int K, const double *__restrict__ rhs, con
 }  // namespace
 
 // ============================================================== launchers
-// The bins' sums only make the residual and the Jacobian faster, so they give way
-// where a step needs their memory for what it cannot do without.
+// The bins' sums, and the FP32 staging where the direct form could serve, only make
+// the residual and the Jacobian faster, so they give way where a step needs their
+// memory for what it cannot do without.
 bool shed_scratch(Ctx &c) {
-  if (!c.rb && !c.jb) return false;
+  const bool pn32 = c.pn32 && !c.s.hencky;
+  if (!c.rb && !c.jb && !pn32) return false;
+  if (pn32) {
+    cudaFree(c.pn32);
+    c.pn32 = nullptr;
+    c.pn32_cap = 0;
+  }
   for (void **p : {(void **)&c.rb, (void **)&c.rb_cnt, &c.jb, (void **)&c.jb_cnt}) {
     cudaFree(*p);
     *p = nullptr;

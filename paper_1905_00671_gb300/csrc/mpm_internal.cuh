@@ -431,7 +431,7 @@ int run_pattern(Ctx &c);                          // builds row_ptr / col / row_
 int run_consistent_p2g(Ctx &c);  // Stage-1 fields by the consistent mass (after run_pattern)
 int ensure_jacobian_staging(Ctx &c);  // the FP64 Jacobian's ring of bins, or its staging buffer
 int ensure_jacobian_staging32(Ctx &c);  // the same in FP32 (mixed mode)
-// cudaMalloc for what a step cannot do without: the bins' buffers give way to it
+// cudaMalloc for what a step cannot do without: what only makes it faster gives way
 int step_malloc(Ctx &c, void **p, size_t bytes);
 bool shed_scratch(Ctx &c);  // frees them; false if there were none
 void run_initial_guess(Ctx &c);   // also sets the active flags

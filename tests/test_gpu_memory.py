@@ -55,3 +55,41 @@ def test_a_step_does_without_the_bins(name, tmp_path):
         pytest.skip("no CUDA device")
     precision, extra = CASES[name]
     shim.run(shim.build(tmp_path), PROGRAM.format(precision=precision, extra=repr(extra)))
+
+
+WIDE = """
+from dataclasses import replace
+import numpy as np
+from paper_1905_00671_gb300 import inputs as I, mpm
+
+w = I.small_block(seed=11, body=(11, 9, 7))
+w = replace(w, lp=np.ascontiguousarray(w.lp * 2.8))        # supports of four nodes
+
+def step():
+    base = shim.shim_used()
+    sim = mpm.Simulation(w, precision=mpm.MPM_MIXED, newton_rtol=1e-6, newton_max=60)
+    sim.step()
+    out = sim.read(("u", "p")), shim.shim_used() - base, sim.stats()
+    sim.close()
+    return out
+
+ref, used, st = step()
+assert st["jac_config"][1] >= 1000, st["jac_config"]       # staged
+staging = int(((st["jac_point_nodes"] + len(w.x)) * 1.25 + 1024) * 24 * 4)
+shim.shim_set_budget(used - staging // 2)
+got, _, st = step()
+assert shim.shim_refused() > 0
+assert st["jac_config"][1] < 1000, st["jac_config"]        # per term
+for f in ref:
+    assert np.abs(got[f] - ref[f]).max() <= 1e-5 * np.abs(ref[f]).max(), f
+"""
+
+
+def test_a_mixed_step_does_without_the_staging(tmp_path):
+    """Supports of four nodes in the mixed mode: the staged records give way to the
+    preconditioner's buffers, and the form that needs none serves (both forms to the
+    Newton tolerance of 1e-6)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    shim.run(shim.build(tmp_path), WIDE)
