@@ -1496,7 +1496,7 @@ struct MGHier<MG_REAL> {
   int *piv = nullptr;                    // row interchanges of the LU factorisation
   MG_REAL *ap[16] = {};                  // A P of a level and the next one, on its window (k_mg_ap)
   int win = 4, cwin = 4;                 // windows of the finest level and of the coarse levels
-  bool ap_wide = false;                  // ap[0] has room for a window of 5
+  int ap_slots = 0;                      // window slots ap[0] has room for
   int ncoarse = 0;                       // unknowns of the coarsest level
   int tail = 15;                         // first level of the dense tail (nlev - 1: the coarsest alone)
   MG_REAL *T = nullptr;                  // its operator
@@ -1770,8 +1770,9 @@ int mg_alloc(Ctx &c, MGHier<real> &H, int B) {
     const int64_t n = H.L[H.tail].nnodes * B;
     if (cudaMalloc(&H.T, sizeof(real) * n * n)) return MPM_ERR_NO_MEMORY;
   }
+  H.ap_slots = D == 2 ? 16 : 64;
   for (int k = 0; k + 1 < H.nlev; ++k)
-    if (cudaMalloc(&H.ap[k], sizeof(real) * H.L[k].nnodes * (D == 2 ? 16 : 64) * B * B)) return MPM_ERR_NO_MEMORY;
+    if (cudaMalloc(&H.ap[k], sizeof(real) * H.L[k].nnodes * H.ap_slots * B * B)) return MPM_ERR_NO_MEMORY;
   return MPM_OK;
 }
 
@@ -1889,12 +1890,15 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
   using namespace MG_NS;
   const int64_t nn = c.g.nnodes, nnzb = c.nnzb;
   const int d = c.d;
-  if (nnzb > S.sub_cap) {
-    // the captured graph reads these buffers (B1c, and Aval / Sval through
-    // the finest multigrid level): drop it, it is re-captured on next use
+  auto drop_graphs = [&] {  // they are captured again on next use
     if (S.gexec) cudaGraphExecDestroy(S.gexec);
     if (S.itexec) cudaGraphExecDestroy(S.itexec);
     S.gexec = S.itexec = nullptr;
+  };
+  if (nnzb > S.sub_cap) {
+    // the captured graph reads these buffers (B1c, and Aval / Sval through
+    // the finest multigrid level)
+    drop_graphs();
     MG_REAL *ptrs[] = {S.Aval, S.Sval, S.B1c, S.W, S.B2c};
     for (MG_REAL *p : ptrs) cudaFree(p);
     S.Aval = S.Sval = S.B1c = S.W = S.B2c = nullptr;
@@ -1909,26 +1913,35 @@ int schur_setup<MG_REAL>(Ctx &c, LinSys<MG_REAL> &S, bool coarse) {
     S.sub_cap = cap;
   }
   const bool full = coarse || !S.coarse_built;
+  // the finest level's A P on a window of so many slots; where the new buffer does not
+  // fit beside the narrower one, in its place (without either, the next set-up
+  // allocates anew)
+  auto reserve_ap = [&](MGHier<real> &H, int slots) -> int {
+    if (H.nlev == 1 || H.ap_slots >= slots) return MPM_OK;
+    const size_t bytes = sizeof(real) * H.L[0].nnodes * slots * H.B * H.B;
+    real *p = nullptr;
+    const bool beside = step_malloc(c, (void **)&p, bytes) == MPM_OK;
+    drop_graphs();
+    cudaFree(H.ap[0]);
+    H.ap[0] = p;
+    H.ap_slots = beside ? slots : 0;
+    if (beside) return MPM_OK;
+    if (const int rc = step_malloc(c, (void **)&H.ap[0], bytes)) return rc;
+    H.ap_slots = slots;
+    return MPM_OK;
+  };
   // the window of A P from the step's largest support
   int win = 3;
   for (int k = 0; k < d; ++k) win = std::max(win, std::min(c.h_cmax[k], 4) + 1);
   for (MGHier<real> *H : {S.mgA, S.mgS}) {
-    if (win == 5 && !H->ap_wide && H->nlev > 1) {
-      real *p = nullptr;  // (the narrower buffer stays if there is no room)
-      if (step_malloc(c, (void **)&p, sizeof(real) * H->L[0].nnodes * (d == 2 ? 25 : 125) * H->B * H->B)) {
-        c.last_error = "device allocation of the block preconditioner failed";
-        return MPM_ERR_NO_MEMORY;
-      }
-      cudaFree(H->ap[0]);
-      H->ap[0] = p;
-      H->ap_wide = true;
+    if (reserve_ap(*H, d == 2 ? (win == 5 ? 25 : 16) : (win == 5 ? 125 : 64))) {
+      c.last_error = "device allocation of the block preconditioner failed";
+      return MPM_ERR_NO_MEMORY;
     }
     // (coarse levels kept from an earlier set-up keep their window)
     const int cwin = !full ? H->cwin : win == 3 ? 3 : 4;
     if (H->win != win || H->cwin != cwin) {  // the captured graphs hold the other window's kernels
-      if (S.gexec) cudaGraphExecDestroy(S.gexec);
-      if (S.itexec) cudaGraphExecDestroy(S.itexec);
-      S.gexec = S.itexec = nullptr;
+      drop_graphs();
       H->win = win;
       H->cwin = cwin;
     }

@@ -76,20 +76,28 @@ def step():
 ref, used, st = step()
 assert st["jac_config"][1] >= 1000, st["jac_config"]       # staged
 staging = int(((st["jac_point_nodes"] + len(w.x)) * 1.25 + 1024) * 24 * 4)
-shim.shim_set_budget(used - staging // 2)
-got, _, st = step()
+shim.shim_set_budget(used - staging + int({extra}))
+sim = mpm.Simulation(w, precision=mpm.MPM_MIXED, newton_rtol=1e-6, newton_max=60)
+sim.step()
+got, st = sim.read(("u", "p")), sim.stats()
 assert shim.shim_refused() > 0
 assert st["jac_config"][1] < 1000, st["jac_config"]        # per term
 for f in ref:
     assert np.abs(got[f] - ref[f]).max() <= 1e-5 * np.abs(ref[f]).max(), f
+shim.shim_set_budget(-1)
+sim.step()
+assert sim.stats()["jac_config"][1] >= 1000                # staged again
+sim.close()
 """
 
 
-def test_a_mixed_step_does_without_the_staging(tmp_path):
+# room for half of the records, or for nothing beside what the step cannot do without
+@pytest.mark.parametrize("extra", ["staging / 2", "1024"])
+def test_a_mixed_step_does_without_the_staging(extra, tmp_path):
     """Supports of four nodes in the mixed mode: the staged records give way to the
-    preconditioner's buffers, and the form that needs none serves (both forms to the
-    Newton tolerance of 1e-6)."""
+    preconditioner's buffers, the wide A P takes the narrow one's place, and the form
+    that needs no records serves (both forms to the Newton tolerance of 1e-6)."""
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    shim.run(shim.build(tmp_path), WIDE)
+    shim.run(shim.build(tmp_path), WIDE.format(extra=extra))
