@@ -18,9 +18,9 @@
 // per pair of nodes, which walks the candidate points around it, as the pattern and
 // the consistent mass do.  Every sum runs in a fixed order: no floating-point
 // atomics, results are deterministic, and every (point, a, b) block term is
-// computed exactly once.  Per-point quantities that do not depend on (a, b) are computed once
-// per Newton iterate by k_point_eval and stored as structure-of-arrays
-// records.
+// computed exactly once.  Per-point quantities that do not depend on (a, b) are
+// computed once per Newton iterate by k_point_eval and stored as
+// structure-of-arrays records.
 #include <math.h>
 
 #include <algorithm>
@@ -2376,9 +2376,9 @@ void launch_jac_bins(Ctx &c, T *val, int apply_bc, const BasisArrays<T> &BA, con
 
 // One assembly with a given kernel configuration: staged (by first-node bins, or
 // for supports of 4 nodes, or without room for the ring, k_point_nodes then
-// k_jacobian on the per-(point, node) vectors) or direct (k_jacobian_direct), tpb threads per block of the kernel
-// that writes the blocks.  Values in precision T computed
-// in precision T from the FP64 records or their FP32 copies.
+// k_jacobian on the per-(point, node) vectors) or direct (k_jacobian_direct),
+// tpb threads per block of the kernel that writes the blocks.  Values in
+// precision T computed in precision T from the FP64 records or their FP32 copies.
 template <typename T>
 void launch_jacobian(Ctx &c, T *val, int apply_bc, int form, int tpb) {
   const DevView v = c.view();
